@@ -1,8 +1,8 @@
 """Build the in-tree CUDA library ``libccmsav.so`` for sm_103a with nvcc.
 
 The translation units (the C ABI, the FP32-bulk and the FP64 instantiations
-of the step, the allocation-free mass and the standalone spectral solver) are
-compiled in parallel and linked into one shared object
+of the step, the allocation-free mass, the standalone spectral solver and the
+FP64 line transforms, one unit for each line length) are compiled in parallel and linked into one shared object
 next to this file.  ``python -m paper_2601_10057_gb300.build`` runs it.
 """
 from __future__ import annotations
@@ -18,7 +18,10 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libccmsav.so")
 LIB_BOUNDS = os.path.join(HERE, "libccmsav_bounds.so")   # index-checked build (-DCCMSAV_BOUNDS), for tests
-SOURCES = ["ccmsav_api.cu", "sim_f32.cu", "sim_f64.cu", "ccmsav_noalloc.cu", "spectral_solve.cu"]
+# (source, extra flags, object)
+SOURCES = [(f, [], f.replace(".cu", ".o")) for f in ("ccmsav_api.cu", "sim_f32.cu", "sim_f64.cu", "ccmsav_noalloc.cu",
+                                                     "spectral_solve.cu", "fixed_ops.cu")]
+SOURCES += [("fixed_m.cu", [f"-DFIXED_M={m}"], f"fixed_m{m}.o") for m in (32, 64, 128, 256, 512, 1024, 2048, 4096)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
@@ -47,9 +50,10 @@ def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> s
     os.makedirs(bdir, exist_ok=True)
     cc = nvcc()
 
-    def compile_one(src):
-        obj = os.path.join(bdir, src.replace(".cu", ".o"))
-        cmd = [cc, *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit):
+        src, flags, name = unit
+        obj = os.path.join(bdir, name)
+        cmd = [cc, *ARCH, *FLAGS, *extra, *flags, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")

@@ -1,0 +1,52 @@
+// fixed_ops.h -- host interface of the FP64 fixed-point line transforms
+// (fixed_kernels.cuh).  The kernels of each line length M = N/2 are compiled
+// in a translation unit of their own (fixed_m.cu with -DFIXED_M=M, so that
+// they build in parallel); fixed_ops(M) returns its launch functions.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace ccm {
+struct SpecCoef;
+struct DevScalars;
+namespace xf {
+
+// Twiddle and pair tables of one line length (device, one allocation: tw2 [M],
+// then the pair tables wn, forward a, b, inverse a, b [M/2 + 1 each]; each
+// entry a complex factor with 62 fractional bits as two (high, signed low)
+// word pairs).
+struct Tables {
+    int4* mem = nullptr;
+    int M = 0, pf = 0, pi = 0;          // powers of two of the forward and inverse DCT factors
+};
+
+struct Ops {
+    int M;
+    // opt in to the kernels' shared memory; *gram_rows: partial rows that col_gram leaves
+    int (*setup)(int* gram_rows);
+    // host values of the tables' M + 5 (M/2 + 1) entries and the powers of two
+    void (*fill)(int4* host, int* pf, int* pi);
+    void (*weights)(const double* ev, const SpecCoef& sc, double* isig, double* itau, cudaStream_t st);
+    // the four transform kernels of a step (fields in a, b as in SimImpl's bufA, bufB)
+    void (*row_step)(const double* a, double* b, const Tables& t, cudaStream_t st);
+    void (*col_gram)(const double* b, double* spec, double* part, const Tables& t, const double* isig, const double* itau,
+                     int rows, cudaStream_t st);
+    void (*comb)(const double* spec, double* b, const Tables& t, const double* isig, const double* itau,
+                 const DevScalars* sc, cudaStream_t st);
+    void (*irow)(const double* b, double* phi_new, double* psi_new, const Tables& t, const double* phn, const double* pho,
+                 const double* psn, const double* pso, int bdf1, cudaStream_t st);
+    // u = (c0 - c1 Lap_h + c2 Lap_h^2)^{-1} f for nf fields of N x N (Neumann; dst: Dirichlet); scr: nf fields.
+    // u may be f.  dcoef: c0, c1, c2 on the device (may be null); dskip: fields to leave alone (may be null).
+    void (*solve)(const double* f, double* u, double* scr, const Tables& t, const double* ev, const double c[3],
+                  const double* dcoef, const int* dskip, int nf, bool dst, cudaStream_t st);
+    int (*oob)(unsigned* flag);         // index-check flag of the translation unit: read and cleared (CCMSAV_BOUNDS)
+};
+
+// Launch functions of line length M, or null (M = 32 .. 4096 are built).
+const Ops* fixed_ops(int M);
+// Device tables of line length M on stream st (the host copy is complete on
+// return); 0 or a CCMSAV_E* code.
+int make_tables(const Ops* o, Tables& t, cudaStream_t st);
+inline void free_tables(Tables& t) { cudaFree(t.mem); t = Tables{}; }
+
+}  // namespace xf
+}  // namespace ccm

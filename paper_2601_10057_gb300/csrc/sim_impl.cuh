@@ -24,6 +24,7 @@
 #include "warp_kernels.cuh"
 #include "spectral_kernels.cuh"
 #include "classical_kernels.cuh"
+#include "fixed_ops.h"
 #include <type_traits>
 #include <map>
 #include <mutex>
@@ -75,6 +76,13 @@ public:
     float4* twI = nullptr;       // (wn, a) per pair; b of pair 0 in twF0 / twI0
     float2 twF0{}, twI0{};
     wf::PairTwTab pair_tab(const float4* t) const { return wf::PairTwTab{t, t == twF ? twF0 : twI0}; }
+    // FP64 path (N >= 64): the fixed-point line transforms and 1/sigma, 1/tau of
+    // the handle's time step in the order of their spectra
+    const xf::Ops* xo = nullptr;
+    xf::Tables xt;
+    double* isig = nullptr;
+    double* itau = nullptr;
+    int xrows = 0;               // partial rows of the Gram sums
     int wRT = 8, wlds = 0, wRT4 = 4, wlds4 = 0, wKC = 1, wRI = 4;
     int ahead_rt = 0;   // L2 prefetch distance of the row kernel (0: none)
     size_t wsm_rt = 0, wsm_col = 0, wsm_comb = 0, wsm_irow = 0;
@@ -143,7 +151,7 @@ public:
         return r;
     }
 
-    long long launches_per_step() const { return 6 + ((flags & CCMSAV_TRACK_ENERGY) ? 2 : 0); }
+    long long launches_per_step() const { return 6 + (xo && M >= 2048 ? 1 : 0) + ((flags & CCMSAV_TRACK_ENERGY) ? 2 : 0); }
 
     void count_steps(int n3) override { steps_taken += n3; nlaunch += n3 * launches_per_step(); }
     void count_steps_grouped(int n3) override { steps_taken += n3; }
@@ -309,6 +317,8 @@ public:
         if (tw2i && tw2i != tw2) cudaFree(tw2i);
         cudaFree(tw2); cudaFree(evf); cudaFree(evp); cudaFree(twF); cudaFree(twI);
         cudaFree(cl); cudaFree(pcg); cudaFree(cl_red);
+        cudaFree(isig); cudaFree(itau); xf::free_tables(xt);
+        isig = itau = nullptr;
         if (pcg_host) cudaFreeHost(pcg_host);
         cl = nullptr; pcg = nullptr; cl_red = nullptr; pcg_host = nullptr;
         tw2 = nullptr; tw2i = nullptr; evf = nullptr; evp = nullptr; twF = nullptr; twI = nullptr;
@@ -437,7 +447,24 @@ public:
             int r = init_warp_path();
             if (r) return r;
         }
+        if constexpr (std::is_same<T, double>::value)
+            if (!(force_block && force_block[0] == '1') && (xo = xf::fixed_ops(M)))
+                if (const int r = init_fixed()) return r;
         CCM_CUDA(cudaStreamSynchronize(st));
+        return CCMSAV_OK;
+    }
+
+    int init_fixed() {
+        if (const int r = xo->setup(&xrows)) return r;
+        if (const int r = xf::make_tables(xo, xt, st)) return r;
+        if (cudaMalloc(&isig, NN * sizeof(double)) != cudaSuccess || cudaMalloc(&itau, NN * sizeof(double)) != cudaSuccess)
+            return CCMSAV_ENOMEM;
+        StencilCoef<T> c;
+        SpecCoef s;
+        SolveCoef so;
+        step_coefs((flags & CCMSAV_BDF1_ALWAYS) != 0, c, s, so);
+        xo->weights(ev, s, isig, itau, st);
+        CCM_CUDA(cudaGetLastError());
         return CCMSAV_OK;
     }
 
@@ -461,15 +488,21 @@ public:
     // z = M^{-1} r for both systems (DCT solve of a - lam Mbar Lap_h with the
     // coefficients on the device); converged systems are skipped.
     void cl_precond(const T* r, T* z, T* scr) {
-        const dim3 g1(N / cl_geo.RT, 2), g2(N / cl_geo.RC, 2), b(cl_geo.threads);
         // device addresses of the convergence flags and the coefficients
         const int* conv = reinterpret_cast<const int*>(reinterpret_cast<const char*>(pcg) + offsetof(PcgScalars, conv));
         const double* coef = reinterpret_cast<const double*>(reinterpret_cast<const char*>(pcg) + offsetof(PcgScalars, coef));
+        nlaunch += 3;
+        if constexpr (std::is_same<T, double>::value)
+            if (xo) {
+                const double c[3] = {0.0, 0.0, 0.0};
+                xo->solve(r, z, scr, xt, ev, c, coef, conv, 2, false, st);
+                return;
+            }
+        const dim3 g1(N / cl_geo.RT, 2), g2(N / cl_geo.RC, 2), b(cl_geo.threads);
         ss::k_ss_row_fwd<T, false><<<g1, b, cl_geo.sm_fwd, st>>>(r, scr, N, cl_geo.RT, cl_geo.lds, twM, twP, conv, NN);
         ss::k_ss_col_solve<T><<<g2, b, cl_geo.sm_col, st>>>(scr, N, cl_geo.RC, twM, twP, ev, 0.0, 0.0, 0.0,
                                                            coef, conv, NN);
         ss::k_ss_row_inv<T, false><<<g1, b, cl_geo.sm_inv, st>>>(scr, z, N, cl_geo.RT, cl_geo.lds, twM, twP, conv, NN);
-        nlaunch += 3;
     }
 
     // The classical scheme's two Cahn-Hilliard solves y1 = zeta_c^{-1} g0c and
@@ -703,7 +736,9 @@ public:
         CCM_CUDA(cudaStreamSynchronize(st));
         CCM_CUDA(cudaMemcpyFromSymbol(&v, g_oob_flag, sizeof(v)));
         CCM_CUDA(cudaMemcpyToSymbol(g_oob_flag, &z, sizeof(z)));
-        return (int)v;
+        unsigned x = 0;
+        if (xo && xo->oob(&x)) return CCMSAV_ECUDA;
+        return (int)(v | x);
 #else
         return CCMSAV_EINVAL;
 #endif
@@ -1097,9 +1132,27 @@ public:
             if (r) return r;
             mark(7);
         }
+        // the handle's 1/sigma and 1/tau, or (BDF1 start step) those of the
+        // start step in the staging buffer, which no queued work holds
+        const double *ws = isig, *wt = itau;
         if (warp_path) {
             warp_forward(s, anchor);
             so.nb2 = N / wKC;
+        } else if (xo) {
+            if (bdf1 && !(flags & CCMSAV_BDF1_ALWAYS)) {
+                double* w = static_cast<double*>(tmp64);
+                xo->weights(ev, s, w, w + NN, st);
+                ws = w; wt = w + NN;
+                ++nlaunch;
+            }
+            const double* a = reinterpret_cast<const double*>(bufA);
+            double* b = reinterpret_cast<double*>(bufB);
+            xo->row_step(a, b, xt, st);
+            mark(1);
+            xo->col_gram(b, reinterpret_cast<double*>(bufA), part2, xt, ws, wt, xrows, st);
+            mark(2);
+            so.nb2 = xrows;
+            if (M >= 2048) ++nlaunch;
         } else {
             k_rowdct_T<T><<<dim3(N / RT, NF), 512, sm_rt, st>>>(bufA, bufB, N, RT, lds_rt, twM, twP);
             mark(1);
@@ -1120,6 +1173,14 @@ public:
         if (warp_path) {
             bdf1_launch = so.bdf1;
             warp_inverse(s, anchor);
+        } else if (xo) {
+            double* b = reinterpret_cast<double*>(bufB);
+            xo->comb(reinterpret_cast<const double*>(bufA), b, xt, ws, wt, sc, st);
+            mark(4);
+            xo->irow(b, reinterpret_cast<double*>(phi[spare]), reinterpret_cast<double*>(psi[spare]), xt,
+                     reinterpret_cast<const double*>(phi[cur]), reinterpret_cast<const double*>(phi[prev]),
+                     reinterpret_cast<const double*>(psi[cur]), reinterpret_cast<const double*>(psi[prev]), so.bdf1, st);
+            mark(5);
         } else {
             k_comb_icolT<T><<<N / RT4, 512, sm_comb, st>>>(bufA, bufB, N, RT4, lds_c, twM, twP, ev, s, sc, anchor);
             mark(4);

@@ -8,6 +8,7 @@
 #include <vector>
 #include "../../include/ccmsav.h"
 #include "spectral_kernels.cuh"
+#include "fixed_ops.h"
 
 struct ccmsav_solver {
     int N = 0, bc = 0, precision = 0;
@@ -22,6 +23,8 @@ struct ccmsav_solver {
     double smin = 0.0;             // smallest 2D eigenvalue of -Lap_h
     int threads = 256, RT = 1, RC = 1, lds = 0;
     size_t sm_fwd = 0, sm_col = 0, sm_inv = 0;
+    const ccm::xf::Ops* xo = nullptr;   // FP64 Neumann / Dirichlet from N = 64 on: fixed-point line transforms
+    ccm::xf::Tables xt;
     long long launches = 0;
 };
 
@@ -73,11 +76,24 @@ template <typename T> int setup(ccmsav_solver* s) {
         if (cudaMemcpyAsync(s->twP, hp.data(), (M / 2 + 1) * sizeof(PostTw<T>), cudaMemcpyHostToDevice, s->st) != cudaSuccess)
             return CCMSAV_ECUDA;
     }
+    if constexpr (sizeof(T) == sizeof(double))
+        if (!per && (s->xo = ccm::xf::fixed_ops(M))) {
+            int rows = 0;
+            if (const int r = s->xo->setup(&rows)) return r;
+            if (const int r = ccm::xf::make_tables(s->xo, s->xt, s->st)) return r;
+        }
     return cudaStreamSynchronize(s->st) == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
 }
 
 template <typename T> int solve(ccmsav_solver* s, const double c[3], const T* f, T* u) {
     const int N = s->N;
+    if constexpr (sizeof(T) == sizeof(double))
+        if (s->xo) {
+            s->xo->solve(f, u, static_cast<double*>(s->scratch), s->xt, s->ev, c, nullptr, nullptr, 1,
+                         s->bc == CCMSAV_BC_DIRICHLET, s->st);
+            s->launches += 3;
+            return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
+        }
     const dim3 b(s->threads);
     const cplx<T>* tw = static_cast<const cplx<T>*>(s->tw);
     if (s->bc == CCMSAV_BC_PERIODIC) {
@@ -124,6 +140,7 @@ void release(ccmsav_solver* s) {
     if (!s) return;
     if (s->st) cudaStreamSynchronize(s->st);
     cudaFree(s->scratch); cudaFree(s->rhs); cudaFree(s->tw); cudaFree(s->twP); cudaFree(s->ev);
+    ccm::xf::free_tables(s->xt);
     if (s->own_stream && s->st) cudaStreamDestroy(s->st);
     delete s;
 }

@@ -386,7 +386,7 @@ __device__ __forceinline__ float bar_add_fb(float a, float b, float du, float an
     return out;
 }
 __device__ __forceinline__ double bar_add(double a, double b, double du, double anc, bool bdf1, uint32_t = 0) {
-    return (bdf1 ? a : a + (a - b) / 3.0) + du + anc;
+    return (bdf1 ? a : fma(a - b, 1.0 / 3.0, a)) + du + anc;
 }
 
 // ------------------------------------------------------------------ k_stencil
