@@ -2,7 +2,7 @@
 
 The translation units (the C ABI, the FP32-bulk and the FP64 instantiations
 of the step, the allocation-free mass, the standalone spectral solver and the
-FP64 line transforms, one unit for each line length) are compiled in parallel and linked into one shared object
+FP64 stencil and line transforms, these one unit for each line length) are compiled in parallel and linked into one shared object
 next to this file.  ``python -m paper_2601_10057_gb300.build`` runs it.
 """
 from __future__ import annotations
@@ -20,7 +20,7 @@ LIB = os.path.join(HERE, "libccmsav.so")
 LIB_BOUNDS = os.path.join(HERE, "libccmsav_bounds.so")   # index-checked build (-DCCMSAV_BOUNDS), for tests
 # (source, extra flags, object)
 SOURCES = [(f, [], f.replace(".cu", ".o")) for f in ("ccmsav_api.cu", "sim_f32.cu", "sim_f64.cu", "ccmsav_noalloc.cu",
-                                                     "spectral_solve.cu", "fixed_ops.cu")]
+                                                     "spectral_solve.cu", "fixed_ops.cu", "fixed_stencil.cu")]
 SOURCES += [("fixed_m.cu", [f"-DFIXED_M={m}"], f"fixed_m{m}.o") for m in (32, 64, 128, 256, 512, 1024, 2048, 4096)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]

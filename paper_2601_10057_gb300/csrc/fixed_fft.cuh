@@ -29,13 +29,19 @@
 // values and scales beyond the FP64 range on the way back are exact up to
 // FP64's own rounding (to_double).
 //
-// The line layout is that of warp_fft.cuh: M = E G complex values on G lanes,
-// an E-point DFT in registers, twiddle, transpose through the line's
-// shared-memory buffer, G-point DFTs; for G = R E the split second pass.
+// Line layout: M = A C D complex values on G = M / A lanes, A = 16 per lane
+// (8 for the shortest lines): an A-point DFT in registers, twiddle, then on
+// each row of B = C D values a C-point and a D-point DFT, exchanged through the
+// line's shared-memory buffer (D = 1: one exchange).  Sixteen values are 64
+// registers of data, so sixteen warps fit an SM; with 32 (two exchanges fewer)
+// eight fit and the kernels waited on instruction latency and, in the ones
+// with the longest unrolled code, on instruction fetch (ncu, N = 2048: issue
+// slots 39 % busy in the row kernel, 15 - 21 % in the others).
 #pragma once
 #include "dct_device.cuh"
 #include "warp_fft.cuh"
 #include "bounds.cuh"
+#include "fixed_ops.h"
 
 namespace ccm {
 namespace xf {
@@ -47,12 +53,6 @@ __device__ __forceinline__ fx operator-(fx a) { return fx{-a.v}; }
 using cx = cplx<fx>;
 
 // ------------------------------------------------------------------ products
-// A factor w (|w| <= 2^62, 62 fractional bits) as w = h 2^32 + l with l a
-// signed word; h and -h, -l fit 32 bits.
-struct Fac { int h, l; };
-__host__ __device__ constexpr Fac fac(long long w) {
-    return Fac{(int)((w + 0x80000000LL) >> 32), (int)(w & 0xffffffffLL)};
-}
 struct CFac { Fac x, y; };              // re, im
 
 // cos(2 pi j / 64) with 62 fractional bits
@@ -149,31 +149,31 @@ struct DIFX {
 template <bool INV, int OFF> struct DIFX<1, INV, OFF> { static __device__ __forceinline__ void run(cx*) {} };
 
 // ------------------------------------------------------------------ line shapes
-// M = E G.  32 values per lane at most (128 registers of data); from M = 2048
-// on a line spans two and four warps (split second pass).
 template <int M> struct Shape;
-template <> struct Shape<32>   { static constexpr int E = 8,  G = 4;   };
-template <> struct Shape<64>   { static constexpr int E = 8,  G = 8;   };
-template <> struct Shape<128>  { static constexpr int E = 16, G = 8;   };
-template <> struct Shape<256>  { static constexpr int E = 16, G = 16;  };
-template <> struct Shape<512>  { static constexpr int E = 32, G = 16;  };
-template <> struct Shape<1024> { static constexpr int E = 32, G = 32;  };
-template <> struct Shape<2048> { static constexpr int E = 32, G = 64;  };
-template <> struct Shape<4096> { static constexpr int E = 32, G = 128; };
+template <> struct Shape<32>   { static constexpr int A = 8,  C = 4,  D = 1;  };
+template <> struct Shape<64>   { static constexpr int A = 8,  C = 8,  D = 1;  };
+template <> struct Shape<128>  { static constexpr int A = 16, C = 8,  D = 1;  };
+template <> struct Shape<256>  { static constexpr int A = 16, C = 16, D = 1;  };
+template <> struct Shape<512>  { static constexpr int A = 16, C = 4,  D = 8;  };
+template <> struct Shape<1024> { static constexpr int A = 16, C = 8,  D = 8;  };
+template <> struct Shape<2048> { static constexpr int A = 16, C = 16, D = 8;  };
+template <> struct Shape<4096> { static constexpr int A = 16, C = 16, D = 16; };
 
 // LINES lines per CTA: eight (one 64-byte segment of eight rows in the
-// transposed writes), fewer where their buffers no longer fit.  A buffer is
-// the padded transpose plus what makes its length odd in units of 16 bytes
-// modulo 128, so that the same element of eight lines lies in distinct banks.
+// transposed writes), fewer where their buffers no longer fit.  Rows of the
+// exchanges are P = B + 1 values apart (odd, so that eight rows' values of one
+// column lie in distinct banks), and so, modulo eight, are the buffers.
 template <int M> struct Geo {
-    static constexpr int E = Shape<M>::E, G = Shape<M>::G, J = E >= G ? E / G : 1, R = G > E ? G / E : 1;
-    static constexpr int N = 2 * M, HI = E / 2;            // HI pairs per lane
+    static constexpr int A = Shape<M>::A, C = Shape<M>::C, D = Shape<M>::D, B = C * D, E = A, G = M / A;
+    static_assert(A * B == M && A % C == 0 && A % D == 0, "line shape");
+    static constexpr int N = 2 * M;
     static constexpr int LINES = M <= 1024 ? 8 : M == 2048 ? 4 : 2;
     static constexpr int THREADS = LINES * G;
     static constexpr int W = G > 32 ? G / 32 : 1;          // warps per line
-    static constexpr int P = E >= G ? G + 1 : G + R;       // transpose row
-    static constexpr int BUF = ((E * P + 7) / 8) * 8 + 1;
+    static constexpr int P = B + 1;
+    static constexpr int BUF = ((A * P + 7) / 8) * 8 + 1;
     static constexpr size_t SMEM = (size_t)LINES * BUF * sizeof(cx);
+    static constexpr int MINB = THREADS <= 128 ? 3 : THREADS <= 256 ? 2 : 1;   // at most 128 registers from 256 threads on
     static_assert(THREADS % 32 == 0, "whole warps");
 };
 
@@ -233,29 +233,32 @@ __device__ __forceinline__ fx to_fixed(double x, int em) {
     int e = (int)((hi >> 20) & 0x7ffu);
     const unsigned m = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
     e = max(e, 1);
-    const unsigned long long t = ((unsigned long long)m << 42) | ((unsigned long long)lo << 10);   // below 2^63
-    const long long q = (long long)(((t >> min(2 + em - e, 63)) + 1) >> 1);
+    // mantissa at bit 62 as two words, right by 2 + em - e, rounded by the last shift
+    unsigned H = __funnelshift_l(lo, m, 10), Lw = lo << 10;
+    const int r = min(2 + em - e, 63);
+    if (r >= 32) { Lw = H; H = 0; }
+    Lw = __funnelshift_r(Lw, H, r);                    // shift counts modulo 32
+    H >>= r & 31;
+    const long long q = (long long)(((((unsigned long long)H << 32) | Lw) + 1) >> 1);
     const long long s = (int)hi >> 31;
     return fx{(q ^ s) - s};
 }
 
+// Beyond FP64's normal range (kept out of line: its conversions would be
+// executed ahead of the branch, on the FP64 pipe).
+static __device__ __noinline__ double to_double_far(long long v, int ex) { return scalbn((double)v, max(-4000, min(4000, ex))); }
+
 // v 2^ex rounded to nearest (ties away from zero)
 __device__ __forceinline__ double to_double(fx v, int ex) {
-    const long long s = v.v >> 63;
-    unsigned long long q = (unsigned long long)((v.v ^ s) - s);
-    const int lz = __clzll((long long)q);
-    int e = ex - lz + 63 + 1022;                       // biased exponent - 1
-    double r = 0.0;
-    if (q) {
-        q <<= lz;
-        if (e >= 0 && e < 2045) {
-            const unsigned long long b = ((unsigned long long)(unsigned)e << 52) + (q >> 11) + ((q >> 10) & 1);
-            r = __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
-        } else {                                       // beyond FP64's normal range
-            r = scalbn((double)(v.v), max(-4000, min(4000, ex)));
-        }
-    }
-    return r;
+    const long long s8 = v.v >> 63, u = (v.v ^ s8) - s8;
+    const unsigned h = (unsigned)(u >> 32), l = (unsigned)u;
+    const unsigned n = h ? h : l, m = h ? l : 0;
+    const int lz = __clz((int)n), e = (h ? ex : ex - 32) - lz + 63 + 1022;   // biased exponent - 1
+    if (n != 0 && (unsigned)e >= 2045u) return to_double_far(v.v, ex);
+    const unsigned H = __funnelshift_l(m, n, lz), Lw = m << (lz & 31);
+    const unsigned long long b = (((unsigned long long)((unsigned)e << 20) + (H >> 11)) << 32 | __funnelshift_r(Lw, H, 11)) + ((Lw >> 10) & 1);
+    const unsigned long long z = n ? b | ((unsigned long long)s8 & 0x8000000000000000ull) : 0;
+    return __longlong_as_double((long long)z);
 }
 // v 2^(ex + p) of a line with exponent ex
 __device__ __forceinline__ double line_double(fx v, int ex, int p = 0) {
@@ -298,57 +301,61 @@ __device__ __forceinline__ cx shift_cx(cx a, int sh, long long h) { return mk(fx
 
 // The unnormalised DFT of the line (value G n1 + n2 in v[n1] of lane n2);
 // the result lies in buf in natural order, visible to the line's lanes.
-// tw2[k1 G + n2] = W_M^{n2 k1}.
+// tw: W_M^{n2 k1} at k1 G + n2, then (D > 1) W_B^{d kc} at kc D + d.
+//   1. A-point DFT over n1, times W_M^{n2 k1}, to row k1 of the buffer;
+//   2. C-point DFTs over c of the row's values D c + d, times W_B^{d kc}, back
+//      to the slots they came from (D = 1: to natural order, k1 + A kc);
+//   3. D-point DFTs over d of D kc + d, to natural order k1 + A (kc + C kd).
+// Lanes run along d in step 2 and along k1 in the last step: both reads and
+// the natural-order write are free of bank conflicts.
 template <int M, bool INV>
-__device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict__ tw2, int n2, int slot, int sh) {
+__device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict__ tw, int n2, int slot, int sh) {
     using Gm = Geo<M>;
-    constexpr int E = Gm::E, G = Gm::G, P = Gm::P;
-    DIFX<E, INV, 0>::run(v);
+    constexpr int A = Gm::A, C = Gm::C, D = Gm::D, G = Gm::G, P = Gm::P;
+    DIFX<A, INV, 0>::run(v);
     const long long h = (1LL << sh) >> 1;
 #pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int k1 = wf::bitrev<E>(r);
+    for (int r = 0; r < A; ++r) {
+        const int k1 = wf::bitrev<A>(r);
         cx u = v[r];
-        if (k1) u = cmulf<INV>(u, ld_fac(tw2 + k1 * G + n2));
+        if (k1) u = cmulf<INV>(u, ld_fac(tw + k1 * G + n2));
         buf[k1 * P + n2] = shift_cx(u, sh, h);
     }
     sync_line<M>(slot);
-    if constexpr (E >= G) {
-        constexpr int J = Gm::J;
+    if constexpr (D > 1) {
+        const int4* __restrict__ t3 = tw + M;
 #pragma unroll
-        for (int j = 0; j < J; ++j)
+        for (int j = 0; j < A / C; ++j) {
+            const int q = n2 + G * j, d = q % D;
+            cx* row = buf + (q / D) * P + d;
+            cx u[C];
 #pragma unroll
-            for (int m = 0; m < G; ++m) v[j * G + m] = buf[(n2 * J + j) * P + m];
-        sync_line<M>(slot);
-        DIFX<G, INV, 0>::run(v);
-        if constexpr (J == 2) DIFX<G, INV, (J == 2 ? G : 0)>::run(v);
+            for (int c = 0; c < C; ++c) u[c] = row[D * c];
+            DIFX<C, INV, 0>::run(u);
 #pragma unroll
-        for (int j = 0; j < J; ++j)
-#pragma unroll
-            for (int r = 0; r < G; ++r) buf[(n2 * J + j) + E * wf::bitrev<G>(r)] = v[j * G + r];
-    } else {
-        // each G-point row on R adjacent lanes (fourstep_split in warp_fft.cuh has the formula)
-        constexpr int R = Gm::R;
-        constexpr unsigned FULL = 0xffffffffu;
-        const int k1 = n2 / R, q = n2 % R;
-#pragma unroll
-        for (int t = 0; t < E; ++t) v[t] = buf[k1 * P + R * t + q];
-        sync_line<M>(slot);
-        DIFX<E, INV, 0>::run(v);
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int k = wf::bitrev<E>(r);
-            cx u = cmulf<INV>(v[r], ld_fac(tw2 + k * G + E * q));       // W_G^{q k}
-            cx p = mk(fx{__shfl_xor_sync(FULL, u.x.v, R / 2)}, fx{__shfl_xor_sync(FULL, u.y.v, R / 2)});
-            if constexpr (R == 2) {
-                buf[k1 + E * (k + E * q)] = q ? p - u : u + p;
-            } else {
-                u = (q & 2) ? p - u : u + p;
-                p = mk(fx{__shfl_xor_sync(FULL, u.x.v, 1)}, fx{__shfl_xor_sync(FULL, u.y.v, 1)});
-                const cx a = (q & 1) ? p : u, b = (q & 1) ? u : p;
-                const cx wb = (q & 2) ? (INV ? mk(-b.y, b.x) : mk(b.y, -b.x)) : b;
-                buf[k1 + E * (k + E * (((q & 1) << 1) | (q >> 1)))] = (q & 1) ? a - wb : a + wb;
+            for (int r = 0; r < C; ++r) {
+                const int kc = wf::bitrev<C>(r);
+                row[D * kc] = kc ? cmulf<INV>(u[r], ld_fac(t3 + kc * D + d)) : u[r];
             }
+        }
+        sync_line<M>(slot);
+    }
+    constexpr int Z = D > 1 ? D : C;              // the last DFT
+#pragma unroll
+    for (int j = 0; j < A / Z; ++j) {
+        const int q = n2 + G * j, k1 = q % A, kc = q / A;     // D = 1: kc = 0
+#pragma unroll
+        for (int d = 0; d < Z; ++d) v[j * Z + d] = buf[k1 * P + Z * kc + d];
+    }
+    sync_line<M>(slot);
+#pragma unroll
+    for (int j = 0; j < A / Z; ++j) {
+        const int q = n2 + G * j, k1 = q % A, kc = q / A;
+        DIFX<Z, INV, 0>::run(v + j * Z);
+#pragma unroll
+        for (int r = 0; r < Z; ++r) {
+            const int kd = wf::bitrev<Z>(r);
+            buf[k1 + A * (D > 1 ? kc + C * kd : kd)] = v[j * Z + r];
         }
     }
     sync_line<M>(slot);
@@ -385,38 +392,39 @@ __device__ __forceinline__ void pre_pair(const Quad64& X, const PairTab& t, int 
     zMk = mk(s.x + u.y, u.x - s.y);
 }
 
-// Pair items of a line: item k in [1, M/2) holds the modes k, N-k, M-k, M+k;
-// item 0 holds the modes 0, M/2, M, N-M/2 (the pairs 0 and M/2), so that the
-// M/2 items hold each of the N modes once.
-template <int M> __device__ __forceinline__ int item_mode(int k, int u) {
-    constexpr int N = 2 * M;
-    const int hi = k == 0 ? (u == 1 ? M / 2 : u == 3 ? N - M / 2 : u == 0 ? 0 : M) : 0;
-    return k == 0 ? hi : u == 0 ? k : u == 1 ? N - k : u == 2 ? M - k : M + k;
+// Slots: a line's N modes as M complex values, slot i = (X[i], X[N-i]) for
+// i >= 1 and slot 0 = (X[0], X[M]).  The pair k fills the slots k and M-k;
+// item k = 0 .. M/2 - 1 is the pair k and, for k = 0, the pairs 0 and M/2
+// (slots 0 and M/2).
+template <int M> __device__ __forceinline__ int slot_mode(int i, int c) {
+    return c == 0 ? i : i == 0 ? M : 2 * M - i;
 }
-// The four modes of item k from the natural-order spectrum z (a second turn
-// of the loop for item 0: one copy of the code).
-template <int M> __device__ __forceinline__ Quad64 post_item(const cx* z, const PairTab& t, int k) {
-    const cx A = z[k], B = z[k == 0 ? M / 2 : M - k];
-    Quad64 q = post_pair(A, k == 0 ? A : B, t, k);
+template <int M> __device__ __forceinline__ int item_slot2(int k) { return k == 0 ? M / 2 : M - k; }
+
+// The two slots of item k from the natural-order spectrum z (a second turn
+// for item 0).
+template <int M> __device__ __forceinline__ void post_item(const cx* z, const PairTab& t, int k, cx& s1, cx& s2) {
+    const cx A = z[k], B = z[item_slot2<M>(k)];
+    const Quad64 q = post_pair(A, k == 0 ? A : B, t, k);
+    s1 = mk(q.xk, q.xNk);
+    s2 = mk(q.xMk, q.xMpk);
     if (k == 0) {
         const Quad64 h = post_pair(B, B, t, M / 2);
-        q.xNk = h.xk;
-        q.xMpk = h.xNk;
+        s1.y = q.xMk;
+        s2 = mk(h.xk, h.xNk);
     }
-    return q;
 }
-template <int M> __device__ __forceinline__ void pre_item(const Quad64& X, const PairTab& t, int k, cx* z) {
+template <int M> __device__ __forceinline__ void pre_item(cx s1, cx s2, const PairTab& t, int k, cx* z) {
     cx a, b;
     if (k != 0) {
-        pre_pair(X, t, k, a, b);
-        z[k] = a;
-        z[M - k] = b;
+        pre_pair(Quad64{s1.x, s1.y, s2.x, s2.y}, t, k, a, b);
     } else {
-        pre_pair(Quad64{X.xk, fx{0}, X.xMk, X.xMk}, t, 0, a, b);
-        z[0] = a;
-        pre_pair(Quad64{X.xNk, X.xMpk, X.xNk, X.xMpk}, t, M / 2, a, b);
-        z[M / 2] = a;
+        cx c;
+        pre_pair(Quad64{s1.x, fx{0}, s1.y, s1.y}, t, 0, a, c);
+        pre_pair(Quad64{s2.x, s2.y, s2.x, s2.y}, t, M / 2, b, c);
     }
+    z[k] = a;
+    z[item_slot2<M>(k)] = b;
 }
 
 // Forward half-length transform of a real line at x (global, 16-byte aligned;
@@ -469,26 +477,26 @@ __device__ __forceinline__ int forward_line(const double* __restrict__ x, cx* bu
     return ex;
 }
 
-// Inverse: the line's modes X (items k = n2 + G i, four values each, in
-// orthonormal DCT coefficients) to the natural-order samples in buf (sample m:
-// x[4m], x[4m+2]; sample M-1-m: x[4m+3], x[4m+1]); the exponent in sm.ex[slot]
-// and returned.
-template <int M>
-__device__ __forceinline__ int inverse_line(double (&X)[2 * Geo<M>::E], cx* buf, const int4* __restrict__ tw2,
-                                             const PairTab& ti, int n2, int slot, LineSm<M>& sm) {
+// Inverse: the line's modes in buf as slots of doubles (orthonormal DCT
+// coefficients; mx: the largest mag_hi of this lane's) to the natural-order
+// samples in buf (sample m: x[4m], x[4m+2]; sample M-1-m: x[4m+3], x[4m+1]);
+// the exponent in sm.ex[slot] and returned.  OWN: every lane has filled the
+// slots of its own items k = n2 + G i itself.
+template <int M, bool OWN>
+__device__ __forceinline__ int inverse_line(unsigned mx, cx* buf, const int4* __restrict__ tw, const PairTab& ti, int n2,
+                                            int slot, LineSm<M>& sm) {
     constexpr int E = Geo<M>::E, G = Geo<M>::G;
-    unsigned mx = 0;
-#pragma unroll
-    for (int i = 0; i < 2 * E; ++i) mx = max(mx, mag_hi(X[i]));
     mx = line_max<M>(mx, slot, sm);
+    if constexpr (!OWN) sync_line<M>(slot);
     const bool bad = mx >= 0x7ff00000u;
     const int em = max((int)(mx >> 20), 1);
     // room for the pairs: a sample of z is at most 4 sqrt(2) times the largest mode
-#pragma unroll
+#pragma unroll 1
     for (int i = 0; i < E / 2; ++i) {
-        const Quad64 q{to_fixed(X[4 * i], em + 2), to_fixed(X[4 * i + 1], em + 2), to_fixed(X[4 * i + 2], em + 2),
-                       to_fixed(X[4 * i + 3], em + 2)};
-        pre_item<M>(q, ti, n2 + G * i, buf);
+        const int k = n2 + G * i;
+        const double2 p = reinterpret_cast<const double2*>(buf)[k], q = reinterpret_cast<const double2*>(buf)[item_slot2<M>(k)];
+        pre_item<M>(mk(to_fixed(p.x, em + 2), to_fixed(p.y, em + 2)), mk(to_fixed(q.x, em + 2), to_fixed(q.y, em + 2)), ti, k,
+                    buf);
     }
     int ex = em + 2 - 1082 + ti.p, sh;
     sync_line<M>(slot);
@@ -497,7 +505,7 @@ __device__ __forceinline__ int inverse_line(double (&X)[2 * Geo<M>::E], cx* buf,
     for (int i = 0; i < E; ++i) v[i] = buf[G * i + n2];
     sync_line<M>(slot);
     fit_line<M>(v, slot, sm, ex, sh);
-    fft_line<M, true>(v, buf, tw2, n2, slot, sh);
+    fft_line<M, true>(v, buf, tw, n2, slot, sh);
     if (bad) ex = kBad;
     if (n2 == 0) sm.ex[slot] = ex;
     return ex;

@@ -4,11 +4,11 @@
 // the Neumann / Dirichlet solver (spectral_solve.cu, and the preconditioner
 // of the classical scheme).
 //
-// Spectra: spec[kx][f][4 k + u], f = f0' S H Q K P g0' L_P, item k = 0 .. M/2 - 1,
-// u its four modes (fixed_fft.cuh, item_mode): every access to them is 32
-// contiguous bytes per lane.  isig = 1/sigma and itau = 1/tau are tables in
-// the same order (they depend on the parameters only; evaluating them costs
-// ten FP64 instructions a mode in each of two kernels, reading them 16 bytes).
+// Spectra: spec[kx][f][2 i + c], f = f0' S H Q K P g0' L_P, in the slot order of
+// fixed_fft.cuh: sixteen contiguous bytes per slot.  isig = 1/sigma and itau =
+// 1/tau are tables in the same order (they depend on the parameters only;
+// evaluating them costs ten FP64 instructions a mode in each of two kernels,
+// reading them 16 bytes).
 #pragma once
 #include "step_kernels.cuh"
 #include "fixed_fft.cuh"
@@ -19,18 +19,18 @@ namespace xf {
 
 inline PairTab pair_fwd(const Tables& t) {
     const int n = t.M / 2 + 1;
-    return PairTab{t.mem + t.M, t.mem + t.M + n, t.mem + t.M + 2 * n, -t.pf};
+    return PairTab{t.mem + 2 * t.M, t.mem + 2 * t.M + n, t.mem + 2 * t.M + 2 * n, -t.pf};
 }
 inline PairTab pair_inv(const Tables& t) {
     const int n = t.M / 2 + 1;
-    return PairTab{t.mem + t.M, t.mem + t.M + 3 * n, t.mem + t.M + 4 * n, -t.pi};
+    return PairTab{t.mem + 2 * t.M, t.mem + 2 * t.M + 3 * n, t.mem + 2 * t.M + 4 * n, -t.pi};
 }
 
 // ------------------------------------------------------------------ forward rows
 // Forward DCT-II along x of LINES rows of field blockIdx.y, written
 // transposed: out[f][kx][y0 + r].  n: values per array (index checks).
 template <int M, bool DST>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_row_fwd(const double* __restrict__ in, double* __restrict__ out, const int4* __restrict__ tw2, PairTab tf,
            const int* __restrict__ dskip, size_t fstride, size_t n) {
     using Gm = Geo<M>;
@@ -46,14 +46,17 @@ kx_row_fwd(const double* __restrict__ in, double* __restrict__ out, const int4* 
     forward_line<M, DST>(in + CCM_IXW(f0 + (size_t)(y0 + slot) * N, N, n), bufs + (size_t)slot * Gm::BUF, tw2, n2, slot, sm,
                          (y0 + slot) & 1);
     __syncthreads();
+#pragma unroll 1
     for (int q = threadIdx.x; q < L * (M / 2); q += Gm::THREADS) {
         const int r = q % L, k = q / L, ex = sm.ex[r];
-        const Quad64 X = post_item<M>(bufs + (size_t)r * Gm::BUF, tf, k);
-        const fx v[4] = {X.xk, X.xNk, X.xMk, X.xMpk};
+        cx s[2];
+        post_item<M>(bufs + (size_t)r * Gm::BUF, tf, k, s[0], s[1]);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t o = f0 + (size_t)item_mode<M>(k, u) * N + y0 + r;
-            if (CCM_OK(o, n)) out[o] = line_double(v[u], ex, tf.p);
+        for (int u = 0; u < 2; ++u) {
+            const int i = u ? item_slot2<M>(k) : k;
+            const size_t o0 = f0 + (size_t)slot_mode<M>(i, 0) * N + y0 + r, o1 = f0 + (size_t)slot_mode<M>(i, 1) * N + y0 + r;
+            if (CCM_OK(o0, n)) out[o0] = line_double(s[u].x, ex, tf.p);
+            if (CCM_OK(o1, n)) out[o1] = line_double(s[u].y, ex, tf.p);
         }
     }
 }
@@ -114,50 +117,59 @@ __device__ __forceinline__ void gram_store(double (&acc)[16], double* __restrict
     }
     if (threadIdx.x == 16) row[0] = 0.0;
 }
-__device__ __forceinline__ vec4<double> ldq(const double* __restrict__ p) {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
-    return {a.x, a.y, b.x, b.y};
-}
+__device__ __forceinline__ double2 ld2(const double* __restrict__ p) { return __ldg(reinterpret_cast<const double2*>(p)); }
 
 // Forward DCT-II along y of the eight fields of a spectral row kx (one line
 // per lane group), the spectra and the Gram sums; each CTA takes the rows
-// blockIdx.x, blockIdx.x + gridDim.x, ... and leaves one partial row.
+// blockIdx.x, blockIdx.x + gridDim.x, ... and leaves one partial row.  The
+// post-process turns each line's buffer into doubles in place (every item
+// writes the two slots it read), and the Gram sums read the eight fields'
+// slots from there.
 template <int M>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_col_gram(const double* __restrict__ in, double* __restrict__ spec, double* __restrict__ part,
             const int4* __restrict__ tw2, PairTab tf, const double* __restrict__ isig, const double* __restrict__ itau) {
     using Gm = Geo<M>;
-    constexpr int N = Gm::N;
+    constexpr int N = Gm::N, G = Gm::G;
     static_assert(Gm::LINES == NF, "one line per field");
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ LineSm<M> sm;
     cx* bufs = reinterpret_cast<cx*>(smraw);
     int n2, slot;
     lane_of<M>(n2, slot);
+    cx* buf = bufs + (size_t)slot * Gm::BUF;
     const size_t NN = (size_t)N * N;
     double acc[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[i] = 0.0;
     for (int kx = blockIdx.x; kx < N; kx += gridDim.x) {
-        forward_line<M, false>(in + CCM_IXW(slot * NN + (size_t)kx * N, N, NF * NN), bufs + (size_t)slot * Gm::BUF, tw2, n2,
-                               slot, sm, false);
+        const int ex = forward_line<M, false>(in + CCM_IXW(slot * NN + (size_t)kx * N, N, NF * NN), buf, tw2, n2, slot, sm, false);
+        double* srow = spec + CCM_IXW(((size_t)kx * NF + slot) * N, N, NF * NN);
+#pragma unroll 1
+        for (int k = n2; k < M / 2; k += G) {
+            cx s[2];
+            post_item<M>(buf, tf, k, s[0], s[1]);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int i = u ? item_slot2<M>(k) : k;
+                const double2 d = make_double2(line_double(s[u].x, ex, tf.p), line_double(s[u].y, ex, tf.p));
+                reinterpret_cast<double2*>(buf)[i] = d;
+                if (slot != 5) reinterpret_cast<double2*>(srow)[i] = d;        // P^ enters the Gram sums only
+            }
+        }
         __syncthreads();
-        for (int k = threadIdx.x; k < M / 2; k += Gm::THREADS) {
-            double v[4][NF];
-            double* srow = spec + CCM_IXW((size_t)kx * NF * N, NF * N, NF * NN) + 4 * k;
+#pragma unroll 1
+        for (int i = threadIdx.x; i < M; i += Gm::THREADS) {
+            const double2 ws = ld2(isig + (size_t)kx * N + 2 * i), wt = ld2(itau + (size_t)kx * N + 2 * i);
+            double a[NF], b[NF];
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                const Quad64 q = post_item<M>(bufs + (size_t)f * Gm::BUF, tf, k);
-                const int ex = sm.ex[f];
-                v[0][f] = line_double(q.xk, ex, tf.p); v[1][f] = line_double(q.xNk, ex, tf.p);
-                v[2][f] = line_double(q.xMk, ex, tf.p); v[3][f] = line_double(q.xMpk, ex, tf.p);
-                if (f != 5) st4(srow + (size_t)f * N, vec4<double>{v[0][f], v[1][f], v[2][f], v[3][f]});
+                const double2 d = reinterpret_cast<const double2*>(bufs + (size_t)f * Gm::BUF)[i];
+                a[f] = d.x;
+                b[f] = d.y;
             }
-            const vec4<double> ws = ldq(isig + (size_t)kx * N + 4 * k), wt = ldq(itau + (size_t)kx * N + 4 * k);
-            gram_mode(acc, v[0], ws.a, wt.a);
-            gram_mode(acc, v[1], ws.b, wt.b);
-            gram_mode(acc, v[2], ws.c, wt.c);
-            gram_mode(acc, v[3], ws.d, wt.d);
+            gram_mode(acc, a, ws.x, wt.x);
+            gram_mode(acc, b, ws.y, wt.y);
         }
         __syncthreads();
     }
@@ -167,7 +179,7 @@ kx_col_gram(const double* __restrict__ in, double* __restrict__ spec, double* __
 // Lines too long for eight buffers per CTA (M >= 2048): the spectra of LINES
 // rows of field blockIdx.y, and the Gram sums from them in a second kernel.
 template <int M>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_col_fwd(const double* __restrict__ in, double* __restrict__ spec, const int4* __restrict__ tw2, PairTab tf) {
     using Gm = Geo<M>;
     constexpr int N = Gm::N;
@@ -180,10 +192,14 @@ kx_col_fwd(const double* __restrict__ in, double* __restrict__ spec, const int4*
     const int f = blockIdx.y, kx = blockIdx.x * Gm::LINES + slot;
     const int ex = forward_line<M, false>(in + CCM_IXW(f * NN + (size_t)kx * N, N, NF * NN), buf, tw2, n2, slot, sm, false);
     double* srow = spec + CCM_IXW(((size_t)kx * NF + f) * N, N, NF * NN);
+#pragma unroll 1
     for (int k = n2; k < M / 2; k += Gm::G) {
-        const Quad64 q = post_item<M>(buf, tf, k);
-        st4(srow + 4 * k, vec4<double>{line_double(q.xk, ex, tf.p), line_double(q.xNk, ex, tf.p),
-                                       line_double(q.xMk, ex, tf.p), line_double(q.xMpk, ex, tf.p)});
+        cx s[2];
+        post_item<M>(buf, tf, k, s[0], s[1]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            reinterpret_cast<double2*>(srow)[u ? item_slot2<M>(k) : k] =
+                make_double2(line_double(s[u].x, ex, tf.p), line_double(s[u].y, ex, tf.p));
     }
 }
 constexpr int kGramThreads = 256;
@@ -205,12 +221,11 @@ kx_gram_rows(const double* __restrict__ spec, double* __restrict__ part, int N, 
 }
 
 // isig, itau in the order of the spectra
-template <int M> __device__ __forceinline__ int slot_mode(int j) { return item_mode<M>(j >> 2, j & 3); }
 template <int M>
 __global__ void kx_weights(const double* __restrict__ ev, SpecCoef sc, double* __restrict__ isig, double* __restrict__ itau) {
     constexpr size_t N = 2 * M;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < N * N; q += (size_t)gridDim.x * blockDim.x) {
-        const double s = ev[q / N] + ev[slot_mode<M>((int)(q % N))];
+        const double s = ev[q / N] + ev[slot_mode<M>((int)(q % N) >> 1, (int)(q & 1))];
         isig[q] = recip(fma(fma(sc.C3, s, sc.C2), s, sc.C1));
         itau[q] = recip(fma(sc.lam, s, sc.Ct));
     }
@@ -223,6 +238,7 @@ __device__ __forceinline__ void write_transposed(const cx* bufs, const LineSm<M>
                                                  int x0, size_t n) {
     using Gm = Geo<M>;
     constexpr int N = Gm::N, L = Gm::LINES;
+#pragma unroll 1
     for (int q = threadIdx.x; q < L * (M / 2); q += Gm::THREADS) {
         const int r = q % L, m = q / L;
         const vec4<double> v = unpack_item<M>(bufs + (size_t)r * Gm::BUF, m, sm.ex[r]);
@@ -239,7 +255,7 @@ __device__ __forceinline__ void write_transposed(const cx* bufs, const LineSm<M>
 // LINES spectral rows of field blockIdx.y (0: phi, 1: psi): recovery
 // combination, inverse DCT along y, transposed write out[f][y][kx].
 template <int M>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_comb_icol(const double* __restrict__ spec, double* __restrict__ out, const int4* __restrict__ tw2, PairTab ti,
              const double* __restrict__ isig, const double* __restrict__ itau, const DevScalars* __restrict__ dsc) {
     using Gm = Geo<M>;
@@ -252,54 +268,60 @@ kx_comb_icol(const double* __restrict__ spec, double* __restrict__ out, const in
     const size_t NN = (size_t)N * N;
     const int f = blockIdx.y, x0 = blockIdx.x * Gm::LINES, kx = x0 + slot;
     const double* s = spec + CCM_IXW((size_t)kx * NF * N, NF * N, NF * NN);
-    double X[2 * E];
+    cx* buf = bufs + (size_t)slot * Gm::BUF;
+    unsigned mx = 0;
+    auto put = [&](int i, double x, double y) {
+        reinterpret_cast<double2*>(buf)[i] = make_double2(x, y);
+        mx = max(mx, max(mag_hi(x), mag_hi(y)));
+    };
     if (f == 0) {
         const double aS = -dsc->alpha[0], aH = -dsc->alpha[1], aQ = -dsc->alpha[2], aK = -dsc->alpha[3];
-#pragma unroll
-        for (int i = 0; i < E / 2; ++i) {
-            const int o = 4 * (n2 + G * i);
-            const vec4<double> v0 = ldq(s + o), v1 = ldq(s + N + o), v2 = ldq(s + 2 * N + o), v3 = ldq(s + 3 * N + o),
-                               v4 = ldq(s + 4 * N + o), w = ldq(isig + (size_t)kx * N + o);
-            X[4 * i] = fma(aK, v4.a, fma(aQ, v3.a, fma(aH, v2.a, fma(aS, v1.a, v0.a)))) * w.a;
-            X[4 * i + 1] = fma(aK, v4.b, fma(aQ, v3.b, fma(aH, v2.b, fma(aS, v1.b, v0.b)))) * w.b;
-            X[4 * i + 2] = fma(aK, v4.c, fma(aQ, v3.c, fma(aH, v2.c, fma(aS, v1.c, v0.c)))) * w.c;
-            X[4 * i + 3] = fma(aK, v4.d, fma(aQ, v3.d, fma(aH, v2.d, fma(aS, v1.d, v0.d)))) * w.d;
+#pragma unroll 4
+        for (int j = 0; j < E; ++j) {
+            const int i = n2 + G * j;
+            const double2 v0 = ld2(s + 2 * i), v1 = ld2(s + N + 2 * i), v2 = ld2(s + 2 * N + 2 * i), v3 = ld2(s + 3 * N + 2 * i),
+                          v4 = ld2(s + 4 * N + 2 * i), w = ld2(isig + (size_t)kx * N + 2 * i);
+            put(i, fma(aK, v4.x, fma(aQ, v3.x, fma(aH, v2.x, fma(aS, v1.x, v0.x)))) * w.x,
+                fma(aK, v4.y, fma(aQ, v3.y, fma(aH, v2.y, fma(aS, v1.y, v0.y)))) * w.y);
         }
     } else {
         const double aL = dsc->alpha[4];
-#pragma unroll
-        for (int i = 0; i < E / 2; ++i) {
-            const int o = 4 * (n2 + G * i);
-            const vec4<double> v6 = ldq(s + 6 * N + o), v7 = ldq(s + 7 * N + o), w = ldq(itau + (size_t)kx * N + o);
-            X[4 * i] = fma(aL, v7.a, v6.a) * w.a;
-            X[4 * i + 1] = fma(aL, v7.b, v6.b) * w.b;
-            X[4 * i + 2] = fma(aL, v7.c, v6.c) * w.c;
-            X[4 * i + 3] = fma(aL, v7.d, v6.d) * w.d;
+#pragma unroll 8
+        for (int j = 0; j < E; ++j) {
+            const int i = n2 + G * j;
+            const double2 v6 = ld2(s + 6 * N + 2 * i), v7 = ld2(s + 7 * N + 2 * i), w = ld2(itau + (size_t)kx * N + 2 * i);
+            put(i, fma(aL, v7.x, v6.x) * w.x, fma(aL, v7.y, v6.y) * w.y);
         }
     }
-    inverse_line<M>(X, bufs + (size_t)slot * Gm::BUF, tw2, ti, n2, slot, sm);
+    inverse_line<M, false>(mx, buf, tw2, ti, n2, slot, sm);
     __syncthreads();
     write_transposed<M>(bufs, sm, out, f * NN, x0, 2 * NN);
 }
 
 // ------------------------------------------------------------------ inverse rows
-// This lane's modes of a row in natural order.
-template <int M> __device__ __forceinline__ void load_modes(double (&X)[2 * Geo<M>::E], const double* row, int n2) {
-#pragma unroll
-    for (int i = 0; i < Geo<M>::E / 2; ++i)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) X[4 * i + u] = row[item_mode<M>(n2 + Geo<M>::G * i, u)];
+// A row's modes (natural order, global) to slots of doubles in buf; returns
+// the largest mag_hi of this lane's.
+template <int M> __device__ __forceinline__ unsigned load_modes(cx* buf, const double* row, int n2) {
+    unsigned mx = 0;
+#pragma unroll 8
+    for (int j = 0; j < Geo<M>::E; ++j) {
+        const int i = n2 + Geo<M>::G * j;
+        const double x = row[i], y = row[slot_mode<M>(i, 1)];
+        reinterpret_cast<double2*>(buf)[i] = make_double2(x, y);
+        mx = max(mx, max(mag_hi(x), mag_hi(y)));
+    }
+    return mx;
 }
 
 // Inverse DCT along x of LINES rows of field blockIdx.y and
 // u^{n+1} = u_bar + du.
 template <int M>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_irow(const double* __restrict__ in, double* __restrict__ phi_new, double* __restrict__ psi_new,
         const int4* __restrict__ tw2, PairTab ti, const double* __restrict__ phn, const double* __restrict__ pho,
         const double* __restrict__ psn, const double* __restrict__ pso, int bdf1) {
     using Gm = Geo<M>;
-    constexpr int N = Gm::N, E = Gm::E, G = Gm::G;
+    constexpr int N = Gm::N, G = Gm::G;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ LineSm<M> sm;
     int n2, slot;
@@ -307,17 +329,18 @@ kx_irow(const double* __restrict__ in, double* __restrict__ phi_new, double* __r
     cx* buf = reinterpret_cast<cx*>(smraw) + (size_t)slot * Gm::BUF;
     const size_t NN = (size_t)N * N;
     const int f = blockIdx.y, y = blockIdx.x * Gm::LINES + slot;
-    double X[2 * E];
-    load_modes<M>(X, in + CCM_IXW(f * NN + (size_t)y * N, N, 2 * NN), n2);
-    const int ex = inverse_line<M>(X, buf, tw2, ti, n2, slot, sm);
+    const unsigned mx = load_modes<M>(buf, in + CCM_IXW(f * NN + (size_t)y * N, N, 2 * NN), n2);
+    const int ex = inverse_line<M, false>(mx, buf, tw2, ti, n2, slot, sm);
     const double* un = f ? psn : phn;
     const double* uo = f ? pso : pho;
     double* u = f ? psi_new : phi_new;
+#pragma unroll 2
     for (int m = n2; m < M / 2; m += G) {
         const size_t o = CCM_IXW((size_t)y * N + 4 * m, 4, NN);
         const vec4<double> d = unpack_item<M>(buf, m, ex), a = ld4(un + o), b = ld4(uo + o);
-        st4(u + o, vec4<double>{bar_add(a.a, b.a, d.a, 0.0, bdf1 != 0), bar_add(a.b, b.b, d.b, 0.0, bdf1 != 0),
-                                bar_add(a.c, b.c, d.c, 0.0, bdf1 != 0), bar_add(a.d, b.d, d.d, 0.0, bdf1 != 0)});
+        // u_bar + du without the FP32 path's correction term (an FP64 addition less)
+        auto add = [&](double p, double q, double x) { return (bdf1 ? p : fma(p - q, 1.0 / 3.0, p)) + x; };
+        st4(u + o, vec4<double>{add(a.a, b.a, d.a), add(a.b, b.b, d.b), add(a.c, b.c, d.c), add(a.d, b.d, d.d)});
     }
 }
 
@@ -325,7 +348,7 @@ kx_irow(const double* __restrict__ in, double* __restrict__ phi_new, double* __r
 // LINES spectral rows (contiguous over y): forward DCT along y, division by
 // c0 + c1 s + c2 s^2, inverse DCT, transposed write out[y][kx].
 template <int M>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_col_solve(const double* __restrict__ in, double* __restrict__ out, const int4* __restrict__ tw2, PairTab tf, PairTab ti,
              const double* __restrict__ ev, double c0, double c1, double c2, const double* __restrict__ dcoef,
              const int* __restrict__ dskip, size_t fstride) {
@@ -342,30 +365,34 @@ kx_col_solve(const double* __restrict__ in, double* __restrict__ out, const int4
     const int x0 = blockIdx.x * Gm::LINES, kx = x0 + slot;
     const int ex = forward_line<M, false>(in + blockIdx.y * fstride + (size_t)kx * N, buf, tw2, n2, slot, sm, false);
     const double evx = ev[kx];
-    double X[2 * E];
+    unsigned mx = 0;
+#pragma unroll 1
+    for (int j = 0; j < E / 2; ++j) {
+        const int k = n2 + G * j;
+        cx z[2];
+        post_item<M>(buf, tf, k, z[0], z[1]);
 #pragma unroll
-    for (int i = 0; i < E / 2; ++i) {
-        const int k = n2 + G * i;
-        const Quad64 q = post_item<M>(buf, tf, k);
-        const fx v[4] = {q.xk, q.xNk, q.xMk, q.xMpk};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const double s = evx + __ldg(ev + item_mode<M>(k, u));
-            X[4 * i + u] = line_double(v[u], ex, tf.p) * recip(c0 + s * (c1 + c2 * s));
+        for (int u = 0; u < 2; ++u) {
+            const int i = u ? item_slot2<M>(k) : k;
+            const double sx = evx + __ldg(ev + slot_mode<M>(i, 0)), sy = evx + __ldg(ev + slot_mode<M>(i, 1));
+            const double x = line_double(z[u].x, ex, tf.p) * recip(c0 + sx * (c1 + c2 * sx));
+            const double y = line_double(z[u].y, ex, tf.p) * recip(c0 + sy * (c1 + c2 * sy));
+            reinterpret_cast<double2*>(buf)[i] = make_double2(x, y);
+            mx = max(mx, max(mag_hi(x), mag_hi(y)));
         }
     }
-    inverse_line<M>(X, buf, tw2, ti, n2, slot, sm);    // writes only the slots this lane has read before its first barrier
+    inverse_line<M, true>(mx, buf, tw2, ti, n2, slot, sm);
     __syncthreads();
     write_transposed<M>(bufs, sm, out, blockIdx.y * fstride, x0, ~(size_t)0);
 }
 
 // Inverse DCT along x of LINES rows (in place allowed).  DST: times (-1)^(i+j).
 template <int M, bool DST>
-__global__ void __launch_bounds__(Geo<M>::THREADS)
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
 kx_row_inv(const double* in, double* out, const int4* __restrict__ tw2, PairTab ti, const int* __restrict__ dskip,
            size_t fstride) {
     using Gm = Geo<M>;
-    constexpr int N = Gm::N, E = Gm::E, G = Gm::G;
+    constexpr int N = Gm::N, G = Gm::G;
     if (dskip && dskip[blockIdx.y]) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ LineSm<M> sm;
@@ -374,9 +401,9 @@ kx_row_inv(const double* in, double* out, const int4* __restrict__ tw2, PairTab 
     cx* buf = reinterpret_cast<cx*>(smraw) + (size_t)slot * Gm::BUF;
     const int y = blockIdx.x * Gm::LINES + slot;
     const size_t o = blockIdx.y * fstride + (size_t)y * N;
-    double X[2 * E];
-    load_modes<M>(X, in + o, n2);
-    const int ex = inverse_line<M>(X, buf, tw2, ti, n2, slot, sm);
+    const unsigned mx = load_modes<M>(buf, in + o, n2);
+    const int ex = inverse_line<M, false>(mx, buf, tw2, ti, n2, slot, sm);
+#pragma unroll 2
     for (int m = n2; m < M / 2; m += G) {
         vec4<double> v = unpack_item<M>(buf, m, ex);
         if (DST) {                                     // x = 4m is even: signs (+, -, +, -) times (-1)^y

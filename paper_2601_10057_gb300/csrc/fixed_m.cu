@@ -84,13 +84,18 @@ int4 entry(long double x, long double y) {
 void fill(int4* t, int* pf, int* pi) {
     const Circle* w = new Circle(4L * N);                          // steps of pi / 2N
     long double c, s;
-    for (int k1 = 0; k1 < Gm::E; ++k1)
+    for (int k1 = 0; k1 < Gm::A; ++k1)
         for (int n2 = 0; n2 < Gm::G; ++n2) {
             w->at(8L * ((long)n2 * k1 % M), c, s);                 // W_M = 8 steps
             t[k1 * Gm::G + n2] = entry(c, -s);
         }
+    for (int kc = 0; kc < Gm::C; ++kc)
+        for (int d = 0; d < Gm::D; ++d) {
+            w->at(8L * Gm::A * ((long)d * kc % Gm::B), c, s);      // W_B = W_M^A
+            t[M + kc * Gm::D + d] = entry(c, -s);
+        }
     const int np = M / 2 + 1;
-    int4 *wn = t + M, *fa = wn + np, *fb = fa + np, *ia = fb + np, *ib = ia + np;
+    int4 *wn = t + 2 * M, *fa = wn + np, *fb = fa + np, *ia = fb + np, *ib = ia + np;
     int lg = 0;
     while ((1 << lg) < N) ++lg;
     const long double h = sqrtl(0.5L);

@@ -26,8 +26,8 @@ const Ops* fixed_ops(int M) {
 
 int make_tables(const Ops* o, Tables& t, cudaStream_t st) {
     t.M = o->M;
-    const size_t n = (size_t)t.M + 5 * (size_t)(t.M / 2 + 1);
-    std::vector<int4> h(n);
+    const size_t n = 2 * (size_t)t.M + 5 * (size_t)(t.M / 2 + 1);
+    std::vector<int4> h(n, int4{0, 0, 0, 0});
     o->fill(h.data(), &t.pf, &t.pi);
     if (cudaMalloc(&t.mem, n * sizeof(int4)) != cudaSuccess) { t.mem = nullptr; return CCMSAV_ENOMEM; }
     if (cudaMemcpyAsync(t.mem, h.data(), n * sizeof(int4), cudaMemcpyHostToDevice, st) != cudaSuccess ||

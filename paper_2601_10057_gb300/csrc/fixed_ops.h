@@ -8,10 +8,37 @@
 namespace ccm {
 struct SpecCoef;
 struct DevScalars;
+template <typename T> struct StencilCoef;
 namespace xf {
 
-// Twiddle and pair tables of one line length (device, one allocation: tw2 [M],
-// then the pair tables wn, forward a, b, inverse a, b [M/2 + 1 each]; each
+// A factor w (|w| <= 2^62, 62 fractional bits) as w = h 2^32 + l with l a
+// signed word; h and -h, -l fit 32 bits.
+struct Fac { int h, l; };
+__host__ __device__ constexpr Fac fac(long long w) {
+    return Fac{(int)((w + 0x80000000LL) >> 32), (int)(w & 0xffffffffLL)};
+}
+
+// Coefficients of the fixed-point stencil (fixed_stencil.cuh).  x_c: factors;
+// _exp: exponents of the outputs (value = fixed 2^exp); long long: with 60
+// fractional bits.  al .. s0: P 2^-g = (al psi - al0) + p (be psi - be0),
+// (f_in -+ f_out) 2^-g = (d2 psi + d1) psi + d0 and s2, s1, s0.
+struct StencilFix {
+    int bdf1;
+    int f_exp, s_exp, h_exp, q_exp, p_exp, gexp;
+    Fac f_lap, f_lap2, f_th, f_bar, s_c, betaf, h_p, h_l, q_x, q_t, M0, al, be, d2, s2, qpi;
+    long long beta, al0, be0, d1, d0, s1, s0;
+    double g_c, l_c, wV, wA, wB, wZ;
+};
+// false: parameters outside the kernel's range (the caller takes k_stencil)
+bool make_stencil(const StencilCoef<double>& c, StencilFix& k);
+int stencil_setup(int N);                // shared-memory opt-in of the kernel for N x N fields
+int stencil_rows(int N);                 // partial rows it writes
+void stencil(const double* phn, const double* pho, const double* psn, const double* pso, double* out, double* part, int N,
+             const StencilFix& k, const StencilCoef<double>& c, cudaStream_t st);
+int stencil_oob(unsigned* flag);         // as Ops::oob
+
+// Twiddle and pair tables of one line length (device, one allocation: the
+// twiddles of the two exchanges [M each], then the pair tables wn, forward a, b, inverse a, b [M/2 + 1 each]; each
 // entry a complex factor with 62 fractional bits as two (high, signed low)
 // word pairs).
 struct Tables {
@@ -23,7 +50,7 @@ struct Ops {
     int M;
     // opt in to the kernels' shared memory; *gram_rows: partial rows that col_gram leaves
     int (*setup)(int* gram_rows);
-    // host values of the tables' M + 5 (M/2 + 1) entries and the powers of two
+    // host values of the tables' 2 M + 5 (M/2 + 1) entries and the powers of two
     void (*fill)(int4* host, int* pf, int* pi);
     void (*weights)(const double* ev, const SpecCoef& sc, double* isig, double* itau, cudaStream_t st);
     // the four transform kernels of a step (fields in a, b as in SimImpl's bufA, bufB)

@@ -83,6 +83,7 @@ public:
     double* isig = nullptr;
     double* itau = nullptr;
     int xrows = 0;               // partial rows of the Gram sums
+    int nb1x = 0;                // partial rows of the fixed-point stencil
     int wRT = 8, wlds = 0, wRT4 = 4, wlds4 = 0, wKC = 1, wRI = 4;
     int ahead_rt = 0;   // L2 prefetch distance of the row kernel (0: none)
     size_t wsm_rt = 0, wsm_col = 0, wsm_comb = 0, wsm_irow = 0;
@@ -368,10 +369,13 @@ public:
         if (cudaMalloc(&bufB, 8 * fb) != cudaSuccess) return CCMSAV_ENOMEM;
         b_st = dim3(TX, TY);
         g_st = dim3((N + TX - 1) / TX, (N + TYB - 1) / TYB);
+        const char* force_block = std::getenv("CCMSAV_FORCE_BLOCK_FFT");   // test switch: block-FFT kernels only
+        if (std::is_same<T, double>::value && !(force_block && force_block[0] == '1')) xo = xf::fixed_ops(M);
         nb1 = g_st.x * g_st.y;
+        nb1x = xo ? xf::stencil_rows(N) : 0;
         g_dg = dim3((N + 31) / 32, (N + 8 * kDiagRows - 1) / (8 * kDiagRows));
         nbd = g_dg.x * g_dg.y;
-        if (cudaMalloc(&part1, (size_t)nb1 * NRED1 * sizeof(double)) != cudaSuccess) return CCMSAV_ENOMEM;
+        if (cudaMalloc(&part1, (size_t)std::max(nb1, nb1x) * NRED1 * sizeof(double)) != cudaSuccess) return CCMSAV_ENOMEM;
         if (cudaMalloc(&part2, (size_t)N * NRED2 * sizeof(double)) != cudaSuccess) return CCMSAV_ENOMEM;
         if (cudaMalloc(&partd, (size_t)nbd * NDIAG * sizeof(double)) != cudaSuccess) return CCMSAV_ENOMEM;
         if (cudaMalloc(&part3, (size_t)kSolveBlocks * NRQ * sizeof(double)) != cudaSuccess) return CCMSAV_ENOMEM;
@@ -442,13 +446,12 @@ public:
             int r = init_classical();
             if (r) return r;
         }
-        const char* force_block = std::getenv("CCMSAV_FORCE_BLOCK_FFT");   // test switch: block-FFT kernels only
         if (std::is_same<T, float>::value && M >= 64 && M <= 4096 && !(force_block && force_block[0] == '1')) {
             int r = init_warp_path();
             if (r) return r;
         }
         if constexpr (std::is_same<T, double>::value)
-            if (!(force_block && force_block[0] == '1') && (xo = xf::fixed_ops(M)))
+            if (xo)
                 if (const int r = init_fixed()) return r;
         CCM_CUDA(cudaStreamSynchronize(st));
         return CCMSAV_OK;
@@ -456,6 +459,7 @@ public:
 
     int init_fixed() {
         if (const int r = xo->setup(&xrows)) return r;
+        if (const int r = xf::stencil_setup(N)) return r;
         if (const int r = xf::make_tables(xo, xt, st)) return r;
         if (cudaMalloc(&isig, NN * sizeof(double)) != cudaSuccess || cudaMalloc(&itau, NN * sizeof(double)) != cudaSuccess)
             return CCMSAV_ENOMEM;
@@ -737,8 +741,9 @@ public:
         CCM_CUDA(cudaMemcpyFromSymbol(&v, g_oob_flag, sizeof(v)));
         CCM_CUDA(cudaMemcpyToSymbol(g_oob_flag, &z, sizeof(z)));
         unsigned x = 0;
-        if (xo && xo->oob(&x)) return CCMSAV_ECUDA;
-        return (int)(v | x);
+        unsigned y = 0;
+        if (xo && (xo->oob(&x) || xf::stencil_oob(&y))) return CCMSAV_ECUDA;
+        return (int)(v | x | y);
 #else
         return CCMSAV_EINVAL;
 #endif
@@ -1124,8 +1129,17 @@ public:
 
         if (prof && ev_used + 16 > 4096) { int r = profile_flush(); if (r) return r; }
         mark(-1);
-        k_stencil<T><<<g_st, b_st, stencil_smem_bytes<T>(), st>>>(phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, c,
-                                                              GroupArgs<false>{}, 0);
+        bool fixed = false;
+        if constexpr (std::is_same<T, double>::value) {
+            xf::StencilFix k;
+            if (xo && (fixed = xf::make_stencil(c, k))) {
+                xf::stencil(phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, k, c, st);
+                so.nb1 = nb1x;
+            }
+        }
+        if (!fixed)
+            k_stencil<T><<<g_st, b_st, stencil_smem_bytes<T>(), st>>>(phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, c,
+                                                                  GroupArgs<false>{}, 0);
         mark(0);
         if (classical) {
             int r = queue_classical_ch(bdf1);

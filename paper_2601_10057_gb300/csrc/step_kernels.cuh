@@ -408,13 +408,13 @@ __device__ __forceinline__ double bar_add(double a, double b, double du, double 
 constexpr int TX = 64, TY = 4, TYB = 32;
 template <typename T> constexpr bool kBarLo = std::is_same<T, float>::value;
 
-template <typename T, bool GRP = false>
-__global__ void __launch_bounds__(TX * TY)
-k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
-          const T* __restrict__ psn, const T* __restrict__ pso,
-          T* __restrict__ out, double* __restrict__ part, int N, StencilCoef<T> c,
-          const __grid_constant__ GroupArgs<GRP> ga, int bps) {
-    extern __shared__ __align__(16) unsigned char smraw[];
+// One tile of the stencil: CTA column bx, row by of a grid of gx columns; a
+// CTA of TX x TY threads, smraw stencil_smem_bytes of shared memory.
+template <typename T, int TX, int TY, int TYB>
+__device__ __forceinline__ void
+stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restrict__ pho,
+             const T* __restrict__ psn, const T* __restrict__ pso,
+             T* __restrict__ out, double* __restrict__ part, int N, const StencilCoef<T>& c, int bx, int by, int gx) {
     constexpr int W2 = TX + 4, W1 = TX + 2, H1 = TYB + 2;
     T* sbar = reinterpret_cast<T*>(smraw);              // [TYB+4][W2]
     T* sph = sbar + (TYB + 4) * W2;                     // [H1][W1] each below
@@ -426,16 +426,7 @@ k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
     __shared__ double sred[(TX * TY / 32) * 4];
     __shared__ double smean[2][TX * TY / 32];
     __shared__ T smin[TX * TY / 32];
-    int bx = blockIdx.x, gx = gridDim.x;
-    if constexpr (GRP) {          // grouped launch (FP32)
-        static_assert(std::is_same<T, float>::value, "grouped launches are FP32");
-        const int sim = blockIdx.x / bps;
-        bx = blockIdx.x - sim * bps;
-        gx = bps;
-        const BatchArgs& A = ga.a[sim];
-        phn = A.phn; pho = A.pho; psn = A.psn; pso = A.pso; out = A.bufA; part = A.part1; c = A.c;
-    }
-    const int i0 = bx * TX, j0 = blockIdx.y * TYB;
+    const int i0 = bx * TX, j0 = by * TYB;
     const int tid = threadIdx.y * TX + threadIdx.x;
     // with d = u^n - u^{n-1} (exact for nearby values): u* = u^n + d,
     // u_bar = u^n + d/3, u_bar - u* = -2d/3 (BDF1: u* = u_bar = u^n)
@@ -592,7 +583,7 @@ k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
             if (gj + 1 < N) mm = min(mm, mN);
         }
     }
-    const size_t prow_i = (size_t)(blockIdx.y * gx + bx) * NRED1;
+    const size_t prow_i = (size_t)(by * gx + bx) * NRED1;
     const int lane = tid & 31, wp = tid >> 5;
     const T w0 = warp_sum(acc0), w1 = warp_sum(acc1), w2 = warp_sum(acc2);
     mm = warp_min(mm);
@@ -640,6 +631,25 @@ k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
             prow[8] = (double)m; prow[9] = 0;
         }
     }
+}
+
+template <typename T, bool GRP = false>
+__global__ void __launch_bounds__(TX * TY)
+k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
+          const T* __restrict__ psn, const T* __restrict__ pso,
+          T* __restrict__ out, double* __restrict__ part, int N, StencilCoef<T> c,
+          const __grid_constant__ GroupArgs<GRP> ga, int bps) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    int bx = blockIdx.x, gx = gridDim.x;
+    if constexpr (GRP) {          // grouped launch (FP32)
+        static_assert(std::is_same<T, float>::value, "grouped launches are FP32");
+        const int sim = blockIdx.x / bps;
+        bx = blockIdx.x - sim * bps;
+        gx = bps;
+        const BatchArgs& A = ga.a[sim];
+        phn = A.phn; pho = A.pho; psn = A.psn; pso = A.pso; out = A.bufA; part = A.part1; c = A.c;
+    }
+    stencil_tile<T, TX, TY, TYB>(smraw, phn, pho, psn, pso, out, part, N, c, bx, blockIdx.y, gx);
 }
 
 template <typename T> __host__ __device__ constexpr size_t stencil_smem_bytes() {
