@@ -18,10 +18,13 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libccmsav.so")
 LIB_BOUNDS = os.path.join(HERE, "libccmsav_bounds.so")   # index-checked build (-DCCMSAV_BOUNDS), for tests
+LINES = (32, 64, 128, 256, 512, 1024, 2048, 4096)   # line lengths N / 2 with kernels of their own
 # (source, extra flags, object)
 SOURCES = [(f, [], f.replace(".cu", ".o")) for f in ("ccmsav_api.cu", "sim_f32.cu", "sim_f64.cu", "ccmsav_noalloc.cu",
-                                                     "spectral_solve.cu", "fixed_ops.cu", "fixed_stencil.cu")]
-SOURCES += [("fixed_m.cu", [f"-DFIXED_M={m}"], f"fixed_m{m}.o") for m in (32, 64, 128, 256, 512, 1024, 2048, 4096)]
+                                                     "spectral_solve.cu", "fixed_ops.cu", "fixed_stencil.cu",
+                                                     "wide_ops.cu")]
+SOURCES += [("fixed_m.cu", [f"-DFIXED_M={m}"], f"fixed_m{m}.o") for m in LINES]
+SOURCES += [("wide_m.cu", [f"-DWIDE_M={m}"], f"wide_m{m}.o") for m in LINES]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

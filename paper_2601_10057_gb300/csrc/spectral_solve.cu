@@ -9,6 +9,7 @@
 #include "../../include/ccmsav.h"
 #include "spectral_kernels.cuh"
 #include "fixed_ops.h"
+#include "wide_ops.h"
 
 struct ccmsav_solver {
     int N = 0, bc = 0, precision = 0;
@@ -25,6 +26,10 @@ struct ccmsav_solver {
     size_t sm_fwd = 0, sm_col = 0, sm_inv = 0;
     const ccm::xf::Ops* xo = nullptr;   // FP64 Neumann / Dirichlet from N = 64 on: fixed-point line transforms
     ccm::xf::Tables xt;
+    const ccm::lf::Ops* lo = nullptr;   // FP32 Neumann / Dirichlet from N = 64 on: wide lines
+    ccm::lf::Tables lt;
+    const ccm::lf::Ops* lc = nullptr;   // FP32 periodic, N = 64 .. 4096: the column lines (length N), lo the rows
+    ccm::lf::Tables ltc;
     long long launches = 0;
 };
 
@@ -82,6 +87,17 @@ template <typename T> int setup(ccmsav_solver* s) {
             if (const int r = s->xo->setup(&rows)) return r;
             if (const int r = ccm::xf::make_tables(s->xo, s->xt, s->st)) return r;
         }
+    if constexpr (sizeof(T) == sizeof(float))
+        if (!per || ccm::lf::wide_ops(N)) {
+            if (!(s->lo = ccm::lf::wide_ops(N / 2))) return cudaStreamSynchronize(s->st) == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
+            if (const int r = s->lo->setup()) return r;
+            if (const int r = ccm::lf::make_tables(s->lo, s->lt, he.data(), 0.5 * s->smin, s->st)) return r;
+            if (per) {
+                s->lc = ccm::lf::wide_ops(N);
+                if (const int r = s->lc->setup()) return r;
+                if (const int r = ccm::lf::make_tables(s->lc, s->ltc, nullptr, 0.0, s->st)) return r;
+            }
+        }
     return cudaStreamSynchronize(s->st) == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
 }
 
@@ -91,6 +107,20 @@ template <typename T> int solve(ccmsav_solver* s, const double c[3], const T* f,
         if (s->xo) {
             s->xo->solve(f, u, static_cast<double*>(s->scratch), s->xt, s->ev, c, nullptr, nullptr, 1,
                          s->bc == CCMSAV_BC_DIRICHLET, s->st);
+            s->launches += 3;
+            return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
+        }
+    if constexpr (sizeof(T) == sizeof(float))
+        if (s->lc && ccm::lf::solve_ok(s->lt, c)) {
+            float2* a = static_cast<float2*>(s->scratch);      // N^2 complex values: the half spectrum twice
+            float2* b = a + (size_t)N * (N / 2);
+            s->lo->prow_fwd(f, a, s->lt, s->st);
+            s->lc->pcol(a, b, s->ltc, s->lt, c, s->st);
+            s->lo->prow_inv(b, u, s->lt, s->st);
+            s->launches += 3;
+            return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
+        } else if (s->lo && !s->lc && ccm::lf::solve_ok(s->lt, c)) {
+            s->lo->solve(f, u, static_cast<float*>(s->scratch), s->lt, c, nullptr, nullptr, 1, s->bc == CCMSAV_BC_DIRICHLET, s->st);
             s->launches += 3;
             return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
         }
@@ -141,6 +171,8 @@ void release(ccmsav_solver* s) {
     if (s->st) cudaStreamSynchronize(s->st);
     cudaFree(s->scratch); cudaFree(s->rhs); cudaFree(s->tw); cudaFree(s->twP); cudaFree(s->ev);
     ccm::xf::free_tables(s->xt);
+    ccm::lf::free_tables(s->lt);
+    ccm::lf::free_tables(s->ltc);
     if (s->own_stream && s->st) cudaStreamDestroy(s->st);
     delete s;
 }
