@@ -30,7 +30,8 @@
 // FP64's own rounding (to_double).
 //
 // Line layout: M = A C D complex values on G = M / A lanes, A = 16 per lane
-// (8 for the shortest lines): an A-point DFT in registers, twiddle, then on
+// (8 and 4 on short lines, whose grids leave most of the chip idle: there a
+// lane's own chain of instructions is the kernel's time): an A-point DFT in registers, twiddle, then on
 // each row of B = C D values a C-point and a D-point DFT, exchanged through the
 // line's shared-memory buffer (D = 1: one exchange).  Sixteen values are 64
 // registers of data, so sixteen warps fit an SM; with 32 (two exchanges fewer)
@@ -150,10 +151,10 @@ template <bool INV, int OFF> struct DIFX<1, INV, OFF> { static __device__ __forc
 
 // ------------------------------------------------------------------ line shapes
 template <int M> struct Shape;
-template <> struct Shape<32>   { static constexpr int A = 8,  C = 4,  D = 1;  };
-template <> struct Shape<64>   { static constexpr int A = 8,  C = 8,  D = 1;  };
-template <> struct Shape<128>  { static constexpr int A = 16, C = 8,  D = 1;  };
-template <> struct Shape<256>  { static constexpr int A = 16, C = 16, D = 1;  };
+template <> struct Shape<32>   { static constexpr int A = 4,  C = 4,  D = 2;  };
+template <> struct Shape<64>   { static constexpr int A = 4,  C = 4,  D = 4;  };
+template <> struct Shape<128>  { static constexpr int A = 8,  C = 4,  D = 4;  };
+template <> struct Shape<256>  { static constexpr int A = 8,  C = 4,  D = 8;  };
 template <> struct Shape<512>  { static constexpr int A = 16, C = 4,  D = 8;  };
 template <> struct Shape<1024> { static constexpr int A = 16, C = 8,  D = 8;  };
 template <> struct Shape<2048> { static constexpr int A = 16, C = 16, D = 8;  };
@@ -173,7 +174,7 @@ template <int M> struct Geo {
     static constexpr int P = B + 1;
     static constexpr int BUF = ((A * P + 7) / 8) * 8 + 1;
     static constexpr size_t SMEM = (size_t)LINES * BUF * sizeof(cx);
-    static constexpr int MINB = THREADS <= 128 ? 3 : THREADS <= 256 ? 2 : 1;   // at most 128 registers from 256 threads on
+    static constexpr int MINB = 512 / THREADS > 4 ? 4 : 512 / THREADS;       // at most 128 registers
     static_assert(THREADS % 32 == 0, "whole warps");
 };
 
