@@ -203,8 +203,12 @@ public:
                                                                          ga, brt);
         kw_coldct_gram<MM, true><<<bcol * n, kWarps * 32, wsm_col, s>>>(nullptr, nullptr, nullptr, nullptr, wf::PairTwTab{},
                                                                        nullptr, nullptr, SpecCoefF{}, ga, bcol);
-        k_solve<float2, true><<<kSolveBlocks * n, kSolveThreads, 0, s>>>(nullptr, 0, nullptr, 0, nullptr, nullptr,
-                                                                         SolveCoef{}, ga, kSolveBlocks);
+        if (nb1 + bcol <= kSolveOneRows)
+            k_solve<float2, true, kSolveOneThreads><<<n, kSolveOneThreads, 0, s>>>(nullptr, 0, nullptr, 0, nullptr, nullptr,
+                                                                                   SolveCoef{}, ga, 1);
+        else
+            k_solve<float2, true><<<kSolveBlocks * n, kSolveThreads, 0, s>>>(nullptr, 0, nullptr, 0, nullptr, nullptr,
+                                                                             SolveCoef{}, ga, kSolveBlocks);
         kw_comb_icolT<MM, true><<<bcomb * n, comb_warps<MM>() * 32, wsm_comb, s>>>(nullptr, nullptr, nullptr, wf::PairTwTab{},
                                                                         nullptr, nullptr, SpecCoefF{}, nullptr, 1, ga, bcomb);
         kw_irow<MM, true><<<birow * n, InvGeo<MM>::WARPS * 32, wsm_irow, s>>>(nullptr, nullptr, nullptr, nullptr,
@@ -1179,9 +1183,14 @@ public:
                 k_cl_inject<P><<<(so.nb2 + 255) / 256, 256, 0, st>>>(reinterpret_cast<P*>(part2), so.nb2, pcg);
                 ++nlaunch;
             }
-            k_solve<P><<<kSolveBlocks, kSolveThreads, 0, st>>>(reinterpret_cast<const P*>(part1), so.nb1,
-                                                               reinterpret_cast<const P*>(part2), so.nb2, part3, sc, so,
-                                                               GroupArgs<false>{}, 0);
+            if (so.nb1 + so.nb2 <= kSolveOneRows)
+                k_solve<P, false, kSolveOneThreads><<<1, kSolveOneThreads, 0, st>>>(
+                    reinterpret_cast<const P*>(part1), so.nb1, reinterpret_cast<const P*>(part2), so.nb2, part3, sc, so,
+                    GroupArgs<false>{}, 0);
+            else
+                k_solve<P><<<kSolveBlocks, kSolveThreads, 0, st>>>(reinterpret_cast<const P*>(part1), so.nb1,
+                                                                   reinterpret_cast<const P*>(part2), so.nb2, part3, sc, so,
+                                                                   GroupArgs<false>{}, 0);
         }
         mark(3);
         if (warp_path) {

@@ -817,7 +817,9 @@ k_coldct_gram(const T* __restrict__ in, T* __restrict__ spec, double* __restrict
 // (thread 0) the scalar algebra of Appendix B Steps 1 and 4.
 __device__ inline bool finite_(double x) { return isfinite(x); }
 
-// kSolveBlocks blocks of kSolveThreads.  FP64 instructions issue at a small
+// Up to kSolveOneRows partial rows: one block of kSolveOneThreads (its warps
+// share the rows; nothing to hand over between blocks).  More: kSolveBlocks
+// blocks of kSolveThreads.  FP64 instructions issue at a small
 // fraction of the FP32 rate on GB300 (about one warp instruction per 64-80
 // cycles per SM sub-partition, dependent or not), so this kernel is laid out
 // to execute few of them:
@@ -830,7 +832,8 @@ __device__ inline bool finite_(double x) { return isfinite(x); }
 //    of the augmented matrix per lane (Gauss-Jordan elimination with partial
 //    pivoting, pivots compared as integer magnitudes).
 // Every sum runs in a fixed order, so the result is deterministic.
-enum { NRQ = NRED1 + NRED2, kSolveThreads = 128, kSolveBlocks = 128, kSolveMinCol = 8 };
+enum { NRQ = NRED1 + NRED2, kSolveThreads = 128, kSolveBlocks = 128, kSolveMinCol = 8, kSolveOneThreads = 512,
+       kSolveOneRows = 1024 };
 static_assert(NRQ <= 32, "one column per lane");
 static_assert(kSolveBlocks == 32 * (kSolveThreads / 32), "32 slices per warp in the last block");
 
@@ -843,22 +846,44 @@ __device__ __forceinline__ double from_order_key(long long k) {
     return __longlong_as_double(k >= 0 ? k : k ^ 0x7fffffffffffffffLL);
 }
 
-// rows [b * per, min(n, (b + 1) * per)) of an n-row array belong to block b
-__device__ __forceinline__ void solve_slice(int n, int b, int& r0, int& cnt) {
-    const int per = (n + kSolveBlocks - 1) / kSolveBlocks;
+// 1/x and 1/sqrt(x) for positive normal x, error within two units in the last
+// place: hardware seed (20 bits or more) and one step of third order (e = 1 -
+// d r, r (1 + e + e^2); e = 1 - x y^2, y (1 + e/2 + 3 e^2/8)).  Three and five
+// dependent FP64 instructions instead of the library routines' longer chains.
+__device__ __forceinline__ double rcp_(double d) {
+    const unsigned h = (unsigned)__double2hiint(d) & 0x7fffffffu;
+    if (h - 0x02000000u >= 0x7b000000u) return 1.0 / d;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    double e = fma(-d, r, 1.0);
+    e = fma(e, e, e);
+    return fma(r, e, r);
+}
+__device__ __forceinline__ double rsqrt_(double x) {
+    if ((unsigned)__double2hiint(x) - 0x02000000u >= 0x7b000000u) return rsqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// rows [b * per, min(n, (b + 1) * per)) of an n-row array belong to slice b
+__device__ __forceinline__ void solve_slice(int n, int b, int nslices, int& r0, int& cnt) {
+    const int per = (n + nslices - 1) / nslices;
     r0 = min(n, b * per);
     cnt = min(n, r0 + per) - r0;
 }
 
-template <typename P, bool GRP = false>
-__global__ void __launch_bounds__(kSolveThreads)
+template <typename P, bool GRP = false, int NT = kSolveThreads>
+__global__ void __launch_bounds__(NT)
 k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
         double* __restrict__ slices, DevScalars* sc, SolveCoef co,
         const __grid_constant__ GroupArgs<GRP> ga, int bps) {
     constexpr int NR = NRQ;
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ double fin_[NR];
-    __shared__ double part[kSolveThreads / 32][NR];
+    constexpr bool ONE = NT == kSolveOneThreads;   // a single block per system
+    __shared__ double part[NT / 32][NR];
     __shared__ double s_state[10];       // V U W Z at n and n-1, conserved mean, steps
     __shared__ int s_status, is_last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -877,14 +902,14 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
         s_state[4] = sc->Vo; s_state[5] = sc->Uo; s_state[6] = sc->Wo; s_state[7] = sc->Zo;
         s_state[8] = sc->mass_mode; s_state[9] = sc->steps; s_status = sc->status;
     }
-    // this block's slice: lane c of warp 0 adds column c
-    if (warp == 0 && lane < NR) {
+    // this block's slice (ONE: this warp's): lane c adds column c
+    if ((ONE || warp == 0) && lane < NR) {
         const int c = lane;
         const bool in1 = c < NRED1;
         const P* col = in1 ? p1 + c : p2 + (c - NRED1);
         const int stride = in1 ? NRED1 : NRED2;
         int r0, cnt;
-        solve_slice(in1 ? nb1 : nb2, bx, r0, cnt);
+        solve_slice(in1 ? nb1 : nb2, ONE ? warp : bx, ONE ? NT / 32 : kSolveBlocks, r0, cnt);
         double acc = 0.0;
         long long kmin = 0x7fffffffffffffffLL;
         if constexpr (std::is_same<P, float2>::value) {
@@ -916,8 +941,11 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
                 }
             }
         }
-        slices[(size_t)bx * NR + c] = (c == kSolveMinCol) ? __longlong_as_double(kmin) : acc;
+        const double v = (c == kSolveMinCol) ? __longlong_as_double(kmin) : acc;
+        if constexpr (ONE) part[warp][c] = v;
+        else slices[(size_t)bx * NR + c] = v;
     }
+    if constexpr (!ONE) {
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) is_last = atomicAdd(&sc->solve_arrivals, 1u) == (unsigned)gx - 1;
@@ -941,6 +969,7 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
         part[warp][c] = (c == kSolveMinCol) ? __longlong_as_double(kmin) : (a4[0] + a4[1]) + (a4[2] + a4[3]);
     }
     if (threadIdx.x == 0) sc->solve_arrivals = 0u;
+    }
     __syncthreads();
     if (warp != 0) return;
     if (lane < NR) {
@@ -948,13 +977,13 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
         if (c == kSolveMinCol) {
             long long kmin = __double_as_longlong(part[0][c]);
 #pragma unroll
-            for (int w = 1; w < kSolveThreads / 32; ++w) kmin = min(kmin, __double_as_longlong(part[w][c]));
+            for (int w = 1; w < NT / 32; ++w) kmin = min(kmin, __double_as_longlong(part[w][c]));
             fin_[c] = from_order_key(kmin);
         } else {
-            double acc = part[0][c];
+            double a4[4] = {part[0][c], part[1][c], part[2][c], part[3][c]};
 #pragma unroll
-            for (int w = 1; w < kSolveThreads / 32; ++w) acc += part[w][c];
-            fin_[c] = acc;
+            for (int w = 4; w < NT / 32; ++w) a4[w & 3] += part[w][c];
+            fin_[c] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
         }
     }
     __syncwarp();
@@ -969,7 +998,7 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
     }
     const double h2 = co.h2;
     // normalisations 1/(2 sqrt I_V), 1/sqrt I_W, 1/sqrt I_Z (lanes 0, 1, 2)
-    const double rr = rsqrt(h2 * (lane == 0 ? IV : lane == 1 ? IW : IZ));
+    const double rr = rsqrt_(h2 * (lane == 0 ? IV : lane == 1 ? IW : IZ));
     const double nS = 0.5 * __shfl_sync(FULL, rr, 0), nQ = __shfl_sync(FULL, rr, 1), nK = __shfl_sync(FULL, rr, 2);
     // reference SAVs X_bar (Step 1 with the increments taken about phi_bar), lane q < 4
     constexpr double third = 1.0 / 3.0;
@@ -997,10 +1026,9 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
             const double nj = j < 4 ? nrm_of(j) : nK, cj = j < 4 ? cc_of(j) : co.cgo;
             a = (i == j ? 1.0 : 0.0) + cj * (h2 * ni * nj * G(i + 1, j < 4 ? j + 1 : 4));
         } else {
-            double bi = G(0, i + 1);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) bi -= w[q] * G(i + 1, q + 1);
-            a = h2 * ni * bi;
+            const double b0 = fma(-w[0], G(i + 1, 1), G(0, i + 1)), b1 = w[1] * G(i + 1, 2);
+            const double b2 = fma(-w[2], G(i + 1, 3), b0), b3 = fma(w[3], G(i + 1, 4), b1);
+            a = h2 * ni * (b2 - b3);
         }
     } else {
         const double PL = h2 * nK * nK * Gm[16];
@@ -1021,7 +1049,7 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
             return;
         }
         a = __shfl_sync(FULL, a, i == k ? 6 * piv + j : i == piv ? 6 * k + j : l);
-        const double rinv = 1.0 / __shfl_sync(FULL, a, 6 * k + k);
+        const double rinv = rcp_(__shfl_sync(FULL, a, 6 * k + k));
         const double akj = __shfl_sync(FULL, a, 6 * k + j) * rinv;
         const double aik = __shfl_sync(FULL, a, 6 * i + k);
         a = (i == k) ? akj : a - aik * akj;
