@@ -25,6 +25,8 @@
 #include "spectral_kernels.cuh"
 #include "classical_kernels.cuh"
 #include "fixed_ops.h"
+#include "wide_step.cuh"
+#include "wide_ops.h"
 #include <type_traits>
 #include <map>
 #include <mutex>
@@ -84,6 +86,8 @@ public:
     double* itau = nullptr;
     int xrows = 0;               // partial rows of the Gram sums
     int nb1x = 0;                // partial rows of the fixed-point stencil
+    lf::Tables lt;               // FP32 wide lines (inverse kernels)
+    lf::PairTab wide_inv() const { return lf::PairTab{lt.pi, lt.pib}; }
     int wRT = 8, wlds = 0, wRT4 = 4, wlds4 = 0, wKC = 1, wRI = 4;
     int ahead_rt = 0;   // L2 prefetch distance of the row kernel (0: none)
     size_t wsm_rt = 0, wsm_col = 0, wsm_comb = 0, wsm_irow = 0;
@@ -185,6 +189,7 @@ public:
             a.bufA = reinterpret_cast<float*>(bufA); a.bufB = reinterpret_cast<float*>(bufB);
             a.part1 = part1; a.part2 = part2; a.part3 = part3; a.sc = sc;
             a.tw2 = tw2; a.twF = pair_tab(twF); a.twI = pair_tab(twI); a.evf = evf; a.evp = evp;
+            a.tww = lt.tw; a.tiw = wide_inv();
             a.c = c;
             a.sf = SpecCoefF{(float)sp.C1, (float)sp.C2, (float)sp.C3, (float)sp.Ct, (float)sp.lam};
             a.so = so;
@@ -195,8 +200,7 @@ public:
     }
     int max_group() const override { return kMaxGroup; }
     template <int MM> void group_launch(const GroupArgs<true>& ga, int n, cudaStream_t s) {
-        const int bst = g_st.x, brt = N / wRT, bcol = N / wKC, bcomb = N / wRT4;
-        const int birow = (2 * N + InvGeo<MM>::LINES - 1) / InvGeo<MM>::LINES;
+        const int bst = g_st.x, brt = N / wRT, bcol = N / wKC;
         k_stencil<float, true><<<dim3(bst * n, g_st.y), b_st, stencil_smem_bytes<float>(), s>>>(
             nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, N, StencilCoef<float>{}, ga, bst);
         kw_rowdct_T<MM, true><<<dim3(brt * n, NF), kWarps * 32, wsm_rt, s>>>(nullptr, nullptr, nullptr, wf::PairTwTab{}, 0,
@@ -209,10 +213,11 @@ public:
         else
             k_solve<float2, true><<<kSolveBlocks * n, kSolveThreads, 0, s>>>(nullptr, 0, nullptr, 0, nullptr, nullptr,
                                                                              SolveCoef{}, ga, kSolveBlocks);
-        kw_comb_icolT<MM, true><<<bcomb * n, comb_warps<MM>() * 32, wsm_comb, s>>>(nullptr, nullptr, nullptr, wf::PairTwTab{},
-                                                                        nullptr, nullptr, SpecCoefF{}, nullptr, 1, ga, bcomb);
-        kw_irow<MM, true><<<birow * n, InvGeo<MM>::WARPS * 32, wsm_irow, s>>>(nullptr, nullptr, nullptr, nullptr,
-            wf::PairTwTab{}, nullptr, nullptr, nullptr, nullptr, 0, nullptr, 1, ga, birow);
+        const int blc = 2 * N / lf::Geo<MM>::LINES, blr = 2 * N / lf::RowGeo<MM>::LINES;
+        lf::kl_comb<MM, true><<<blc * n, lf::Geo<MM>::THREADS, lf::Geo<MM>::SMEM, s>>>(
+            nullptr, nullptr, nullptr, lf::PairTab{}, nullptr, nullptr, SpecCoefF{}, nullptr, 1, ga, blc);
+        lf::kl_irow<MM, true><<<blr * n, lf::RowGeo<MM>::THREADS, lf::RowGeo<MM>::SMEM, s>>>(
+            nullptr, nullptr, nullptr, nullptr, lf::PairTab{}, nullptr, nullptr, nullptr, nullptr, 0, nullptr, 1, ga, blr);
     }
     // recs: host records, three blocks of `stride` (one per step), of which
     // this group's n are at the start of each block; copied into the launch
@@ -322,6 +327,7 @@ public:
         if (tw2i && tw2i != tw2) cudaFree(tw2i);
         cudaFree(tw2); cudaFree(evf); cudaFree(evp); cudaFree(twF); cudaFree(twI);
         cudaFree(cl); cudaFree(pcg); cudaFree(cl_red);
+        lf::free_tables(lt);
         cudaFree(isig); cudaFree(itau); xf::free_tables(xt);
         isig = itau = nullptr;
         if (pcg_host) cudaFreeHost(pcg_host);
@@ -810,6 +816,12 @@ public:
                 set_smem_limit((const void*)kw_comb_icolT<MM, true>, wsm_comb, kCombCarveout) ||
                 set_smem_limit((const void*)kw_irow<MM, true>, wsm_irow))
                 return CCMSAV_ECUDA;
+        if (set_smem_limit((const void*)lf::kl_comb<MM>, lf::Geo<MM>::SMEM) || set_smem_limit((const void*)lf::kl_irow<MM>, lf::RowGeo<MM>::SMEM))
+            return CCMSAV_ECUDA;
+        if constexpr (WGeo<MM>::WPL == 1)
+            if (set_smem_limit((const void*)lf::kl_comb<MM, true>, lf::Geo<MM>::SMEM) ||
+                set_smem_limit((const void*)lf::kl_irow<MM, true>, lf::RowGeo<MM>::SMEM))
+                return CCMSAV_ECUDA;
         // L2 prefetch one residency ahead only where few CTAs fit per SM (one
         // at N = 4096); with three per SM (N <= 2048) it evicts rows before
         // their use and costs time (73.3 vs 71.5 us at N = 2048)
@@ -881,6 +893,9 @@ public:
         CCM_CUDA(cudaMemcpyAsync(twI, pi.data(), pi.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
         CCM_CUDA(cudaStreamSynchronize(st));
         int r = CCMSAV_EINVAL;
+        if (const lf::Ops* lo = lf::wide_ops(Mh)) {
+            if (const int e = lf::make_tables(lo, lt, nullptr, 0.0, st)) return e;
+        }
         if constexpr (std::is_same<T, float>::value)
         switch (M) {
             case 64: r = setup_warp<64>(); break;
@@ -924,14 +939,13 @@ public:
     template <int MM>
     void launch_warp_inverse(const SpecCoef& s, int anchor) {
         SpecCoefF sf{(float)s.C1, (float)s.C2, (float)s.C3, (float)s.Ct, (float)s.lam};
-        kw_comb_icolT<MM><<<N / wRT4, comb_warps<MM>() * 32, wsm_comb, st>>>(reinterpret_cast<const float*>(bufA),
-            reinterpret_cast<float*>(bufB), comb_shape<MM>() ? tw2i : tw2, pair_tab(twI), evf, evp, sf, sc, anchor,
+        lf::kl_comb<MM><<<2 * N / lf::Geo<MM>::LINES, lf::Geo<MM>::THREADS, lf::Geo<MM>::SMEM, st>>>(
+            reinterpret_cast<const float*>(bufA), reinterpret_cast<float*>(bufB), lt.tw, wide_inv(), evf, evp, sf, sc, anchor,
             GroupArgs<false>{}, 0);
         mark(4);
-        kw_irow<MM><<<(2 * N + InvGeo<MM>::LINES - 1) / InvGeo<MM>::LINES, InvGeo<MM>::WARPS * 32, wsm_irow, st>>>(
+        lf::kl_irow<MM><<<2 * N / lf::RowGeo<MM>::LINES, lf::RowGeo<MM>::THREADS, lf::RowGeo<MM>::SMEM, st>>>(
             reinterpret_cast<const float*>(bufB),
-            reinterpret_cast<float*>(phi[spare]), reinterpret_cast<float*>(psi[spare]), irow_shape<MM>() ? tw2i : tw2,
-            pair_tab(twI),
+            reinterpret_cast<float*>(phi[spare]), reinterpret_cast<float*>(psi[spare]), lt.tw, wide_inv(),
             reinterpret_cast<const float*>(phi[cur]), reinterpret_cast<const float*>(phi[prev]),
             reinterpret_cast<const float*>(psi[cur]), reinterpret_cast<const float*>(psi[prev]),
             bdf1_launch, sc, anchor, GroupArgs<false>{}, 0);

@@ -46,6 +46,7 @@
 #include <type_traits>
 #include "dct_device.cuh"
 #include "warp_fft.cuh"
+#include "wide_fft.cuh"
 #include "bounds.cuh"
 
 namespace ccm {
@@ -120,13 +121,14 @@ struct BatchArgs {
     DevScalars* sc;
     const cplx<float>* tw2;                                                   // four-step twiddles
     wf::PairTwTab twF, twI;                                                   // DCT pair twiddles
+    const float2* tww; lf::PairTab tiw;                                       // wide lines: twiddles, inverse pairs
     const float* evf; const float4* evp;                                      // FP32 eigenvalues
     StencilCoef<float> c;
     SpecCoefF sf;
     SolveCoef so;
 };
 
-// Simulations per grouped launch: 64 records of 328 bytes stay well inside
+// Simulations per grouped launch: 64 records of 352 bytes stay well inside
 // the 32764 bytes of kernel parameters.
 constexpr int kMaxGroup = 64;
 template <bool GRP> struct GroupArgs { int unused = 0; };

@@ -1,0 +1,202 @@
+// wide_step.cuh -- the FP32 step's inverse kernels on the lines of
+// wide_fft.cuh: recovery + inverse columns and inverse rows (N = 128 .. 8192).
+//
+// Both wait on memory, and on warp-level lines (32 or 64 values per lane, 72 -
+// 128 registers) they held 16 - 24 warps per SM; with sixteen values per lane
+// 32 warps fit.  The recovery kernel takes one field per CTA (the phi CTAs,
+// five spectra, come first, the lighter psi CTAs fill the tail).
+#pragma once
+#include "warp_kernels.cuh"
+#include "wide_fft.cuh"
+
+namespace ccm {
+namespace lf {
+
+// LINES spectral rows of one field: recovery combination and divide, inverse
+// DCT along y, transposed write out[f][y][kx].  Block b: field b / (N / LINES).
+template <int M, bool GRP = false>
+__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
+kl_comb(const float* __restrict__ spec, float* __restrict__ out, const float2* __restrict__ tw, PairTab ti,
+        const float* __restrict__ evf, const float4* __restrict__ evp, SpecCoefF sc, DevScalars* __restrict__ dsc,
+        int anchor_mass, const __grid_constant__ GroupArgs<GRP> ga, int bps) {
+    using Gm = Geo<M>;
+    constexpr int N = Gm::N, E = Gm::E, G = Gm::G, NB = N / Gm::LINES;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    cf* bufs = reinterpret_cast<cf*>(smraw);
+    const size_t NN = (size_t)N * N;
+    int bx = blockIdx.x;
+    if constexpr (GRP) {          // grouped launch
+        const int sim = blockIdx.x / bps;
+        bx = blockIdx.x - sim * bps;
+        const BatchArgs& A = ga.a[sim];
+        spec = A.bufA; out = A.bufB; tw = A.tww; ti = A.tiw; evf = A.evf; evp = A.evp; sc = A.sf; dsc = A.sc;
+    }
+    int n2, slot;
+    lane_of<M>(n2, slot);
+    const int f = bx / NB, x0 = (bx % NB) * Gm::LINES, kx = x0 + slot;
+    cf* buf = bufs + (size_t)slot * Gm::BUF;
+    const float evx = __ldg(evf + kx);
+    const size_t base = CCM_IXW((size_t)kx * SpecRow<M>::KS, SpecRow<M>::KS, (size_t)N * SpecRow<M>::KS);
+    constexpr size_t FS = SpecRow<M>::FO;
+    auto put = [&](int k, const Quad<float>& X) {
+        cf zk, zMk;
+        wf::pre_pair_lean(X, ld_pair(ti, k), zk, zMk);
+        buf[k] = zk;
+        if (k > 0) buf[M - k] = zMk;
+    };
+    if (f == 0) {
+        const float aS = (float)dsc->alpha[0], aH = (float)dsc->alpha[1], aQ = (float)dsc->alpha[2], aK = (float)dsc->alpha[3];
+#pragma unroll 2
+        for (int k = n2; k <= M / 2; k += G) {
+            const float4 e4 = __ldg(evp + k);
+            const float* src = spec + base + 4 * k;
+            const float4 f0 = __ldg(reinterpret_cast<const float4*>(src));
+            const float4 f1 = __ldg(reinterpret_cast<const float4*>(src + FS));
+            const float4 f2 = __ldg(reinterpret_cast<const float4*>(src + 2 * FS));
+            const float4 f3 = __ldg(reinterpret_cast<const float4*>(src + 3 * FS));
+            const float4 f4 = __ldg(reinterpret_cast<const float4*>(src + 4 * FS));
+            auto comb = [&](float a0, float a1, float a2, float a3, float a4, float ev) {
+                const float s = evx + ev;
+                return (a0 - aS * a1 - aH * a2 - aQ * a3 - aK * a4) * __frcp_rn(sc.C1 + s * (sc.C2 + sc.C3 * s));
+            };
+            put(k, Quad<float>{comb(f0.x, f1.x, f2.x, f3.x, f4.x, e4.x), comb(f0.y, f1.y, f2.y, f3.y, f4.y, e4.y),
+                               comb(f0.z, f1.z, f2.z, f3.z, f4.z, e4.z), comb(f0.w, f1.w, f2.w, f3.w, f4.w, e4.w)});
+        }
+    } else {
+        const float aL = (float)dsc->alpha[4];
+#pragma unroll 4
+        for (int k = n2; k <= M / 2; k += G) {
+            const float4 e4 = __ldg(evp + k);
+            const float* src = spec + base + 4 * k;
+            const float4 f6 = __ldg(reinterpret_cast<const float4*>(src + 5 * FS));
+            const float4 f7 = __ldg(reinterpret_cast<const float4*>(src + 6 * FS));
+            auto comb = [&](float a6, float a7, float ev) {
+                return (a6 + aL * a7) * __frcp_rn(sc.Ct + sc.lam * (evx + ev));
+            };
+            Quad<float> X{comb(f6.x, f7.x, e4.x), comb(f6.y, f7.y, e4.y), comb(f6.z, f7.z, e4.z), comb(f6.w, f7.w, e4.w)};
+            // d_psi has zero mean (mass conservation); the zero mode is set exactly and the stored mean kept with the anchor
+            if (anchor_mass && kx == 0 && k == 0) X.xk = 0.f;
+            put(k, X);
+        }
+    }
+    sync_line<M>(slot);
+    inverse_line<M>(buf, tw, n2, slot);
+    if (anchor_mass && f == 1 && x0 == 0) {
+        // the zero-mean psi increment's kx = 0 column should sum to 0 over y; record what the
+        // FP32 transform left (removed in the inverse row kernel).  Every line of the block takes part in the sum.
+        __shared__ float2 lsum[Gm::LINES * (G > 32 ? G / 32 : 1)];
+        float dhi = 0.f, dlo = 0.f;
+#pragma unroll 1
+        for (int m = n2; m < M / 2; m += G) {
+            const cf a = buf[m], b = buf[M - 1 - m];
+            df_add(dhi, dlo, a.x); df_add(dhi, dlo, b.y); df_add(dhi, dlo, a.y); df_add(dhi, dlo, b.x);
+        }
+        const double dsum = line_sum_exact<G>(dhi, dlo, slot, lsum);
+        if (slot == 0 && n2 == 0) dsc->dc_col = dsum;
+    }
+    __syncthreads();
+    write_samples<M, Gm::LINES>(bufs, out + f * NN + x0);
+}
+
+// Rows per CTA of the inverse row kernel: four (the lines are independent;
+// smaller CTAs leave less of a last wave idle), two at M = 4096.
+template <int M> struct RowGeo {
+    static constexpr int G = Geo<M>::G;
+    static constexpr int LINES = M == 4096 ? 2 : G < 8 ? 8 : 4;
+    static constexpr int THREADS = LINES * G;
+    static constexpr size_t SMEM = (size_t)LINES * Geo<M>::BUF * sizeof(cf);
+    static constexpr int MINB = 1024 / THREADS > 16 ? 16 : 1024 / THREADS;
+    static_assert(THREADS % 32 == 0, "whole warps");
+};
+
+// Inverse DCT along x of LINES rows of one field and u^{n+1} = u_bar + du with
+// the compensated (and, for psi, error-feedback and mass-anchored) final
+// rounding of kw_irow.  Block b: field b / (N / LINES).
+template <int M, bool GRP = false>
+__global__ void __launch_bounds__(RowGeo<M>::THREADS, RowGeo<M>::MINB)
+kl_irow(const float* __restrict__ in, float* __restrict__ phi_new, float* __restrict__ psi_new,
+        const float2* __restrict__ tw, PairTab ti, const float* __restrict__ phn, const float* __restrict__ pho,
+        const float* __restrict__ psn, const float* __restrict__ pso, int bdf1, const DevScalars* __restrict__ dsc,
+        int anchor_mass, const __grid_constant__ GroupArgs<GRP> ga, int bps) {
+    using Gm = Geo<M>;
+    constexpr int N = Gm::N, E = Gm::E, G = Gm::G, L = RowGeo<M>::LINES, NB = N / L;
+    int bx = blockIdx.x;
+    if constexpr (GRP) {          // grouped launch
+        const int sim = blockIdx.x / bps;
+        bx = blockIdx.x - sim * bps;
+        const BatchArgs& A = ga.a[sim];
+        in = A.bufB; phi_new = A.phi_new; psi_new = A.psi_new; tw = A.tww; ti = A.tiw;
+        phn = A.phn; pho = A.pho; psn = A.psn; pso = A.pso; dsc = A.sc;
+    }
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ float2 lsum[L * (G > 32 ? G / 32 : 1)];
+    int n2, slot;
+    lane_of<M>(n2, slot);
+    cf* buf = reinterpret_cast<cf*>(smraw) + (size_t)slot * Gm::BUF;
+    const size_t NN = (size_t)N * N;
+    const int fld = bx / NB, y = (bx % NB) * L + slot;
+    const float* row = in + CCM_IXW(fld * NN + (size_t)y * N, N, 2 * NN);
+    const float x0 = __ldg(row);                          // the row's DC coefficient
+#pragma unroll 4
+    for (int k = n2; k <= M / 2; k += G) {
+        const Quad<float> X{__ldg(row + k), k > 0 ? __ldg(row + N - k) : 0.f, __ldg(row + M - k), __ldg(row + M + k)};
+        cf zk, zMk;
+        wf::pre_pair_lean(X, ld_pair(ti, k), zk, zMk);
+        buf[k] = zk;
+        if (k > 0) buf[M - k] = zMk;
+    }
+    sync_line<M>(slot);
+    inverse_line<M>(buf, tw, n2, slot);
+    const size_t roff = (size_t)y * N;
+    const float4* un = reinterpret_cast<const float4*>((fld == 0 ? phn : psn) + roff);
+    const float4* uo = reinterpret_cast<const float4*>((fld == 0 ? pho : pso) + roff);
+    float* dst = (fld == 0 ? phi_new : psi_new) + roff;
+    const bool b1 = bdf1 != 0;
+    if (fld == 0 || !anchor_mass) {                       // uniform over the CTA
+#pragma unroll 4
+        for (int j = 0; j < E / 2; ++j) {
+            const int m = n2 + G * j;
+            if (!CCM_OKW(roff + 4 * m, 4, NN)) continue;
+            const cf a = buf[m], b = buf[M - 1 - m];
+            const float4 p = __ldg(un + m), q = __ldg(uo + m);
+            *reinterpret_cast<float4*>(dst + 4 * m) =
+                make_float4(bar_add(p.x, q.x, a.x, 0.f, b1), bar_add(p.y, q.y, b.y, 0.f, b1),
+                            bar_add(p.z, q.z, a.y, 0.f, b1), bar_add(p.w, q.w, b.x, 0.f, b1));
+        }
+        return;
+    }
+    // psi: the row's increments should sum to sqrt(N) x0; the residual of the FP32 transform and the column residual
+    // dc_col are removed, with the mean anchor, in the final rounding (error feedback along each lane's values, the
+    // lanes' remaining errors folded into the row's first value with one dithered rounding: kw_irow)
+    const uint32_t step = (uint32_t)dsc->steps;           // dither key (graph replays read it here)
+    float rhi = 0.f, rlo = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < E / 2; ++j) {
+        const int m = n2 + G * j;
+        const cf a = buf[m], b = buf[M - 1 - m];
+        df_add(rhi, rlo, a.x); df_add(rhi, rlo, b.y); df_add(rhi, rlo, a.y); df_add(rhi, rlo, b.x);
+    }
+    const double rsum = line_sum_exact<G>(rhi, rlo, slot, lsum);
+    const double sN = sqrt((double)N);
+    const float an = (float)(dsc->anchor - sN * dsc->dc_col / ((double)N * N) + (sN * (double)x0 - rsum) / (double)N);
+    float carry = 0.f, first = 0.f;
+#pragma unroll 4
+    for (int j = 0; j < E / 2; ++j) {
+        const int m = n2 + G * j;
+        if (!CCM_OKW(roff + 4 * m, 4, NN)) continue;
+        const cf a = buf[m], b = buf[M - 1 - m];
+        const float4 p = __ldg(un + m), q = __ldg(uo + m);
+        float4 o;
+        o.x = bar_add_fb(p.x, q.x, a.x, an, b1, carry);
+        o.y = bar_add_fb(p.y, q.y, b.y, an, b1, carry);
+        o.z = bar_add_fb(p.z, q.z, a.y, an, b1, carry);
+        o.w = bar_add_fb(p.w, q.w, b.x, an, b1, carry);
+        if (j == 0) first = o.x;
+        *reinterpret_cast<float4*>(dst + 4 * m) = o;
+    }
+    const double rest = line_sum_exact<G>(carry, 0.f, slot, lsum);
+    if (n2 == 0) dst[0] = dither_round(first, (float)rest, dither_key(step, (uint32_t)roff) | 1u);
+}
+
+}  // namespace lf
+}  // namespace ccm
