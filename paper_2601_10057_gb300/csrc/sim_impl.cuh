@@ -71,13 +71,11 @@ public:
     // FP32 warp-FFT path (N = 128 .. 2048): twiddle matrix W_M^{n2 k1} and FP32 eigenvalues
     bool warp_path = false;
     cplx<float>* tw2 = nullptr;
-    cplx<float>* tw2i = nullptr;   // table of the inverse kernels' variant line shape (or tw2)
     float* evf = nullptr;
     float4* evp = nullptr;   // eigenvalues in the pair order of the warp-path spectra
-    float4* twF = nullptr;       // forward / inverse pair twiddles of the warp path
-    float4* twI = nullptr;       // (wn, a) per pair; b of pair 0 in twF0 / twI0
-    float2 twF0{}, twI0{};
-    wf::PairTwTab pair_tab(const float4* t) const { return wf::PairTwTab{t, t == twF ? twF0 : twI0}; }
+    float4* twF = nullptr;       // forward pair twiddles of the warp path: (wn, a) per pair; b of pair 0 in twF0
+    float2 twF0{};
+    wf::PairTwTab pair_tab() const { return wf::PairTwTab{twF, twF0}; }
     // FP64 path (N >= 64): the fixed-point line transforms and 1/sigma, 1/tau of
     // the handle's time step in the order of their spectra
     const xf::Ops* xo = nullptr;
@@ -86,11 +84,12 @@ public:
     double* itau = nullptr;
     int xrows = 0;               // partial rows of the Gram sums
     int nb1x = 0;                // partial rows of the fixed-point stencil
-    lf::Tables lt;               // FP32 wide lines (inverse kernels)
+    lf::Tables lt;               // FP32 wide lines (the inverse kernels; every pass of N = 8192)
+    lf::PairTab wide_fwd() const { return lf::PairTab{lt.pf, lt.pfb}; }
     lf::PairTab wide_inv() const { return lf::PairTab{lt.pi, lt.pib}; }
-    int wRT = 8, wlds = 0, wRT4 = 4, wlds4 = 0, wKC = 1, wRI = 4;
+    int wRT = 8, wKC = 1;
     int ahead_rt = 0;   // L2 prefetch distance of the row kernel (0: none)
-    size_t wsm_rt = 0, wsm_col = 0, wsm_comb = 0, wsm_irow = 0;
+    size_t wsm_rt = 0, wsm_col = 0;
     DevScalars* sc_host = nullptr;   // pinned
     double* h_part = nullptr;        // pinned, diag partial rows
     void* tmp64 = nullptr;           // FP64 staging for host I/O
@@ -188,8 +187,8 @@ public:
             a.phi_new = phi[s0]; a.psi_new = psi[s0];
             a.bufA = reinterpret_cast<float*>(bufA); a.bufB = reinterpret_cast<float*>(bufB);
             a.part1 = part1; a.part2 = part2; a.part3 = part3; a.sc = sc;
-            a.tw2 = tw2; a.twF = pair_tab(twF); a.twI = pair_tab(twI); a.evf = evf; a.evp = evp;
-            a.tww = lt.tw; a.tiw = wide_inv();
+            a.tw2 = tw2; a.twF = pair_tab(); a.evf = evf; a.evp = evp;
+            a.tww = lt.tw; a.tfw = wide_fwd(); a.tiw = wide_inv();
             a.c = c;
             a.sf = SpecCoefF{(float)sp.C1, (float)sp.C2, (float)sp.C3, (float)sp.Ct, (float)sp.lam};
             a.so = so;
@@ -324,15 +323,14 @@ public:
         for (int i = 0; i < 3; ++i) { cudaFree(phi[i]); cudaFree(psi[i]); phi[i] = psi[i] = nullptr; }
         cudaFree(bufA); cudaFree(bufB); cudaFree(part1); cudaFree(part2); cudaFree(partd); cudaFree(part3);
         cudaFree(twM); cudaFree(twP); cudaFree(ev); cudaFree(sc); cudaFree(tmp64);
-        if (tw2i && tw2i != tw2) cudaFree(tw2i);
-        cudaFree(tw2); cudaFree(evf); cudaFree(evp); cudaFree(twF); cudaFree(twI);
+        cudaFree(tw2); cudaFree(evf); cudaFree(evp); cudaFree(twF);
         cudaFree(cl); cudaFree(pcg); cudaFree(cl_red);
         lf::free_tables(lt);
         cudaFree(isig); cudaFree(itau); xf::free_tables(xt);
         isig = itau = nullptr;
         if (pcg_host) cudaFreeHost(pcg_host);
         cl = nullptr; pcg = nullptr; cl_red = nullptr; pcg_host = nullptr;
-        tw2 = nullptr; tw2i = nullptr; evf = nullptr; evp = nullptr; twF = nullptr; twI = nullptr;
+        tw2 = nullptr; evf = nullptr; evp = nullptr; twF = nullptr;
         if (sc_host) cudaFreeHost(sc_host);
         if (h_part) cudaFreeHost(h_part);
         if (h_up) cudaFreeHost(h_up);
@@ -579,19 +577,13 @@ public:
     }
 
     // ---- autotuner --------------------------------------------------------
-    template <int MM> static const void* coldct_fn() {
-        if constexpr (WGeo<MM>::WPL > 1) return (const void*)kw_coldct_gram_split<MM>;
-        else return (const void*)kw_coldct_gram<MM>;
-    }
     template <int MM> int apply_carveout_M(int c) {
         if (cudaFuncSetAttribute((const void*)kw_rowdct_T<MM>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-            cudaFuncSetAttribute(coldct_fn<MM>(), cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-            cudaFuncSetAttribute((const void*)kw_comb_icolT<MM>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess)
+            cudaFuncSetAttribute((const void*)kw_coldct_gram<MM>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess)
             return CCMSAV_ECUDA;
-        if constexpr (WGeo<MM>::WPL == 1)
+        if constexpr (MM <= 1024)
             if (cudaFuncSetAttribute((const void*)kw_rowdct_T<MM, true>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-                cudaFuncSetAttribute((const void*)kw_coldct_gram<MM, true>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-                cudaFuncSetAttribute((const void*)kw_comb_icolT<MM, true>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess)
+                cudaFuncSetAttribute((const void*)kw_coldct_gram<MM, true>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess)
                 return CCMSAV_ECUDA;
         return CCMSAV_OK;
     }
@@ -604,7 +596,6 @@ public:
                 case 512: return apply_carveout_M<512>(c);
                 case 1024: return apply_carveout_M<1024>(c);
                 case 2048: return apply_carveout_M<2048>(c);
-                case 4096: return apply_carveout_M<4096>(c);
             }
         }
         return CCMSAV_OK;
@@ -768,12 +759,10 @@ public:
 
     // Shared-memory share (percent of 228 KB) of the 8-line transform kernels;
     // the driver rounds it up to a supported size: 72 % -> 196 KB, three of
-    // the forward kernels' 65 KB CTAs (swizzled line buffers) or two of the
-    // recovery kernel's 68 KB ones at N = 2048, and 60 KB of L1 for the
+    // the forward kernels' 65 KB CTAs (swizzled line buffers) at N = 2048, and 60 KB of L1 for the
     // twiddle and eigenvalue tables (the full 228 KB leaves 28 KB).
     static constexpr int kRowCarveout = 72;
     static constexpr int kColCarveout = 72;
-    static constexpr int kCombCarveout = 72;
     // four-step twiddle table W_M^{n2 k1} of an E x G line shape, entry k1 G + n2
     int make_tw2(int MM, int E, int G, cplx<float>** out) {
         std::vector<cplx<float>> h2((size_t)MM);
@@ -788,44 +777,30 @@ public:
         return CCMSAV_OK;
     }
     template <int MM> int setup_warp() {
-        using Gm = WGeo<MM>;
-        using Gc = WGeo<MM, comb_shape<MM>(), comb_warps<MM>()>;   // the recovery kernel's geometry
-        using Gv = WGeo<MM, 1>;                     // the variant of the inverse kernels
-        if (int r = make_tw2(MM, Gm::E, Gm::G, &tw2)) return r;
-        if constexpr (comb_shape<MM>() != 0 || irow_shape<MM>() != 0) {
-            if (int r = make_tw2(MM, Gv::E, Gv::G, &tw2i)) return r;
-        } else {
-            tw2i = tw2;
-        }
-        const size_t bb = Gm::buf_bytes();
-        wRT = Gm::SLOTS; wsm_rt = bb;
-        wKC = Gm::SLOTS / NF; wsm_col = bb;
-        if constexpr (Gm::WPL > 1) {     // two-warp lines: column pass split into the two field groups, one column per CTA
-            wKC = 1;
-            wsm_col = (size_t)5 * Gm::BUF * sizeof(cplx<float>);
-        }
-        wRT4 = Gc::SLOTS / 2; wsm_comb = Gc::bufp_bytes();
-        wsm_irow = InvGeo<MM>::smem_bytes();
-        if (set_smem_limit((const void*)kw_rowdct_T<MM>, wsm_rt, kRowCarveout) || set_smem_limit(coldct_fn<MM>(), wsm_col, kColCarveout) ||
-            set_smem_limit((const void*)kw_comb_icolT<MM>, wsm_comb, kCombCarveout) || set_smem_limit((const void*)kw_irow<MM>, wsm_irow))
-            return CCMSAV_ECUDA;
-        // the grouped-launch instantiations (one warp or less per line)
-        if constexpr (WGeo<MM>::WPL == 1)
-            if (set_smem_limit((const void*)kw_rowdct_T<MM, true>, wsm_rt, kRowCarveout) ||
-                set_smem_limit((const void*)kw_coldct_gram<MM, true>, wsm_col, kColCarveout) ||
-                set_smem_limit((const void*)kw_comb_icolT<MM, true>, wsm_comb, kCombCarveout) ||
-                set_smem_limit((const void*)kw_irow<MM, true>, wsm_irow))
-                return CCMSAV_ECUDA;
         if (set_smem_limit((const void*)lf::kl_comb<MM>, lf::Geo<MM>::SMEM) || set_smem_limit((const void*)lf::kl_irow<MM>, lf::RowGeo<MM>::SMEM))
             return CCMSAV_ECUDA;
-        if constexpr (WGeo<MM>::WPL == 1)
+        if constexpr (MM <= 1024)        // the grouped-launch instantiations
             if (set_smem_limit((const void*)lf::kl_comb<MM, true>, lf::Geo<MM>::SMEM) ||
                 set_smem_limit((const void*)lf::kl_irow<MM, true>, lf::RowGeo<MM>::SMEM))
                 return CCMSAV_ECUDA;
-        // L2 prefetch one residency ahead only where few CTAs fit per SM (one
-        // at N = 4096); with three per SM (N <= 2048) it evicts rows before
-        // their use and costs time (73.3 vs 71.5 us at N = 2048)
-        {
+        if constexpr (MM == 4096) {      // forward passes on wide lines as well
+            wKC = 1;
+            if (set_smem_limit((const void*)lf::kl_row<MM>, lf::FwdGeo<MM>::SMEM) || set_smem_limit((const void*)lf::kl_col<MM>, lf::ColGeo<MM>::SMEM))
+                return CCMSAV_ECUDA;
+        } else {
+            using Gm = WGeo<MM>;
+            if (int r = make_tw2(MM, Gm::E, Gm::G, &tw2)) return r;
+            wRT = Gm::SLOTS; wKC = Gm::SLOTS / NF;
+            wsm_rt = wsm_col = Gm::buf_bytes();
+            if (set_smem_limit((const void*)kw_rowdct_T<MM>, wsm_rt, kRowCarveout) || set_smem_limit((const void*)kw_coldct_gram<MM>, wsm_col, kColCarveout))
+                return CCMSAV_ECUDA;
+            if constexpr (MM <= 1024)
+                if (set_smem_limit((const void*)kw_rowdct_T<MM, true>, wsm_rt, kRowCarveout) ||
+                    set_smem_limit((const void*)kw_coldct_gram<MM, true>, wsm_col, kColCarveout))
+                    return CCMSAV_ECUDA;
+            // L2 prefetch one residency ahead only where few CTAs fit per SM (one
+            // at N = 4096); with three per SM (N <= 2048) it evicts rows before
+            // their use and costs time (73.3 vs 71.5 us at N = 2048)
             int dev = 0, nsm = 0;
             if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
                 return CCMSAV_ECUDA;
@@ -846,7 +821,7 @@ public:
 
     int init_warp_path() {
         std::vector<float> he(N), hp;
-        std::vector<wf::PairTw> hf, hi;
+        std::vector<wf::PairTw> hf;
         const double hh = p.L / N;
         for (int k = 0; k < N; ++k) { const double s = std::sin(M_PI * k / (2.0 * N)); he[k] = (float)(4.0 * s * s / (hh * hh)); }
         if (cudaMalloc(&evf, N * sizeof(float)) != cudaSuccess) return CCMSAV_ENOMEM;
@@ -864,33 +839,23 @@ public:
         CCM_CUDA(cudaMemcpyAsync(evp, hp.data(), hp.size() * sizeof(float), cudaMemcpyHostToDevice, st));
         // pair twiddles (FP64 closed forms, see wf::PairTw)
         hf.assign(Mh / 2 + 1, wf::PairTw{});
-        hi.assign(Mh / 2 + 1, wf::PairTw{});
         const double c0 = std::sqrt(1.0 / N), c1 = std::sqrt(2.0 / N);
-        const double s0 = 1.0 / (Mh * c0), s1 = 1.0 / (Mh * c1);
         for (int k = 0; k <= Mh / 2; ++k) {
             const double a = 2.0 * M_PI * k / N, th = M_PI * k / (2.0 * N), q = M_PI / 4.0;
-            const double ck = k == 0 ? c0 : c1, sk = k == 0 ? s0 : s1;
-            wf::PairTw f{}, v{};
-            f.wnx = v.wnx = (float)std::cos(a);
-            f.wny = v.wny = (float)(-std::sin(a));
+            const double ck = k == 0 ? c0 : c1;
+            wf::PairTw f{};
+            f.wnx = (float)std::cos(a);
+            f.wny = (float)(-std::sin(a));
             f.ax = (float)(0.5 * ck * std::cos(th)); f.ay = (float)(-0.5 * ck * std::sin(th));
             f.bx = (float)(0.5 * c1 * std::cos(th - q)); f.by = (float)(0.5 * c1 * std::sin(th - q));
-            v.ax = (float)(0.5 * sk * std::cos(th)); v.ay = (float)(0.5 * sk * std::sin(th));
-            v.bx = (float)(0.5 * s1 * std::cos(q - th)); v.by = (float)(0.5 * s1 * std::sin(q - th));
-            hf[k] = f; hi[k] = v;
+            hf[k] = f;
         }
         const int np = Mh / 2 + 1;
-        std::vector<float4> pf(np), pi(np);
-        for (int k = 0; k < np; ++k) {
-            pf[k] = make_float4(hf[k].wnx, hf[k].wny, hf[k].ax, hf[k].ay);
-            pi[k] = make_float4(hi[k].wnx, hi[k].wny, hi[k].ax, hi[k].ay);
-        }
+        std::vector<float4> pf(np);
+        for (int k = 0; k < np; ++k) pf[k] = make_float4(hf[k].wnx, hf[k].wny, hf[k].ax, hf[k].ay);
         twF0 = make_float2(hf[0].bx, hf[0].by);
-        twI0 = make_float2(hi[0].bx, hi[0].by);
         if (cudaMalloc(&twF, pf.size() * sizeof(float4)) != cudaSuccess) return CCMSAV_ENOMEM;
-        if (cudaMalloc(&twI, pi.size() * sizeof(float4)) != cudaSuccess) return CCMSAV_ENOMEM;
         CCM_CUDA(cudaMemcpyAsync(twF, pf.data(), pf.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
-        CCM_CUDA(cudaMemcpyAsync(twI, pi.data(), pi.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
         CCM_CUDA(cudaStreamSynchronize(st));
         int r = CCMSAV_EINVAL;
         if (const lf::Ops* lo = lf::wide_ops(Mh)) {
@@ -924,23 +889,26 @@ public:
         SpecCoefF sf{(float)s.C1, (float)s.C2, (float)s.C3, (float)s.Ct, (float)s.lam};
         const float* fin = reinterpret_cast<const float*>(bufA);
         float* fB = reinterpret_cast<float*>(bufB);
-        const cplx<float>* t2 = tw2;
-        kw_rowdct_T<MM><<<dim3(N / wRT, NF), kWarps * 32, wsm_rt, st>>>(fin, fB, t2, pair_tab(twF), ahead_rt, GroupArgs<false>{}, 0);
-        mark(1);
-        if constexpr (WGeo<MM>::WPL > 1)
-            kw_coldct_gram_split<MM><<<dim3(N, 2), kSplitWarps * 32, wsm_col, st>>>(fB, reinterpret_cast<float*>(bufA), part2,
-                                                                                  t2, pair_tab(twF), evf, evp, sf);
-        else
-            kw_coldct_gram<MM><<<N / wKC, kWarps * 32, wsm_col, st>>>(fB, reinterpret_cast<float*>(bufA), part2, t2, pair_tab(twF), evf, evp, sf,
-                                                                     GroupArgs<false>{}, 0);
+        if constexpr (MM == 4096) {
+            lf::launch_cluster(lf::FwdGeo<MM>::CLUSTER, lf::kl_row<MM>, dim3(N / lf::FwdGeo<MM>::LINES, NF), lf::FwdGeo<MM>::THREADS,
+                               lf::FwdGeo<MM>::SMEM, st, fin, fB, lt.tw, wide_fwd());
+            mark(1);
+            lf::kl_col<MM><<<N, lf::ColGeo<MM>::THREADS, lf::ColGeo<MM>::SMEM, st>>>(fB, reinterpret_cast<float*>(bufA), part2, lt.tw,
+                                                                                     wide_fwd(), evf, sf);
+        } else {
+            kw_rowdct_T<MM><<<dim3(N / wRT, NF), kWarps * 32, wsm_rt, st>>>(fin, fB, tw2, pair_tab(), ahead_rt, GroupArgs<false>{}, 0);
+            mark(1);
+            kw_coldct_gram<MM><<<N / wKC, kWarps * 32, wsm_col, st>>>(fB, reinterpret_cast<float*>(bufA), part2, tw2, pair_tab(), evf, evp,
+                                                                     sf, GroupArgs<false>{}, 0);
+        }
         mark(2);
     }
     int bdf1_launch = 0;
     template <int MM>
     void launch_warp_inverse(const SpecCoef& s, int anchor) {
         SpecCoefF sf{(float)s.C1, (float)s.C2, (float)s.C3, (float)s.Ct, (float)s.lam};
-        lf::kl_comb<MM><<<2 * N / lf::Geo<MM>::LINES, lf::Geo<MM>::THREADS, lf::Geo<MM>::SMEM, st>>>(
-            reinterpret_cast<const float*>(bufA), reinterpret_cast<float*>(bufB), lt.tw, wide_inv(), evf, evp, sf, sc, anchor,
+        lf::launch_cluster(lf::comb_cluster<MM>(), lf::kl_comb<MM>, 2 * N / lf::Geo<MM>::LINES, lf::Geo<MM>::THREADS,
+            lf::Geo<MM>::SMEM, st, reinterpret_cast<const float*>(bufA), reinterpret_cast<float*>(bufB), lt.tw, wide_inv(), evf, evp, sf, sc, anchor,
             GroupArgs<false>{}, 0);
         mark(4);
         lf::kl_irow<MM><<<2 * N / lf::RowGeo<MM>::LINES, lf::RowGeo<MM>::THREADS, lf::RowGeo<MM>::SMEM, st>>>(
@@ -1042,26 +1010,30 @@ public:
         return CCMSAV_OK;
     }
 
-    int init_scalars_from_fields(double psi_sum_fp64) {
-        double s[NDIAG];
-        int r = CCMSAV_OK;
+    // The sums of set_state over the current level (k_diag's columns; FP32:
+    // column 5 counts the cells with a non-finite value).
+    int init_sums(double s[NDIAG]) {
         if constexpr (std::is_same<T, float>::value) {
-            // FP32 fields: the five sums in the step's FP32 arithmetic
+            // the five sums in the step's FP32 arithmetic
             const double hh = h();
             InitCoefF ic{(float)(1.0 / hh), (float)p.eps, (float)(1.0 / p.eps), (float)p.beta, (float)p.gamma_in,
                          (float)p.gamma_out, (float)p.psi_in, (float)p.psi_out, (float)p.beta_in, (float)p.beta_out};
             k_init_sums_f32<<<g_dg, 256, 0, st>>>(phi[cur], psi[cur], partd, N, ic);
-            ++nlaunch;
-            CCM_CUDA(cudaGetLastError());
-            CCM_CUDA(cudaMemcpyAsync(h_part, partd, (size_t)nbd * NDIAG * sizeof(double), cudaMemcpyDeviceToHost, st));
-            CCM_CUDA(cudaStreamSynchronize(st));
-            for (int q = 0; q < NDIAG; ++q) s[q] = 0.0;
-            for (int bk = 0; bk < nbd; ++bk)
-                for (int q = 0; q < 5; ++q) s[q] += h_part[(size_t)bk * NDIAG + q];
         } else {
-            r = diag_sums(phi[cur], phi[cur], psi[cur], s);
+            k_diag<T, true><<<g_dg, 256, 0, st>>>(phi[cur], phi[cur], psi[cur], partd, N, diag_coef());
         }
-        if (r) return r;
+        ++nlaunch;
+        CCM_CUDA(cudaGetLastError());
+        CCM_CUDA(cudaMemcpyAsync(h_part, partd, (size_t)nbd * NDIAG * sizeof(double), cudaMemcpyDeviceToHost, st));
+        CCM_CUDA(cudaStreamSynchronize(st));
+        for (int q = 0; q < NDIAG; ++q) s[q] = 0.0;
+        for (int bk = 0; bk < nbd; ++bk)
+            for (int q = 0; q < NDIAG; ++q) s[q] += h_part[(size_t)bk * NDIAG + q];
+        return CCMSAV_OK;
+    }
+
+    // Initial SAVs, arc length and conserved mean from those sums.
+    int init_scalars(const double s[NDIAG], double psi_sum_fp64) {
         const double h2 = h() * h();
         std::memset(sc_host, 0, sizeof(DevScalars));
         sc_host->V = sc_host->Vo = std::sqrt(h2 * s[0]);
@@ -1082,7 +1054,9 @@ public:
         cur = 0; prev = 1; spare = 2;
         double psum = 0.0;
         int r = upload_levels(phi0, psi0, phi1, psi1, &psum);
-        if (r == CCMSAV_OK) r = init_scalars_from_fields(psum);
+        double s[NDIAG];
+        if (r == CCMSAV_OK) r = init_sums(s);
+        if (r == CCMSAV_OK) r = init_scalars(s, psum);
         if (r) { have_state = false; return r; }   // the levels were overwritten: no state
         have_state = true; poisoned = false;
         steps_taken = (phi1 && psi1) ? 1 : 0;   // two given levels: continue with BDF2
@@ -1097,10 +1071,14 @@ public:
         CCM_CUDA(cudaMemcpyAsync(phi[prev], dphi, fb, cudaMemcpyDeviceToDevice, st));
         CCM_CUDA(cudaMemcpyAsync(psi[prev], dpsi, fb, cudaMemcpyDeviceToDevice, st));
         double s[NDIAG];
-        int r = diag_sums(phi[cur], phi[cur], psi[cur], s);
+        int r = init_sums(s);
         if (r) return r;
-        for (int q = 0; q < NDIAG; ++q) if (!std::isfinite(s[q])) return CCMSAV_ENONFINITE;
-        r = init_scalars_from_fields(s[13]);
+        if (std::is_same<T, float>::value) {
+            if (s[5] != 0.0 || !std::isfinite(s[13])) return CCMSAV_ENONFINITE;
+        } else {
+            for (int q = 0; q < NDIAG; ++q) if (!std::isfinite(s[q])) return CCMSAV_ENONFINITE;
+        }
+        r = init_scalars(s, s[13]);
         if (r) return r;
         have_state = true; poisoned = false; steps_taken = 0;
         return CCMSAV_OK;

@@ -120,8 +120,8 @@ struct BatchArgs {
     double* part1; double* part2; double* part3;                              // partial rows, solve slices
     DevScalars* sc;
     const cplx<float>* tw2;                                                   // four-step twiddles
-    wf::PairTwTab twF, twI;                                                   // DCT pair twiddles
-    const float2* tww; lf::PairTab tiw;                                       // wide lines: twiddles, inverse pairs
+    wf::PairTwTab twF;                                                        // DCT pair twiddles
+    const float2* tww; lf::PairTab tfw, tiw;                                  // wide lines: twiddles, pairs
     const float* evf; const float4* evp;                                      // FP32 eigenvalues
     StencilCoef<float> c;
     SpecCoefF sf;

@@ -174,28 +174,21 @@ template <int R> __host__ __device__ constexpr int bitrev(int r) {
     return o;
 }
 
-// Line shapes M = E x G (E values on each of G lanes).  S selects a variant:
-// the forward transforms run 2048-point lines as 64 x 32 (one warp per line)
-// and 4096-point lines as 64 x 64; the inverse kernels, which wait on memory
-// and gain from the lower register use, take 32 x 64 and 32 x 128 (two and
-// four warps per line, fourstep_split).
-template <int M> struct ShapeBase;
-template <> struct ShapeBase<64>   { static constexpr int E = 8,  G = 8;  };
-template <> struct ShapeBase<128>  { static constexpr int E = 16, G = 8;  };
-template <> struct ShapeBase<256>  { static constexpr int E = 16, G = 16; };
-template <> struct ShapeBase<512>  { static constexpr int E = 32, G = 16; };
-template <> struct ShapeBase<1024> { static constexpr int E = 32, G = 32; };
-template <> struct ShapeBase<2048> { static constexpr int E = 64, G = 32; };
-template <> struct ShapeBase<4096> { static constexpr int E = 64, G = 64; };
-template <int M, int S = 0> struct Shape : ShapeBase<M> {};
-template <> struct Shape<2048, 1> { static constexpr int E = 32, G = 64; };
-template <> struct Shape<4096, 1> { static constexpr int E = 32, G = 128; };
+// Line shapes M = E x G (E values on each of G lanes, one line per lane group
+// of a warp).
+template <int M> struct Shape;
+template <> struct Shape<64>   { static constexpr int E = 8,  G = 8;  };
+template <> struct Shape<128>  { static constexpr int E = 16, G = 8;  };
+template <> struct Shape<256>  { static constexpr int E = 16, G = 16; };
+template <> struct Shape<512>  { static constexpr int E = 32, G = 16; };
+template <> struct Shape<1024> { static constexpr int E = 32, G = 32; };
+template <> struct Shape<2048> { static constexpr int E = 64, G = 32; };
 
 // Lane n2 of its line's group and the line's slot in the CTA: G <= 32 puts
 // 32 / G lines in a warp; G = 64, 128 spreads a line over 2, 4 consecutive
 // warps.
-template <int M, int S = 0> __device__ __forceinline__ void lane_geo(int& n2, int& slot) {
-    constexpr int G = Shape<M, S>::G;
+template <int M> __device__ __forceinline__ void lane_geo(int& n2, int& slot) {
+    constexpr int G = Shape<M>::G;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if constexpr (G <= 32) {
         n2 = lane % G;
@@ -222,10 +215,8 @@ template <int G> __device__ __forceinline__ void line_sync(int slot) {
 // that, as float rows, consecutive line buffers sit 4 banks apart (the
 // strided reads of the transposed writes).  Swizzled (SWZ = true): M values
 // + 2, for kernels that need more lines per SM.
-template <int M, bool SWZ = false, int S = 0> __host__ __device__ constexpr int buf_len() {
-    return Shape<M, S>::E < Shape<M, S>::G                                          // fourstep_split's rows
-             ? Shape<M, S>::E * (Shape<M, S>::G + Shape<M, S>::G / Shape<M, S>::E)
-         : SWZ ? M + 2 : Shape<M, S>::E * (Shape<M, S>::G + 1) + 2;
+template <int M, bool SWZ = false> __host__ __device__ constexpr int buf_len() {
+    return SWZ ? M + 2 : Shape<M>::E * (Shape<M>::G + 1) + 2;
 }
 
 // Position of element c of transpose row R (E rows of G values).  Padded:
@@ -236,82 +227,17 @@ template <int M, bool SWZ = false, int S = 0> __host__ __device__ constexpr int 
 // values of its row (n2 J + j) with one 16-byte load, on distinct banks within
 // each quarter-warp for G >= 16.  For E = 64, swz(R) = (R / J) mod G with
 // 8-byte reads (measured faster there).
-template <int M, int S = 0> __host__ __device__ constexpr bool wide_reads() { return Shape<M, S>::E <= 32; }
-template <int M, bool SWZ, int S = 0> __device__ __forceinline__ int tpos(int R, int c) {
-    constexpr int G = Shape<M, S>::G, J = Shape<M, S>::E / Shape<M, S>::G, W = wide_reads<M, S>() ? 2 : 1;
+template <int M> __host__ __device__ constexpr bool wide_reads() { return Shape<M>::E <= 32; }
+template <int M, bool SWZ> __device__ __forceinline__ int tpos(int R, int c) {
+    constexpr int G = Shape<M>::G, J = Shape<M>::E / Shape<M>::G, W = wide_reads<M>() ? 2 : 1;
     return SWZ ? R * G + (c ^ ((W * (R / J)) & (G - 1))) : R * (G + 1) + c;
-}
-
-// The four steps for lines of G = R E lanes (E values each, R = 2 or 4): the
-// E-point DFTs and the twiddles as below, then each G-point row k1 of the
-// transpose is split over R adjacent lanes (lane R k1 + q takes the columns
-// R t + q, t = 0 .. E-1), each lane takes an E-point DFT Y_q of its part,
-// multiplies it by W_G^{q k} (U_q), and the R lanes combine by an R-point DFT
-// through shuffles:
-//   X[k1 + E (k + E s)] = sum_q W_R^{q s} U_q[k]        (conjugates for INV),
-// R = 2 in one radix-2 step (lane q keeps s = q), R = 4 in two (pairs q, q^2,
-// then q, q^1; lane q keeps s = bit-reversed q).  W_G^{q k} = W_M^{E q k} is
-// the table entry of k1 = k, n2 = E q: tw2[k G + E q].  Transpose rows are
-// padded to G + R values:
-// the row writes (one row, all lanes) and the part-row reads (16 / R rows and
-// all R parts per half-warp, 8-byte words) touch distinct banks.
-template <typename T, int M, bool INV, int S = 0>
-__device__ __forceinline__ void fourstep_split(cplx<T>* v, cplx<T>* buf, const cplx<T>* __restrict__ tw2, int n2, int slot) {
-    constexpr int E = Shape<M, S>::E, G = Shape<M, S>::G, R = G / E, P = G + R;
-    static_assert(R == 2 || R == 4, "two or four lanes per transpose row");
-    DIF<T, E, INV, 0>::run(v);                   // v[r] = X1[k1 = bitrev(r)] of column n2
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int k1 = bitrev<E>(r);
-        const cplx<T> w = tw2[k1 * G + n2];
-        buf[k1 * P + n2] = INV ? cmulc(v[r], w) : cmul(v[r], w);
-    }
-    line_sync<G>(slot);
-    const int k1 = n2 / R, q = n2 % R;
-#pragma unroll
-    for (int t = 0; t < E; ++t) v[t] = buf[k1 * P + R * t + q];
-    line_sync<G>(slot);
-    DIF<T, E, INV, 0>::run(v);                   // v[r] = Y_q[k = bitrev(r)]
-    constexpr unsigned FULL = 0xffffffffu;
-    if constexpr (R == 2) {
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int k = bitrev<E>(r);
-            const T px = __shfl_xor_sync(FULL, v[r].x, 1);
-            const T py = __shfl_xor_sync(FULL, v[r].y, 1);
-            const cplx<T> y0 = q ? mk(px, py) : v[r];
-            const cplx<T> y1 = twid<T, G, INV>(q ? v[r] : mk(px, py), k);
-            buf[k1 + E * (k + E * q)] = q ? y0 - y1 : y0 + y1;
-        }
-    } else {
-        const int s = ((q & 1) << 1) | (q >> 1);  // output index of this lane
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int k = bitrev<E>(r);
-            const cplx<T> w = tw2[k * G + E * q];            // W_G^{q k}
-            cplx<T> u = INV ? cmulc(v[r], w) : cmul(v[r], w);
-            // pairs (q, q ^ 2): lanes q < 2 keep U_q + U_{q^2}, lanes q >= 2 keep U_{q^2} - U_q
-            T px = __shfl_xor_sync(FULL, u.x, 2), py = __shfl_xor_sync(FULL, u.y, 2);
-            u = (q & 2) ? mk(px - u.x, py - u.y) : mk(u.x + px, u.y + py);
-            // pairs (q, q ^ 1): even lanes X = A_q + w4 A_{q^1}, odd lanes X = A_{q^1} - w4 A_q,
-            // w4 = 1 for q < 2 and W_4 (-i; +i for INV) for q >= 2
-            px = __shfl_xor_sync(FULL, u.x, 1); py = __shfl_xor_sync(FULL, u.y, 1);
-            const cplx<T> a = (q & 1) ? mk(px, py) : u, b = (q & 1) ? u : mk(px, py);
-            const cplx<T> wb = (q & 2) ? (INV ? mk(-b.y, b.x) : mk(b.y, -b.x)) : b;
-            buf[k1 + E * (k + E * s)] = (q & 1) ? a - wb : a + wb;
-        }
-    }
-    line_sync<G>(slot);
 }
 
 // Steps 1-4.  v: this lane's E values in four-step order.  buf: this line's
 // buffer.  On return buf[k] = Z[k], k = 0..M-1 (visible to the warp).
-template <typename T, int M, bool INV, bool SWZ = false, int S = 0>
+template <typename T, int M, bool INV, bool SWZ = false>
 __device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>* __restrict__ tw2, int n2, int slot) {
-  if constexpr (Shape<M, S>::E < Shape<M, S>::G) {
-    fourstep_split<T, M, INV, S>(v, buf, tw2, n2, slot);
-  } else {
-    constexpr int E = Shape<M, S>::E, G = Shape<M, S>::G, J = E / G;
+    constexpr int E = Shape<M>::E, G = Shape<M>::G, J = E / G;
     DIF<T, E, INV, 0>::run(v);
     if constexpr (!INV) {
         // twiddles W_M^{n2 k1}: k1 = bitrev(r) is below E/2 for even r; for odd
@@ -323,23 +249,23 @@ __device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>
         for (int r = 0; r < E; r += 2) {
             const int k1 = bitrev<E>(r);
             const cplx<T> w = tw2[k1 * G + n2];
-            buf[tpos<M, SWZ, S>(k1, n2)] = cmul(v[r], w);
-            buf[tpos<M, SWZ, S>(k1 + E / 2, n2)] = cmul(v[r + 1], cmul(w, wh));
+            buf[tpos<M, SWZ>(k1, n2)] = cmul(v[r], w);
+            buf[tpos<M, SWZ>(k1 + E / 2, n2)] = cmul(v[r + 1], cmul(w, wh));
         }
     } else {
 #pragma unroll
         for (int r = 0; r < E; ++r) {
             const int k1 = bitrev<E>(r);
-            buf[tpos<M, SWZ, S>(k1, n2)] = cmulc(v[r], tw2[k1 * G + n2]);
+            buf[tpos<M, SWZ>(k1, n2)] = cmulc(v[r], tw2[k1 * G + n2]);
         }
     }
     line_sync<G>(slot);
-    if constexpr (SWZ && wide_reads<M, S>() && std::is_same<T, float>::value) {
+    if constexpr (SWZ && wide_reads<M>() && std::is_same<T, float>::value) {
 #pragma unroll
         for (int j = 0; j < J; ++j)
 #pragma unroll
             for (int m = 0; m < G; m += 2) {
-                const float4 q = *reinterpret_cast<const float4*>(buf + tpos<M, SWZ, S>(n2 * J + j, m));
+                const float4 q = *reinterpret_cast<const float4*>(buf + tpos<M, SWZ>(n2 * J + j, m));
                 v[j * G + m] = mk(q.x, q.y);
                 v[j * G + m + 1] = mk(q.z, q.w);
             }
@@ -347,7 +273,7 @@ __device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>
 #pragma unroll
         for (int j = 0; j < J; ++j)
 #pragma unroll
-            for (int m = 0; m < G; ++m) v[j * G + m] = buf[tpos<M, SWZ, S>(n2 * J + j, m)];
+            for (int m = 0; m < G; ++m) v[j * G + m] = buf[tpos<M, SWZ>(n2 * J + j, m)];
     }
     line_sync<G>(slot);
 #pragma unroll
@@ -360,7 +286,6 @@ __device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>
 #pragma unroll
         for (int r = 0; r < G; ++r) buf[(n2 * J + j) + E * bitrev<G>(r)] = v[j * G + r];
     line_sync<G>(slot);
-  }
 }
 
 // Forward pack from a real line x in global memory (16-byte aligned):

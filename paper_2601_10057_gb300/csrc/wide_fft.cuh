@@ -8,6 +8,7 @@
 // one up to M = 1024 in the step, but at M = 2048 and 4096 it needs 219 - 255
 // registers per thread and eight warps per SM then wait on memory.
 #pragma once
+#include <cooperative_groups.h>
 #include "dct_device.cuh"
 #include "warp_fft.cuh"
 #include "bounds.cuh"
@@ -228,6 +229,80 @@ __device__ __forceinline__ void write_samples(const cf* bufs, float* __restrict_
         *reinterpret_cast<float4*>(d + 2 * (size_t)N) = make_float4(a[0].y, a[1].y, a[2].y, a[3].y);
         *reinterpret_cast<float4*>(d + 3 * (size_t)N) = make_float4(b[0].x, b[1].x, b[2].x, b[3].x);
     }
+}
+
+// The same writes by a cluster of two CTAs of four lines each, which together
+// hold eight rows: each CTA writes half of the modes (samples) of all eight,
+// reading the other's four lines through distributed shared memory, so that a
+// row segment is 32 bytes (a whole sector) where eight lines do not fit one
+// CTA.  dst: the first of the eight rows.
+template <int M>
+__device__ __forceinline__ void write_modes_pair(cf* bufs, float* __restrict__ dst, const PairTab& t, size_t o0, size_t lim) {
+    using Gm = Geo<M>;
+    constexpr int N = Gm::N;
+    auto cl = cooperative_groups::this_cluster();
+    const int rank = (int)cl.block_rank(), r4 = threadIdx.x & 1;
+    const cf* z = cl.map_shared_rank(bufs, r4);
+    cl.sync();
+    auto put = [&](int mode, float a, float b, float c, float d) {
+        if (CCM_OKW(o0 + (size_t)mode * N + 4 * r4, 4, lim))
+            *reinterpret_cast<float4*>(dst + (size_t)mode * N + 4 * r4) = make_float4(a, b, c, d);
+    };
+#pragma unroll 1
+    for (int q = threadIdx.x; q < M / 2; q += blockDim.x) {
+        const int k = rank * (M / 4) + (q >> 1);
+        cf s1[4], s2[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) post_item<M>(z + (size_t)r * Gm::BUF, t, k, s1[r], s2[r]);
+        const int i2 = item_slot2<M>(k);
+        put(slot_mode<M>(k, 0), s1[0].x, s1[1].x, s1[2].x, s1[3].x);
+        put(slot_mode<M>(k, 1), s1[0].y, s1[1].y, s1[2].y, s1[3].y);
+        put(slot_mode<M>(i2, 0), s2[0].x, s2[1].x, s2[2].x, s2[3].x);
+        put(slot_mode<M>(i2, 1), s2[0].y, s2[1].y, s2[2].y, s2[3].y);
+    }
+    cl.sync();                                         // the other CTA may still read these lines
+}
+template <int M> __device__ __forceinline__ void write_samples_pair(cf* bufs, float* __restrict__ dst) {
+    using Gm = Geo<M>;
+    constexpr int N = Gm::N;
+    auto cl = cooperative_groups::this_cluster();
+    const int rank = (int)cl.block_rank(), r4 = threadIdx.x & 1;
+    const cf* zr = cl.map_shared_rank(bufs, r4);
+    cl.sync();
+#pragma unroll 1
+    for (int q = threadIdx.x; q < M / 2; q += blockDim.x) {
+        const int m = rank * (M / 4) + (q >> 1);
+        cf a[4], b[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const cf* z = zr + (size_t)r * Gm::BUF;
+            a[r] = z[m];
+            b[r] = z[M - 1 - m];
+        }
+        float* d = dst + (size_t)(4 * m) * N + 4 * r4;
+        *reinterpret_cast<float4*>(d) = make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
+        *reinterpret_cast<float4*>(d + N) = make_float4(b[0].y, b[1].y, b[2].y, b[3].y);
+        *reinterpret_cast<float4*>(d + 2 * (size_t)N) = make_float4(a[0].y, a[1].y, a[2].y, a[3].y);
+        *reinterpret_cast<float4*>(d + 3 * (size_t)N) = make_float4(b[0].x, b[1].x, b[2].x, b[3].x);
+    }
+    cl.sync();
+}
+
+// Launch in clusters of `cluster` CTAs along x (1: a plain launch).
+template <typename... KA, typename... A>
+inline void launch_cluster(int cluster, void (*kernel)(KA...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);        // errors: cudaGetLastError, as after <<<>>>
 }
 
 }  // namespace lf

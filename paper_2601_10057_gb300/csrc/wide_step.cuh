@@ -1,9 +1,11 @@
-// wide_step.cuh -- the FP32 step's inverse kernels on the lines of
-// wide_fft.cuh: recovery + inverse columns and inverse rows (N = 128 .. 8192).
+// wide_step.cuh -- FP32 step kernels on the lines of wide_fft.cuh: recovery +
+// inverse columns and inverse rows (N = 128 .. 8192), and the forward passes of
+// N = 8192.
 //
-// Both wait on memory, and on warp-level lines (32 or 64 values per lane, 72 -
-// 128 registers) they held 16 - 24 warps per SM; with sixteen values per lane
-// 32 warps fit.  The recovery kernel takes one field per CTA (the phi CTAs,
+// The inverse kernels wait on memory, and on warp-level lines (32 or 64 values
+// per lane, 72 - 128 registers) they held 16 - 24 warps per SM; with sixteen
+// values per lane 32 warps fit: N = 2048 recovery 61 -> 45 us, inverse rows
+// 40 -> 31; N = 8192 1112 -> 743, 839 -> 394.  The recovery kernel takes one field per CTA (the phi CTAs,
 // five spectra, come first, the lighter psi CTAs fill the tail).
 #pragma once
 #include "warp_kernels.cuh"
@@ -12,6 +14,177 @@
 namespace ccm {
 namespace lf {
 
+// ------------------------------------------------------------------ forward rows
+// 4096-point lines: clusters of two CTAs of four rows each (write_modes_pair).
+// Shorter lines take the warp-level kernels of warp_kernels.cuh, which move a
+// line through shared memory once less: measured at N = 8192 row 1894 us with
+// 64 x 64 lines on two warps, 1995 on wide lines with 16-byte segments, 1610
+// with the cluster; column pass 2022 -> 1300; but N = 4096 row 294 (warp) / 374
+// (cluster), column 338 / 349, N = 2048 row 63 / 81, column 64 / 82.
+template <int M> struct FwdGeo {
+    static constexpr int LINES = 4, CLUSTER = 2;
+    static constexpr int THREADS = LINES * Geo<M>::G;
+    static constexpr size_t SMEM = (size_t)LINES * Geo<M>::BUF * sizeof(cf);
+    static constexpr int MINB = 1024 / THREADS;
+};
+
+// Forward DCT-II along x of four rows of field blockIdx.y per CTA, eight per
+// cluster, transposed write.
+template <int M>
+__global__ void __launch_bounds__(FwdGeo<M>::THREADS, FwdGeo<M>::MINB)
+kl_row(const float* __restrict__ in, float* __restrict__ out, const float2* __restrict__ tw, PairTab tf) {
+    using Gm = Geo<M>;
+    constexpr int N = Gm::N;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    cf* bufs = reinterpret_cast<cf*>(smraw);
+    int n2, slot;
+    lane_of<M>(n2, slot);
+    const size_t NN = (size_t)N * N, f0 = blockIdx.y * NN;
+    const int y = blockIdx.x * FwdGeo<M>::LINES + slot, y0 = (blockIdx.x & ~1) * FwdGeo<M>::LINES;
+    forward_line<M, false>(in + CCM_IXW(f0 + (size_t)y * N, N, NF * NN), bufs + (size_t)slot * Gm::BUF, tw, n2, slot, false);
+    write_modes_pair<M>(bufs, out + f0 + y0, tf, f0 + y0, NF * NN);
+}
+
+// ------------------------------------------------------------------ forward columns and Gram sums
+// Sixteen of the seventeen Gram sums of a mode, f0' f0' left out (not used by
+// the solve; its column stays 0): for b = 1 .. 4 the products with a = 0 .. b,
+// then PG, PL.  psi only / phi only for the split column pass.
+template <bool PHI, bool PSI>
+__device__ __forceinline__ void gram_mode(float (&acc)[16], const float (&v)[NF], float isig, float itau) {
+    if constexpr (PHI) {
+        int p = 0;
+#pragma unroll
+        for (int b = 1; b < 5; ++b) {
+            const float w = v[b] * isig;
+#pragma unroll
+            for (int a = 0; a <= b; ++a) { acc[p] = fmaf(v[a], w, acc[p]); ++p; }
+        }
+    }
+    if constexpr (PSI) {
+        const float w = v[5] * itau;
+        acc[14] = fmaf(v[6], w, acc[14]);
+        acc[15] = fmaf(v[7], w, acc[15]);
+    }
+}
+// Accumulator p -> column of a partial row (a <= b over f0' S H Q K row by row, PG, PL)
+__device__ __forceinline__ int gram_col(int p) {
+    if (p >= 14) return p + 1;
+    const int b = p < 2 ? 1 : p < 5 ? 2 : p < 9 ? 3 : 4, a = p - (b == 1 ? 0 : b == 2 ? 2 : b == 3 ? 5 : 9);
+    return a * 5 - a * (a - 1) / 2 + (b - a);
+}
+// Block sums into a partial row of float pairs: FP32 over a warp by recursive
+// halving (16 values in 16 exchanges), double-float over the warps.
+template <int THREADS>
+__device__ __forceinline__ void gram_store(float (&acc)[16], float2* __restrict__ row, float* __restrict__ sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int idx = 0;
+#pragma unroll
+    for (int h = 8; h >= 1; h >>= 1) {
+        const bool up = lane & h;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float give = up ? acc[i] : acc[i + h], keep = up ? acc[i + h] : acc[i];
+            acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+        }
+        if (up) idx += h;
+    }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 16);
+    __syncthreads();                                   // the line buffers are free
+    if (lane < 16) sm[warp * 16 + idx] = acc[0];
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        float hi = 0.f, lo = 0.f;
+#pragma unroll 8
+        for (int w = 0; w < THREADS / 32; ++w) df_add(hi, lo, sm[w * 16 + threadIdx.x]);
+        row[gram_col(threadIdx.x)] = make_float2(hi, lo);
+    }
+    if (threadIdx.x == 16) row[0] = make_float2(0.f, 0.f);
+}
+
+// Columns: the eight lines of a spectral row do not fit a CTA, so they go four
+// at a time through five buffers: first P, g0', L_P and K, whose psi sums are
+// formed before f0', S, H, Q take places beside K.
+template <int M> struct ColGeo {
+    static constexpr int LINES = 4, COLS = 5;
+    static constexpr int THREADS = LINES * Geo<M>::G;
+    static constexpr size_t SMEM = (size_t)COLS * Geo<M>::BUF * sizeof(cf);
+};
+
+// Post-process of a line in place (slots of modes) and its spectrum in pair
+// order (SpecRow: float4 of modes k, N-k, M-k, M+k for k = 0 .. M/2; pair 0 holds
+// X[0], 0, X[M], X[M], pair M/2 its two modes twice); dst null: not stored.
+template <int M> __device__ __forceinline__ void post_line(cf* buf, const PairTab& tf, float* dst, int n2) {
+#pragma unroll 2
+    for (int k = n2; k < M / 2; k += Geo<M>::G) {
+        cf s1, s2;
+        post_item<M>(buf, tf, k, s1, s2);
+        buf[k] = s1;
+        buf[item_slot2<M>(k)] = s2;
+        if (dst) {
+            float4* d = reinterpret_cast<float4*>(dst);
+            d[k] = k == 0 ? make_float4(s1.x, 0.f, s1.y, s1.y) : make_float4(s1.x, s1.y, s2.x, s2.y);
+            if (k == 0) d[M / 2] = make_float4(s2.x, s2.y, s2.x, s2.y);
+        }
+    }
+}
+// Gram sums over the slots of a spectral row; buffer of field f: bufs + pos[f] BUF
+template <int M, bool PHI, bool PSI>
+__device__ __forceinline__ void gram_slots(float (&acc)[16], const cf* bufs, const int (&pos)[NF], float evx,
+                                           const float* __restrict__ evf, const SpecCoefF& sc) {
+#pragma unroll 1
+    for (int i = threadIdx.x; i < M; i += ColGeo<M>::THREADS) {
+        float a[NF], b[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            if (f < 5 ? !PHI : !PSI) { a[f] = b[f] = 0.f; continue; }
+            const cf z = bufs[(size_t)pos[f] * Geo<M>::BUF + i];
+            a[f] = z.x;
+            b[f] = z.y;
+        }
+        const float s0 = evx + __ldg(evf + slot_mode<M>(i, 0)), s1 = evx + __ldg(evf + slot_mode<M>(i, 1));
+        // correctly rounded reciprocals (the same values as 1.0f / x)
+        gram_mode<PHI, PSI>(acc, a, PHI ? __frcp_rn(sc.C1 + s0 * (sc.C2 + sc.C3 * s0)) : 0.f, PSI ? __frcp_rn(sc.Ct + sc.lam * s0) : 0.f);
+        gram_mode<PHI, PSI>(acc, b, PHI ? __frcp_rn(sc.C1 + s1 * (sc.C2 + sc.C3 * s1)) : 0.f, PSI ? __frcp_rn(sc.Ct + sc.lam * s1) : 0.f);
+    }
+}
+
+// Forward DCT-II along y of the eight fields of spectral row kx, the spectra
+// and the Gram sums.
+template <int M>
+__global__ void __launch_bounds__(ColGeo<M>::THREADS, 1)
+kl_col(const float* __restrict__ in, float* __restrict__ spec, double* __restrict__ part, const float2* __restrict__ tw,
+       PairTab tf, const float* __restrict__ evf, SpecCoefF sc) {
+    using Gm = Geo<M>;
+    constexpr int N = Gm::N;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    cf* bufs = reinterpret_cast<cf*>(smraw);
+    const int kx = blockIdx.x;
+    int n2, slot;
+    lane_of<M>(n2, slot);
+    const size_t NN = (size_t)N * N;
+    const float evx = __ldg(evf + kx);
+    float acc[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+    float* srow = spec + CCM_IXW((size_t)kx * SpecRow<M>::KS, SpecRow<M>::KS, (size_t)N * SpecRow<M>::KS);
+    auto line = [&](int f, int p) {
+        cf* buf = bufs + (size_t)p * Gm::BUF;
+        forward_line<M, false>(in + CCM_IXW(f * NN + (size_t)kx * N, N, NF * NN), buf, tw, n2, slot, false);
+        post_line<M>(buf, tf, f == 5 ? nullptr : srow + (size_t)(f < 5 ? f : f - 1) * SpecRow<M>::FO, n2);   // P^: Gram sums only
+    };
+    constexpr int pos[NF] = {0, 1, 2, 4, 3, 0, 1, 2};     // buffer of each field
+    line(slot < 3 ? 5 + slot : 4, slot);
+    __syncthreads();
+    gram_slots<M, false, true>(acc, bufs, pos, evx, evf, sc);
+    __syncthreads();
+    line(slot, slot < 3 ? slot : 4);
+    __syncthreads();
+    gram_slots<M, true, false>(acc, bufs, pos, evx, evf, sc);
+    __syncthreads();
+    gram_store<ColGeo<M>::THREADS>(acc, reinterpret_cast<float2*>(part) + (size_t)kx * NRED2, reinterpret_cast<float*>(smraw));
+}
+
+// ------------------------------------------------------------------ recovery and inverse columns
 // LINES spectral rows of one field: recovery combination and divide, inverse
 // DCT along y, transposed write out[f][y][kx].  Block b: field b / (N / LINES).
 template <int M, bool GRP = false>
@@ -94,9 +267,14 @@ kl_comb(const float* __restrict__ spec, float* __restrict__ out, const float2* _
         const double dsum = line_sum_exact<G>(dhi, dlo, slot, lsum);
         if (slot == 0 && n2 == 0) dsc->dc_col = dsum;
     }
-    __syncthreads();
-    write_samples<M, Gm::LINES>(bufs, out + f * NN + x0);
+    if constexpr (Gm::LINES == 4) {                       // comb_cluster: two CTAs
+        write_samples_pair<M>(bufs, out + f * NN + (size_t)(x0 & ~7));
+    } else {
+        __syncthreads();
+        write_samples<M, Gm::LINES>(bufs, out + f * NN + x0);
+    }
 }
+template <int M> __host__ __device__ constexpr int comb_cluster() { return Geo<M>::LINES == 4 ? 2 : 1; }
 
 // Rows per CTA of the inverse row kernel: four (the lines are independent;
 // smaller CTAs leave less of a last wave idle), two at M = 4096.
@@ -111,7 +289,7 @@ template <int M> struct RowGeo {
 
 // Inverse DCT along x of LINES rows of one field and u^{n+1} = u_bar + du with
 // the compensated (and, for psi, error-feedback and mass-anchored) final
-// rounding of kw_irow.  Block b: field b / (N / LINES).
+// rounding (bar_add, bar_add_fb).  Block b: field b / (N / LINES).
 template <int M, bool GRP = false>
 __global__ void __launch_bounds__(RowGeo<M>::THREADS, RowGeo<M>::MINB)
 kl_irow(const float* __restrict__ in, float* __restrict__ phi_new, float* __restrict__ psi_new,
@@ -167,7 +345,8 @@ kl_irow(const float* __restrict__ in, float* __restrict__ phi_new, float* __rest
     }
     // psi: the row's increments should sum to sqrt(N) x0; the residual of the FP32 transform and the column residual
     // dc_col are removed, with the mean anchor, in the final rounding (error feedback along each lane's values, the
-    // lanes' remaining errors folded into the row's first value with one dithered rounding: kw_irow)
+    // lanes' remaining errors, summed exactly over the row, folded into the row's first value with one dithered rounding,
+    // so that the stored row sums to its exact value within about one ulp)
     const uint32_t step = (uint32_t)dsc->steps;           // dither key (graph replays read it here)
     float rhi = 0.f, rlo = 0.f;
 #pragma unroll 1
