@@ -29,7 +29,10 @@ __device__ __forceinline__ double at(const T* u, int N, int i, int j) {
 // kDiagRows cells before the block reduction.
 enum { kDiagRows = 8 };
 
-template <typename T>
+// INIT: only the columns that set_state needs (0 - 4 and 13; the others are
+// written as 0).  All fourteen sums of FP64 fields take 1.08 ms at N = 2048,
+// bound by FP64 issue; these six about half.
+template <typename T, bool INIT = false>
 __global__ void __launch_bounds__(256)
 k_diag(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ psi,
        double* __restrict__ part, int N, DiagCoef c) {
@@ -42,10 +45,6 @@ k_diag(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ p
         if (i < N && j < N) {
             const double aC = at(a, N, i, j), aE = at(a, N, i + 1, j), aW = at(a, N, i - 1, j);
             const double aN = at(a, N, i, j + 1), aS = at(a, N, i, j - 1);
-            const double bC = at(b, N, i, j), bE = at(b, N, i + 1, j), bW = at(b, N, i - 1, j);
-            const double bN = at(b, N, i, j + 1), bS = at(b, N, i, j - 1);
-            const double la = (aE + aW + aN + aS - 4 * aC) * c.inv_h2;
-            const double lb = (bE + bW + bN + bS - 4 * bC) * c.inv_h2;
             const double gE = (aE - aC) * c.inv_h, gW = (aC - aW) * c.inv_h, gN = (aN - aC) * c.inv_h, gS = (aC - aS) * c.inv_h;
             const double gbar = 0.5 * (gE * gE + gW * gW) + 0.5 * (gN * gN + gS * gS);
             const double vv = aC * aC - 1.0 - c.beta;
@@ -60,15 +59,21 @@ k_diag(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ p
             v[2] += (1.0 + sp) * fin + (1.0 - sp) * fout;
             v[3] += 0.25 * (aC * aC - 1.0) * (aC * aC - 1.0);
             // interior faces owned by this cell: east (i+1/2) and north (j+1/2)
+            if (i + 1 < N) v[4] += gE * gE;
+            if (j + 1 < N) v[4] += gN * gN;
+            v[13] += ps;
+            if constexpr (INIT) continue;
+            const double bC = at(b, N, i, j), bE = at(b, N, i + 1, j), bW = at(b, N, i - 1, j);
+            const double bN = at(b, N, i, j + 1), bS = at(b, N, i, j - 1);
+            const double la = (aE + aW + aN + aS - 4 * aC) * c.inv_h2;
+            const double lb = (bE + bW + bN + bS - 4 * bC) * c.inv_h2;
             const double cE = 2 * aC - bC, cEe = 2 * aE - bE, cNn = 2 * aN - bN;
             const double dC = aC - bC, dEe = aE - bE, dNn = aN - bN;
             if (i + 1 < N) {
-                v[4] += gE * gE;
                 v[7] += (cEe - cE) * (cEe - cE) * c.inv_h2;
                 v[8] += (dEe - dC) * (dEe - dC) * c.inv_h2;
             }
             if (j + 1 < N) {
-                v[4] += gN * gN;
                 v[7] += (cNn - cE) * (cNn - cE) * c.inv_h2;
                 v[8] += (dNn - dC) * (dNn - dC) * c.inv_h2;
             }
@@ -79,10 +84,17 @@ k_diag(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ p
             const double w = a3 * c.inv_eps - c.eps * la;
             v[11] += w * w;
             v[12] += 0.5 * (1.0 + sp) * fin + 0.5 * (1.0 - sp) * fout;
-            v[13] += ps;
         }
     }
-    block_sum_store<NDIAG, double>(v, part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * NDIAG, sred);
+    double* row = part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * NDIAG;
+    if constexpr (INIT) {
+        double w[6] = {v[0], v[1], v[2], v[3], v[4], v[13]};
+        block_sum_store<6, double>(w, row, sred);      // row[5]: sum of psi, moved by thread 5, which wrote it
+        if (threadIdx.x == 5) { row[13] = row[5]; row[5] = 0.0; }
+        if (threadIdx.x >= 6 && threadIdx.x < 13) row[threadIdx.x] = 0.0;
+    } else {
+        block_sum_store<NDIAG, double>(v, row, sred);
+    }
 }
 
 // ||d||^2 / (lam^2 h^2): sum over interior faces of (D w)^2 / M_psi(A phi*),
@@ -108,13 +120,13 @@ k_dnorm(const T* __restrict__ phn, const T* __restrict__ pho, const T* __restric
     block_sum_store<1, double>(v, part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x), sred);
 }
 
-// The five sums set_state needs for the initial SAVs and the arc length
-// (columns 0-4 of k_diag; the other columns are written as 0) for FP32
-// fields, in the FP32 arithmetic of the step's own stencil (sin/cos by the
-// same polynomials) with double-float accumulation per thread.  k_diag
-// evaluates every cell in FP64, whose issue rate on GB300 makes it a
-// millisecond at N = 2048; this pass costs about as much as reading the two
-// fields.
+// The sums set_state needs for FP32 fields: columns 0 - 4 of k_diag (initial
+// SAVs and arc length) in the FP32 arithmetic of the step's own stencil
+// (sin/cos by the same polynomials) with double-float accumulation per thread,
+// in column 13 the FP64 sum of psi and in column 5 the number of cells with a
+// non-finite value (the other columns are 0).  k_diag evaluates every cell in
+// FP64, whose issue rate on GB300 makes it a millisecond at N = 2048 and 17 ms
+// at N = 8192; this pass costs about as much as reading the two fields.
 struct InitCoefF { float inv_h, eps, inv_eps, beta, gin, gout, psin, psout, bin, bout; };
 
 static __global__ void __launch_bounds__(256)
@@ -123,6 +135,8 @@ k_init_sums_f32(const float* __restrict__ a, const float* __restrict__ psi, doub
     __shared__ double sred[8 * NDIAG];
     const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     float hi[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, lo[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    double psum = 0.0;
+    int bad = 0;
     auto ld = [&](int ii, int jj) {
         ii = ii < 0 ? 0 : (ii >= N ? N - 1 : ii);
         jj = jj < 0 ? 0 : (jj >= N ? N - 1 : jj);
@@ -136,6 +150,8 @@ k_init_sums_f32(const float* __restrict__ a, const float* __restrict__ psi, doub
             const float gbar = 0.5f * (gE * gE + gW * gW) + 0.5f * (gN * gN + gS * gS);
             const float a2 = aC * aC, vv = a2 - 1.0f - c.beta, a3 = aC * (a2 - 1.0f);
             const float ps = psi[(size_t)j * N + i];
+            psum += (double)ps;
+            bad += !(isfinite(aC) && isfinite(ps));
             float sp, cp;
             sincospi_<float>(0.5f * aC, &sp, &cp);
             const float fin = 0.5f * c.gin * (ps - c.psin) * (ps - c.psin) + c.bin;
@@ -151,7 +167,8 @@ k_init_sums_f32(const float* __restrict__ a, const float* __restrict__ psi, doub
     }
     double v[NDIAG];
 #pragma unroll
-    for (int q = 0; q < NDIAG; ++q) v[q] = q < 5 ? (double)hi[q] + (double)lo[q] : 0.0;
+    for (int q = 0; q < NDIAG; ++q)
+        v[q] = q < 5 ? (double)hi[q] + (double)lo[q] : q == 5 ? (double)bad : q == 13 ? psum : 0.0;
     block_sum_store<NDIAG, double>(v, part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * NDIAG, sred);
 }
 
