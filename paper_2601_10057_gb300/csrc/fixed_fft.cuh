@@ -267,6 +267,16 @@ __device__ __forceinline__ double line_double(fx v, int ex, int p = 0) {
 }
 
 // ------------------------------------------------------------------ scaling
+// v 2^-sh rounded to nearest, ties to even (sh < 32).  Ties are frequent at
+// small shifts; rounded up, they moved every value of a line by a quarter of
+// a unit, which the transform gathers in its zero mode (psi's mean drifted by
+// 2e-16 a step at N = 2048).
+__device__ __forceinline__ fx shift_fx(fx a, int sh) {
+    const int odd = (int)__funnelshift_r((unsigned)a.v, (unsigned)(a.v >> 32), sh) & (sh ? 1 : 0);
+    return fx{(a.v + (((1LL << sh) - 1) >> 1) + odd) >> sh};
+}
+__device__ __forceinline__ cx shift_cx(cx a, int sh) { return mk(shift_fx(a.x, sh), shift_fx(a.y, sh)); }
+
 // v: this lane's E values, components below 2^60.6.  Shifts the line right by
 // s0 (returned through ex, which it is added to) so that no lane's first pass
 // can exceed 2^60, and sets sh, the further shift at the twiddles that keeps
@@ -286,9 +296,8 @@ __device__ __forceinline__ void fit_line(cx* v, int slot, LineSm<M>& sm, int& ex
     const int et = ((__float_as_int(tot) >> 23) & 0xff) - 126;          // line sum below 2^et
     sh = max(0, et - 22 - s0);
     if (s0 > 0) {
-        const long long h = 1LL << (s0 - 1);
 #pragma unroll
-        for (int i = 0; i < E; ++i) v[i] = mk(fx{(v[i].x.v + h) >> s0}, fx{(v[i].y.v + h) >> s0});
+        for (int i = 0; i < E; ++i) v[i] = shift_cx(v[i], s0);
     }
     ex += s0 + sh;
 }
@@ -298,7 +307,6 @@ __device__ __forceinline__ CFac ld_fac(const int4* __restrict__ t) {
     const int4 q = __ldg(t);
     return CFac{Fac{q.x, q.y}, Fac{q.z, q.w}};
 }
-__device__ __forceinline__ cx shift_cx(cx a, int sh, long long h) { return mk(fx{(a.x.v + h) >> sh}, fx{(a.y.v + h) >> sh}); }
 
 // The unnormalised DFT of the line (value G n1 + n2 in v[n1] of lane n2);
 // the result lies in buf in natural order, visible to the line's lanes.
@@ -314,13 +322,12 @@ __device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict_
     using Gm = Geo<M>;
     constexpr int A = Gm::A, C = Gm::C, D = Gm::D, G = Gm::G, P = Gm::P;
     DIFX<A, INV, 0>::run(v);
-    const long long h = (1LL << sh) >> 1;
 #pragma unroll
     for (int r = 0; r < A; ++r) {
         const int k1 = wf::bitrev<A>(r);
         cx u = v[r];
         if (k1) u = cmulf<INV>(u, ld_fac(tw + k1 * G + n2));
-        buf[k1 * P + n2] = shift_cx(u, sh, h);
+        buf[k1 * P + n2] = shift_cx(u, sh);
     }
     sync_line<M>(slot);
     if constexpr (D > 1) {

@@ -231,7 +231,7 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
             const ll D = mulv<Q>(split(mulc(ps, k.d2) + k.d1), pf) + k.d0;
             const ll S = mulv<Q>(split(mulc(ps, k.s2) + k.s1), pf) + k.s0;
             out[4 * NN + (size_t)gj * N + gi] = to_double(fx{mulc(mulc(D, split(cp)), k.qpi)}, k.gexp);
-            accZ += (S + mulc(D, spf)) >> 4;
+            accZ += (S + mulc(D, spf) + 8) >> 4;
         }
     }
     __syncthreads();
@@ -288,9 +288,9 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
             out[6 * NN + g] = to_double(fx{lapd}, -Q) * k.g_c;
             out[7 * NN + g] = to_double(fx{(E_.fl - W_.fl) + (N_.fl - S_.fl)}, -Q) * k.l_c;
         }
-        accV += sqrv<Q>(split(vv)) >> 4;
-        accA += mulv<Q>(split(sd2), split(p2)) >> 4;
-        accB += sqrv<Q>(split(p3m)) >> 4;
+        accV += (sqrv<Q>(split(vv)) + 8) >> 4;
+        accA += (mulv<Q>(split(sd2), split(p2)) + 8) >> 4;
+        accB += (sqrv<Q>(split(p3m)) + 8) >> 4;
         S_ = N_;
     }
     // sums with 53 fractional bits over the warp (at most 2^10 cells of size below 2), then FP64
