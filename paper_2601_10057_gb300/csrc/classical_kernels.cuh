@@ -38,7 +38,9 @@ struct PcgScalars {
 constexpr int kClThreads = 256;
 
 // Fixed-order block sum of NV values, then the last block to arrive adds the
-// block sums (in block order) and runs fin(total) on thread 0.
+// block sums (every thread a strided part, then the warps in order: a single
+// chain over 1216 block sums took 39 us, a dependent FP64 addition being 32 ns)
+// and runs fin(total) on thread 0.
 template <int NV, typename Fin>
 __device__ __forceinline__ void cl_reduce(double (&v)[NV], double* __restrict__ red, PcgScalars* pc, Fin fin) {
     __shared__ double sm[kClThreads / 32][NV];
@@ -63,16 +65,27 @@ __device__ __forceinline__ void cl_reduce(double (&v)[NV], double* __restrict__ 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    if (threadIdx.x < NV) {
-        double s = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) s += __ldcg(red + (size_t)b * NV + threadIdx.x);
-        sm[0][threadIdx.x] = s;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] += __ldcg(red + (size_t)b * NV + k);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        double x = v[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) sm[w][k] = x;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double tot[NV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) tot[k] = sm[0][k];
+        for (int k = 0; k < NV; ++k) {
+            double a = sm[0][k], b = sm[1][k];
+            for (int q = 2; q < kClThreads / 32; q += 2) { a += sm[q][k]; b += sm[q + 1][k]; }
+            tot[k] = a + b;
+        }
         fin(tot);
         pc->arrivals = 0u;
     }

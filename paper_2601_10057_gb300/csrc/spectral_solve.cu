@@ -156,7 +156,8 @@ template <typename T> int smooth(ccmsav_solver* s, double eps, double mob, doubl
     T* r = static_cast<T*>(s->rhs);
     const int nb = (int)(((size_t)N * N + 255) / 256 < 4096 ? ((size_t)N * N + 255) / 256 : 4096);
     for (int n = 0; n < nsteps; ++n) {
-        ss::k_smooth_rhs<T><<<nb, 256, 0, s->st>>>(phi, r, N, s->bc, 1.0 / dt, mob / (h * h), 1.0 / eps);
+        ss::k_smooth_rhs<T><<<dim3((N + ss::kSmX - 1) / ss::kSmX, (N + ss::kSmY - 1) / ss::kSmY), 256, 0, s->st>>>(
+            phi, r, N, s->bc, 1.0 / dt, mob / (h * h) / eps);
         ++s->launches;
         int e = solve<T>(s, c, r, phi);
         if (e) return e;
