@@ -200,7 +200,8 @@ public:
     int max_group() const override { return kMaxGroup; }
     template <int MM> void group_launch(const GroupArgs<true>& ga, int n, cudaStream_t s) {
         const int bst = g_st.x, brt = N / wRT, bcol = N / wKC;
-        k_stencil<float, true><<<dim3(bst * n, g_st.y), b_st, stencil_smem_bytes<float>(), s>>>(
+        constexpr StencilTile tile = stencil_tile_of<float>(2 * MM);
+        k_stencil<float, true, tile.x, tile.y><<<dim3(bst * n, g_st.y), b_st, stencil_smem_bytes<float>(tile.x, tile.y), s>>>(
             nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, N, StencilCoef<float>{}, ga, bst);
         kw_rowdct_T<MM, true><<<dim3(brt * n, NF), kWarps * 32, wsm_rt, s>>>(nullptr, nullptr, nullptr, wf::PairTwTab{}, 0,
                                                                          ga, brt);
@@ -375,8 +376,9 @@ public:
         }
         if (cudaMalloc(&bufA, 8 * fb) != cudaSuccess) return CCMSAV_ENOMEM;
         if (cudaMalloc(&bufB, 8 * fb) != cudaSuccess) return CCMSAV_ENOMEM;
-        b_st = dim3(TX, TY);
-        g_st = dim3((N + TX - 1) / TX, (N + TYB - 1) / TYB);
+        const StencilTile tile = stencil_tile_of<T>(N);
+        b_st = dim3(tile.x, TY);
+        g_st = dim3((N + tile.x - 1) / tile.x, (N + tile.y - 1) / tile.y);
         const char* force_block = std::getenv("CCMSAV_FORCE_BLOCK_FFT");   // test switch: block-FFT kernels only
         if (std::is_same<T, double>::value && !(force_block && force_block[0] == '1')) xo = xf::fixed_ops(M);
         nb1 = g_st.x * g_st.y;
@@ -1133,9 +1135,21 @@ public:
                 so.nb1 = nb1x;
             }
         }
-        if (!fixed)
-            k_stencil<T><<<g_st, b_st, stencil_smem_bytes<T>(), st>>>(phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, c,
-                                                                  GroupArgs<false>{}, 0);
+        if (!fixed) {
+            auto launch = [&](auto x, auto y) {
+                constexpr int X = decltype(x)::value, Y = decltype(y)::value;
+                k_stencil<T, false, X, Y><<<g_st, b_st, stencil_smem_bytes<T>(X, Y), st>>>(
+                    phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, c, GroupArgs<false>{}, 0);
+            };
+            using std::integral_constant;
+            if constexpr (std::is_same<T, float>::value) {
+                if (b_st.x == TX) launch(integral_constant<int, TX>(), integral_constant<int, TYB>());
+                else if (N == 512) launch(integral_constant<int, 32>(), integral_constant<int, 16>());
+                else launch(integral_constant<int, 32>(), integral_constant<int, 8>());
+            } else {
+                launch(integral_constant<int, TX>(), integral_constant<int, TYB>());
+            }
+        }
         mark(0);
         if (classical) {
             int r = queue_classical_ch(bdf1);

@@ -407,7 +407,14 @@ __device__ __forceinline__ double bar_add(double a, double b, double du, double 
 // not in the final update, the mismatch was fed back into phi every step
 // (measured: 4.0e-5 max-norm deviation from the FP64 path after 1000 steps
 // at N = 2048 with the rounded phi_bar, 2.6e-6 with phi_bar exact in f0').
+// Smaller tiles on grids that would leave SMs without one (N = 512: 128 tiles
+// of 64 x 32, ten microseconds for one tile's chain of instructions).
 constexpr int TX = 64, TY = 4, TYB = 32;
+struct StencilTile { int x, y; };
+template <typename T> __host__ __device__ constexpr StencilTile stencil_tile_of(int N) {
+    if (!std::is_same<T, float>::value || N > 512 || N < 128) return StencilTile{TX, TYB};
+    return N == 512 ? StencilTile{32, 16} : StencilTile{32, 8};
+}
 template <typename T> constexpr bool kBarLo = std::is_same<T, float>::value;
 
 // One tile of the stencil: CTA column bx, row by of a grid of gx columns; a
@@ -534,37 +541,43 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
     __syncthreads();
     T acc0 = 0, acc1 = 0;
     T mm = (T)1e30;
+    // Each thread takes TYB / TY consecutive rows of a column: a row's centre
+    // and north values and its north face (gradient, phi^2 flux, P flux) are
+    // the next row's south and centre values and south face.
     const int gi = i0 + threadIdx.x;
     const int li = threadIdx.x + 1;
-    for (int jj = threadIdx.y; jj < TYB; jj += TY) {
+    constexpr int RPT = TYB / TY;
+    auto mob = [&](T a) { T s = a * a - (T)1; return (T)1 - c.M0 * s * s; };
+    const int o0 = (threadIdx.y * RPT + 1) * W1 + li;
+    T pS = sph[o0 - W1], pC = sph[o0], dS = sdq[o0 - W1], dC = sdq[o0], lS = slb[o0 - W1], lC = slb[o0], PC = sP[o0];
+    T p2 = pC * pC, gS = (pC - pS) * ih, qS = ((T)0.5 * (p2 + pS * pS)) * gS, fS = mob((T)0.5 * (pC + pS)) * (PC - sP[o0 - W1]);
+#pragma unroll 2
+    for (int jj = threadIdx.y * RPT; jj < (threadIdx.y + 1) * RPT; ++jj) {
         const int lj = jj + 1, gj = j0 + jj;
         const bool inside = gi < N && gj < N;   // tiles overhang grids smaller than the tile
         const size_t g = inside ? (size_t)gj * N + gi : 0;
         const int o = lj * W1 + li;
-        const T pC = sph[o], pE = sph[o + 1], pW = sph[o - 1], pN = sph[o + W1], pS = sph[o - W1];
+        const T pE = sph[o + 1], pW = sph[o - 1], pN = sph[o + W1];
         const T lapp = (((pE - pC) + (pW - pC)) + ((pN - pC) + (pS - pC))) * ih2;
-        const T dC = sdq[o];
-        const T lapd = (((sdq[o + 1] - dC) + (sdq[o - 1] - dC)) + ((sdq[o + W1] - dC) + (sdq[o - W1] - dC))) * ih2;
-        const T lbC = slb[o];
-        const T lap2b = (((slb[o + 1] - lbC) + (slb[o - 1] - lbC)) + ((slb[o + W1] - lbC) + (slb[o - W1] - lbC))) * ih2;
-        const T p2 = pC * pC, p3m = pC * (p2 - (T)1);
+        const T dN = sdq[o + W1];
+        const T lapd = (((sdq[o + 1] - dC) + (sdq[o - 1] - dC)) + ((dN - dC) + (dS - dC))) * ih2;
+        const T lN = slb[o + W1];
+        const T lap2b = (((slb[o + 1] - lC) + (slb[o - 1] - lC)) + ((lN - lC) + (lS - lC))) * ih2;
+        const T p3m = pC * (p2 - (T)1);
         // face gradients (zero on boundary faces through the mirrored ghosts)
-        const T gE = (pE - pC) * ih, gW = (pC - pW) * ih, gN = (pN - pC) * ih, gS = (pC - pS) * ih;
+        const T gE = (pE - pC) * ih, gW = (pC - pW) * ih, gN = (pN - pC) * ih;
         const T gbar = (T)0.5 * (gE * gE + gW * gW) + (T)0.5 * (gN * gN + gS * gS);
-        const T divp2g = (((T)0.5 * (p2 + pE * pE)) * gE - ((T)0.5 * (p2 + pW * pW)) * gW
-                          + ((T)0.5 * (p2 + pN * pN)) * gN - ((T)0.5 * (p2 + pS * pS)) * gS) * ih;
+        const T p2N = pN * pN, qN = ((T)0.5 * (p2 + p2N)) * gN;
+        const T divp2g = (((T)0.5 * (p2 + pE * pE)) * gE - ((T)0.5 * (p2 + pW * pW)) * gW + qN - qS) * ih;
         const T Snum = pC * (p2 - (T)1 - c.beta) * c.inv_eps;
         const T Hv = (T)1.0606601717798212866 * (p3m * c.inv_eps - c.eps * lapp);   // 3 sqrt2 / 4
         const T Qnum = (T)6 * (pC * gbar - divp2g) + p3m * ((T)3 * p2 - (T)1) * c.inv_eps2;
-        const T PC = sP[o];
         // face mobilities M(A phi*) and the flux divergence of P
-        auto mob = [&](T a) { T s = a * a - (T)1; return (T)1 - c.M0 * s * s; };
-        const T mE = mob((T)0.5 * (pC + pE)), mW = mob((T)0.5 * (pC + pW));
-        const T mN = mob((T)0.5 * (pC + pN)), mS = mob((T)0.5 * (pC + pS));
-        const T LP = (mE * (sP[o + 1] - PC) - mW * (PC - sP[o - 1])
-                      + mN * (sP[o + W1] - PC) - mS * (PC - sP[o - W1])) * ih2;
+        const T mE = mob((T)0.5 * (pC + pE)), mW = mob((T)0.5 * (pC + pW)), mN = mob((T)0.5 * (pC + pN));
+        const T PN = sP[o + W1], fN = mN * (PN - PC);
+        const T LP = (mE * (sP[o + 1] - PC) - mW * (PC - sP[o - 1]) + fN - fS) * ih2;
         const T bC = sbar[(lj + 1) * W2 + li + 1];
-        T f0 = c.C2 * lbC - c.C3 * lap2b - c.Mth * lapp - c.betap * bC;
+        T f0 = c.C2 * lC - c.C3 * lap2b - c.Mth * lapp - c.betap * bC;
         if constexpr (kBarLo<T>) f0 = fmaf(-c.betap, slo[(lj + 1) * W2 + li + 1], f0);
         const T g0 = c.lam * lapd;
         if (inside && CCM_OK(7 * NN + g, 8 * NN)) {
@@ -584,6 +597,11 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
             if (gi + 1 < N) mm = min(mm, mE);
             if (gj + 1 < N) mm = min(mm, mN);
         }
+        pS = pC; pC = pN; p2 = p2N;
+        dS = dC; dC = dN;
+        lS = lC; lC = lN;
+        PC = PN;
+        gS = gN; qS = qN; fS = fN;
     }
     const size_t prow_i = (size_t)(by * gx + bx) * NRED1;
     const int lane = tid & 31, wp = tid >> 5;
@@ -635,8 +653,8 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
     }
 }
 
-template <typename T, bool GRP = false>
-__global__ void __launch_bounds__(TX * TY)
+template <typename T, bool GRP = false, int X = TX, int YB = TYB>
+__global__ void __launch_bounds__(X * TY)
 k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
           const T* __restrict__ psn, const T* __restrict__ pso,
           T* __restrict__ out, double* __restrict__ part, int N, StencilCoef<T> c,
@@ -651,11 +669,11 @@ k_stencil(const T* __restrict__ phn, const T* __restrict__ pho,
         const BatchArgs& A = ga.a[sim];
         phn = A.phn; pho = A.pho; psn = A.psn; pso = A.pso; out = A.bufA; part = A.part1; c = A.c;
     }
-    stencil_tile<T, TX, TY, TYB>(smraw, phn, pho, psn, pso, out, part, N, c, bx, blockIdx.y, gx);
+    stencil_tile<T, X, TY, YB>(smraw, phn, pho, psn, pso, out, part, N, c, bx, blockIdx.y, gx);
 }
 
-template <typename T> __host__ __device__ constexpr size_t stencil_smem_bytes() {
-    return ((size_t)(kBarLo<T> ? 2 : 1) * (TYB + 4) * (TX + 4) + 4 * (size_t)(TYB + 2) * (TX + 2)) * sizeof(T);
+template <typename T> __host__ __device__ constexpr size_t stencil_smem_bytes(int X = TX, int YB = TYB) {
+    return ((size_t)(kBarLo<T> ? 2 : 1) * (YB + 4) * (X + 4) + 4 * (size_t)(YB + 2) * (X + 2)) * sizeof(T);
 }
 
 // The pair k (0 <= k <= M/2) of the line transforms touches the modes
@@ -1036,15 +1054,16 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
         const double PL = h2 * nK * nK * Gm[16];
         a = j == 3 ? -PL : j == 4 ? 1.0 - PL : j == 5 ? h2 * nK * Gm[15] + xb[3] * PL : 0.0;
     }
-#pragma unroll
+    // rolled: the kernel runs once per step and fetches its instructions anew
+#pragma unroll 1
     for (int k = 0; k < 5; ++k) {
         const unsigned long long mag = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
         unsigned long long best = __shfl_sync(FULL, mag, 6 * k + k);
         int piv = k;
 #pragma unroll
-        for (int rr2 = k + 1; rr2 < 5; ++rr2) {
+        for (int rr2 = 1; rr2 < 5; ++rr2) {
             const unsigned long long m = __shfl_sync(FULL, mag, 6 * rr2 + k);
-            if (m > best) { best = m; piv = rr2; }
+            if (rr2 > k && m > best) { best = m; piv = rr2; }
         }
         if (best == 0ull) {
             if (lane == 0) sc->status = -5;

@@ -19,10 +19,10 @@ namespace lf {
 using cf = cplx<float>;
 
 template <int M> struct Shape;
-template <> struct Shape<32>   { static constexpr int A = 8,  C = 4,  D = 1;  };
-template <> struct Shape<64>   { static constexpr int A = 8,  C = 8,  D = 1;  };
-template <> struct Shape<128>  { static constexpr int A = 16, C = 8,  D = 1;  };
-template <> struct Shape<256>  { static constexpr int A = 16, C = 16, D = 1;  };
+template <> struct Shape<32>   { static constexpr int A = 4,  C = 4,  D = 2;  };
+template <> struct Shape<64>   { static constexpr int A = 4,  C = 4,  D = 4;  };
+template <> struct Shape<128>  { static constexpr int A = 8,  C = 4,  D = 4;  };
+template <> struct Shape<256>  { static constexpr int A = 8,  C = 4,  D = 8;  };
 template <> struct Shape<512>  { static constexpr int A = 16, C = 4,  D = 8;  };
 template <> struct Shape<1024> { static constexpr int A = 16, C = 8,  D = 8;  };
 template <> struct Shape<2048> { static constexpr int A = 16, C = 16, D = 8;  };
