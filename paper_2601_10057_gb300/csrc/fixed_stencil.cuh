@@ -154,6 +154,7 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
     ll* slb = sdq + H1 * W1;                            // h^2 Lap 3 phi_bar / 8
     __shared__ ll ssum[NW][4];
     __shared__ ll smin[NW];
+    __shared__ float stiny[NW][3];
     const int bx = blockIdx.x, by = blockIdx.y, i0 = bx * TX, j0 = by * TYB;
     const int tid = threadIdx.y * TX + threadIdx.x;
     const size_t NN = (size_t)N * N;
@@ -238,6 +239,7 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
     const int gi = i0 + threadIdx.x, li = threadIdx.x + 1, lane = tid & 31;
     const int r0 = threadIdx.y * RPT;
     ll accV = 0, accA = 0, accB = 0, mmin = 1LL << 62;
+    float tiny[3] = {0.f, 0.f, 0.f};                    // the same three sums times 2^120
     ll mN;
     Face S_;
     {
@@ -288,9 +290,19 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
             out[6 * NN + g] = to_double(fx{lapd}, -Q) * k.g_c;
             out[7 * NN + g] = to_double(fx{(E_.fl - W_.fl) + (N_.fl - S_.fl)}, -Q) * k.l_c;
         }
-        accV += (sqrv<Q>(split(vv)) + 8) >> 4;
-        accA += (mulv<Q>(split(sd2), split(p2)) + 8) >> 4;
-        accB += (sqrv<Q>(split(p3m)) + 8) >> 4;
+        // Away from the interfaces the three terms are below the last bit; there they are added in FP32, so that
+        // a state without any interface (phi within 1e-9 of +-1 everywhere) still has its radicands.
+        if (__all_sync(0xffffffffu, !outside(vv, hi_of(0x1p-14)) && (sd2 >> 32) == 0)) {
+            const float fv = __ll2float_rn(vv), f3 = __ll2float_rn(p3m), fp = __ll2float_rn(pC) * 0x1p-60f;
+            const float fe = __ll2float_rn(E_.d), fw = __ll2float_rn(W_.d), fn = __ll2float_rn(N_.d), fs = __ll2float_rn(S_.d);
+            tiny[0] = fmaf(fv, fv, tiny[0]);
+            tiny[1] = fmaf(fp * fp, (fe * fe + fw * fw) + (fn * fn + fs * fs), tiny[1]);
+            tiny[2] = fmaf(f3, f3, tiny[2]);
+        } else {
+            accV += (sqrv<Q>(split(vv)) + 8) >> 4;
+            accA += (mulv<Q>(split(sd2), split(p2)) + 8) >> 4;
+            accB += (sqrv<Q>(split(p3m)) + 8) >> 4;
+        }
         S_ = N_;
     }
     // sums with 53 fractional bits over the warp (at most 2^10 cells of size below 2), then FP64
@@ -301,6 +313,11 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (lane == 0) ssum[tid >> 5][q] = x;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float x = warp_sum(tiny[q]);
+        if (lane == 0) stiny[tid >> 5][q] = x;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mmin = min(mmin, __shfl_xor_sync(0xffffffffu, mmin, o));
@@ -314,6 +331,7 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
         auto sum = [&](int q) {
             double s = 0.0;
             for (int w = 0; w < NW; ++w) s += to_double(fx{ssum[w][q]}, -53);
+            for (int w = 0; q < 3 && w < NW; ++w) s += (double)stiny[w][q] * 0x1p-120;
             return s;
         };
         if (tid == 0) r = sum(0) * k.wV;

@@ -97,3 +97,25 @@ def test_periodic_fp32_against_fp64(N):
     want = _solve(f.astype(np.float32).astype(np.float64), coef, "periodic")
     got = _solve(f, coef, "periodic", "fp32")
     assert np.abs(got - want).max() <= 2e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("amp", [1e-12, 1e-9, 1e-4])
+def test_state_without_an_interface(amp, monkeypatch):
+    """phi within amp of 1 everywhere: the SAV radicands are sums of terms of
+    size amp^2, far below the fixed-point fields' last bit for the smaller
+    ones.  The run goes on as on the block path, within 1e-12 of the largest value."""
+    N = 128
+    p = I.growth_params(eps=8.0 / N, dt=1e-6, L=1.0)
+    x = (np.arange(N) + 0.5) / N
+    phi = 1.0 - amp * (1.5 + np.cos(np.pi * x)[None, :] * np.cos(2 * np.pi * x)[:, None])
+    psi = 0.5 + 0.1 * np.cos(np.pi * x)[:, None] * np.ones(N)[None, :]
+    out = []
+    for block in ("0", "1"):
+        monkeypatch.setenv("CCMSAV_FORCE_BLOCK_FFT", block)
+        sim = cc.Simulation(p, N, precision="fp64")
+        sim.set_state(phi, psi)
+        sim.step(3)
+        out.append(sim.state())
+        sim.close()
+    for a, b in zip(*out):
+        assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
