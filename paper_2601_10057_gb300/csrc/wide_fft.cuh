@@ -208,9 +208,9 @@ __device__ __forceinline__ void write_modes(const cf* bufs, float* __restrict__ 
         put(slot_mode<M>(i2, 1), r4, s2[0].y, s2[1].y, s2[2].y, s2[3].y);
     }
 }
-// The samples of the CTA's lines to dst[y N + r].
+// The samples of the CTA's lines to dst[y N + r] (o0, lim as above).
 template <int M, int LINES>
-__device__ __forceinline__ void write_samples(const cf* bufs, float* __restrict__ dst) {
+__device__ __forceinline__ void write_samples(const cf* bufs, float* __restrict__ dst, size_t o0, size_t lim) {
     using Gm = Geo<M>;
     constexpr int N = Gm::N, R4 = LINES / 4;
 #pragma unroll 1
@@ -223,6 +223,7 @@ __device__ __forceinline__ void write_samples(const cf* bufs, float* __restrict_
             a[r] = z[m];
             b[r] = z[M - 1 - m];
         }
+        if (!CCM_OKW(o0 + (size_t)(4 * m + 3) * N + 4 * r4, 4, lim)) continue;
         float* d = dst + (size_t)(4 * m) * N + 4 * r4;
         *reinterpret_cast<float4*>(d) = make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
         *reinterpret_cast<float4*>(d + N) = make_float4(b[0].y, b[1].y, b[2].y, b[3].y);
@@ -262,7 +263,8 @@ __device__ __forceinline__ void write_modes_pair(cf* bufs, float* __restrict__ d
     }
     cl.sync();                                         // the other CTA may still read these lines
 }
-template <int M> __device__ __forceinline__ void write_samples_pair(cf* bufs, float* __restrict__ dst) {
+template <int M>
+__device__ __forceinline__ void write_samples_pair(cf* bufs, float* __restrict__ dst, size_t o0, size_t lim) {
     using Gm = Geo<M>;
     constexpr int N = Gm::N;
     auto cl = cooperative_groups::this_cluster();
@@ -279,6 +281,7 @@ template <int M> __device__ __forceinline__ void write_samples_pair(cf* bufs, fl
             a[r] = z[m];
             b[r] = z[M - 1 - m];
         }
+        if (!CCM_OKW(o0 + (size_t)(4 * m + 3) * N + 4 * r4, 4, lim)) continue;
         float* d = dst + (size_t)(4 * m) * N + 4 * r4;
         *reinterpret_cast<float4*>(d) = make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
         *reinterpret_cast<float4*>(d + N) = make_float4(b[0].y, b[1].y, b[2].y, b[3].y);

@@ -99,7 +99,7 @@ kl_col_solve(const float* __restrict__ in, float* __restrict__ out, const float2
     sync_line<M>(slot);
     inverse_line<M>(buf, tw, n2, slot);
     __syncthreads();
-    write_samples<M, Gm::LINES>(bufs, out + blockIdx.y * fstride + x0);
+    write_samples<M, Gm::LINES>(bufs, out + blockIdx.y * fstride + x0, x0, (size_t)N * N);
 }
 
 // Inverse DCT along x of LINES rows (in place allowed).  DST: times (-1)^(i+j).

@@ -268,10 +268,10 @@ kl_comb(const float* __restrict__ spec, float* __restrict__ out, const float2* _
         if (slot == 0 && n2 == 0) dsc->dc_col = dsum;
     }
     if constexpr (Gm::LINES == 4) {                       // comb_cluster: two CTAs
-        write_samples_pair<M>(bufs, out + f * NN + (size_t)(x0 & ~7));
+        write_samples_pair<M>(bufs, out + f * NN + (size_t)(x0 & ~7), f * NN + (size_t)(x0 & ~7), 2 * NN);
     } else {
         __syncthreads();
-        write_samples<M, Gm::LINES>(bufs, out + f * NN + x0);
+        write_samples<M, Gm::LINES>(bufs, out + f * NN + x0, f * NN + x0, 2 * NN);
     }
 }
 template <int M> __host__ __device__ constexpr int comb_cluster() { return Geo<M>::LINES == 4 ? 2 : 1; }
