@@ -417,6 +417,15 @@ template <typename T> __host__ __device__ constexpr StencilTile stencil_tile_of(
 }
 template <typename T> constexpr bool kBarLo = std::is_same<T, float>::value;
 
+// Products and multiply-adds as written: sums of two products and products
+// carried to the next row may be contracted in more than one way, and the
+// kernel for one simulation and the one for a group of them (and the
+// index-checked build of each) have to give the same bits.
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
 // One tile of the stencil: CTA column bx, row by of a grid of gx columns; a
 // CTA of TX x TY threads, smraw stencil_smem_bytes of shared memory.
 template <typename T, int TX, int TY, int TYB>
@@ -528,14 +537,14 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
         const T ph = sph[q], ps = sps[q];
         T sp, cp;
         sincospi_<T>((T)0.5 * ph, &sp, &cp);
-        sP[q] = (T)0.5 * (c.gin * ((T)1 + sp) * (ps - c.psin) + c.gout * ((T)1 - sp) * (ps - c.psout));
+        sP[q] = (T)0.5 * fma_(c.gin * ((T)1 + sp), ps - c.psin, mul_(c.gout * ((T)1 - sp), ps - c.psout));
         const int gi = i0 + li1 - 1, gj = j0 + lj1 - 1;
         if (lj1 >= 1 && lj1 <= TYB && li1 >= 1 && li1 <= TX && gi < N && gj < N &&
             CCM_OK(4 * NN + (size_t)gj * N + gi, 8 * NN)) {
             const T fin = c.hgin * (ps - c.psin) * (ps - c.psin) + c.bin;
             const T fout = c.hgout * (ps - c.psout) * (ps - c.psout) + c.bout;
             out[4 * NN + (size_t)gj * N + gi] = (T)0.5 * ((T)1.5707963267948966192 * cp) * (fin - fout);
-            acc2 += ((T)1 + sp) * fin + ((T)1 - sp) * fout;
+            acc2 += fma_((T)1 + sp, fin, mul_((T)1 - sp, fout));
         }
     }
     __syncthreads();
@@ -547,10 +556,11 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
     const int gi = i0 + threadIdx.x;
     const int li = threadIdx.x + 1;
     constexpr int RPT = TYB / TY;
-    auto mob = [&](T a) { T s = a * a - (T)1; return (T)1 - c.M0 * s * s; };
+    auto mob = [&](T a) { T s = fma_(a, a, (T)-1); return fma_(-c.M0 * s, s, (T)1); };
     const int o0 = (threadIdx.y * RPT + 1) * W1 + li;
     T pS = sph[o0 - W1], pC = sph[o0], dS = sdq[o0 - W1], dC = sdq[o0], lS = slb[o0 - W1], lC = slb[o0], PC = sP[o0];
-    T p2 = pC * pC, gS = (pC - pS) * ih, qS = ((T)0.5 * (p2 + pS * pS)) * gS, fS = mob((T)0.5 * (pC + pS)) * (PC - sP[o0 - W1]);
+    T p2 = mul_(pC, pC), gS = mul_(pC - pS, ih), qS = mul_((T)0.5 * (p2 + mul_(pS, pS)), gS);
+    T fS = mul_(mob((T)0.5 * (pC + pS)), PC - sP[o0 - W1]);
 #pragma unroll 2
     for (int jj = threadIdx.y * RPT; jj < (threadIdx.y + 1) * RPT; ++jj) {
         const int lj = jj + 1, gj = j0 + jj;
@@ -565,19 +575,19 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
         const T lap2b = (((slb[o + 1] - lC) + (slb[o - 1] - lC)) + ((lN - lC) + (lS - lC))) * ih2;
         const T p3m = pC * (p2 - (T)1);
         // face gradients (zero on boundary faces through the mirrored ghosts)
-        const T gE = (pE - pC) * ih, gW = (pC - pW) * ih, gN = (pN - pC) * ih;
-        const T gbar = (T)0.5 * (gE * gE + gW * gW) + (T)0.5 * (gN * gN + gS * gS);
-        const T p2N = pN * pN, qN = ((T)0.5 * (p2 + p2N)) * gN;
-        const T divp2g = (((T)0.5 * (p2 + pE * pE)) * gE - ((T)0.5 * (p2 + pW * pW)) * gW + qN - qS) * ih;
+        const T gE = mul_(pE - pC, ih), gW = mul_(pC - pW, ih), gN = mul_(pN - pC, ih);
+        const T gbar = (T)0.5 * fma_(gE, gE, mul_(gW, gW)) + (T)0.5 * fma_(gN, gN, mul_(gS, gS));
+        const T p2N = mul_(pN, pN), qN = mul_((T)0.5 * (p2 + p2N), gN);
+        const T divp2g = mul_(fma_((T)0.5 * fma_(pE, pE, p2), gE, -mul_((T)0.5 * fma_(pW, pW, p2), gW)) + (qN - qS), ih);
         const T Snum = pC * (p2 - (T)1 - c.beta) * c.inv_eps;
-        const T Hv = (T)1.0606601717798212866 * (p3m * c.inv_eps - c.eps * lapp);   // 3 sqrt2 / 4
-        const T Qnum = (T)6 * (pC * gbar - divp2g) + p3m * ((T)3 * p2 - (T)1) * c.inv_eps2;
+        const T Hv = (T)1.0606601717798212866 * fma_(p3m, c.inv_eps, -mul_(c.eps, lapp));   // 3 sqrt2 / 4
+        const T Qnum = fma_((T)6, fma_(pC, gbar, -divp2g), mul_(p3m * fma_((T)3, p2, (T)-1), c.inv_eps2));
         // face mobilities M(A phi*) and the flux divergence of P
         const T mE = mob((T)0.5 * (pC + pE)), mW = mob((T)0.5 * (pC + pW)), mN = mob((T)0.5 * (pC + pN));
-        const T PN = sP[o + W1], fN = mN * (PN - PC);
-        const T LP = (mE * (sP[o + 1] - PC) - mW * (PC - sP[o - 1]) + fN - fS) * ih2;
+        const T PN = sP[o + W1], fN = mul_(mN, PN - PC);
+        const T LP = (fma_(mE, sP[o + 1] - PC, -mul_(mW, PC - sP[o - 1])) + (fN - fS)) * ih2;
         const T bC = sbar[(lj + 1) * W2 + li + 1];
-        T f0 = c.C2 * lC - c.C3 * lap2b - c.Mth * lapp - c.betap * bC;
+        T f0 = fma_(-c.betap, bC, fma_(-c.Mth, lapp, fma_(c.C2, lC, -mul_(c.C3, lap2b))));
         if constexpr (kBarLo<T>) f0 = fmaf(-c.betap, slo[(lj + 1) * W2 + li + 1], f0);
         const T g0 = c.lam * lapd;
         if (inside && CCM_OK(7 * NN + g, 8 * NN)) {
@@ -589,8 +599,8 @@ stencil_tile(unsigned char* smraw, const T* __restrict__ phn, const T* __restric
             out[6 * NN + g] = g0;
             out[7 * NN + g] = LP;
             const T vv = p2 - (T)1 - c.beta;
-            acc0 += vv * vv * c.quarter_inv_eps;
-            acc1 += (T)6 * p2 * gbar + p3m * p3m * c.inv_eps2;
+            acc0 = fma_(mul_(vv, vv), c.quarter_inv_eps, acc0);
+            acc1 += fma_((T)6 * p2, gbar, mul_(mul_(p3m, p3m), c.inv_eps2));
             // minimum face mobility over interior faces: each interior face
             // is the east or north face of exactly one cell (boundary faces
             // carry no flux)
