@@ -119,3 +119,22 @@ def test_state_without_an_interface(amp, monkeypatch):
         sim.close()
     for a, b in zip(*out):
         assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("wl,N", [("ellipse_shrink", 64), ("three_vesicles", 1024), ("three_vesicles", 4096)])
+def test_classical_fp32_preconditioner_lines(wl, N):
+    """FP32 conjugate gradients to 1e-6, preconditioned on the wide lines (the
+    shortest, a middle and the clustered ones), against FP64 after 2 steps: 2e-5, the CG
+    tolerance and the FP32 fields' rounding over the steps."""
+    w = I.workload(wl, N=N, dt=1e-6)
+    out = []
+    for prec, tol in (("fp64", 1e-10), ("fp32", 1e-6)):
+        sim = cc.Simulation(w.params, N, precision=prec, classical=True)
+        sim.set_pcg(tol, 400)
+        sim.set_state(w.phi0, w.psi0)
+        sim.step(2)
+        out.append(sim.state())
+        assert 1 <= sim.pcg_stats()[0] < 400
+        sim.close()
+    for a, b in zip(*out):
+        assert np.abs(a - b).max() <= 2e-5 * np.abs(a).max()
