@@ -11,11 +11,8 @@
 //      written to the buffer in natural order.
 // One smem round trip per stage pair instead of one per radix-8 stage, no
 // block barriers (only __syncwarp), and 32 independent values per lane.
-// Supported lines: M in {64, ..., 4096} (N = 2M in 128 .. 8192); the shapes
-// E x G are listed below (Shape).  A group of G = 32 W lanes (W = 2, 4)
-// spans W warps: its lanes synchronise through a named barrier of the line
-// (id 1 + line slot, G threads) instead of __syncwarp.  Shapes with E < G
-// take fourstep_split for steps 3-4.
+// Lines of the forward passes: M in {64, ..., 2048} (N = 2M in 128 .. 4096),
+// 32 / G lines per warp; the shapes E x G are listed below (Shape).
 #pragma once
 #include <type_traits>
 #include "dct_device.cuh"
@@ -184,24 +181,18 @@ template <> struct Shape<512>  { static constexpr int E = 32, G = 16; };
 template <> struct Shape<1024> { static constexpr int E = 32, G = 32; };
 template <> struct Shape<2048> { static constexpr int E = 64, G = 32; };
 
-// Lane n2 of its line's group and the line's slot in the CTA: G <= 32 puts
-// 32 / G lines in a warp; G = 64, 128 spreads a line over 2, 4 consecutive
-// warps.
+// Lane n2 of its line's group and the line's slot in the CTA.
 template <int M> __device__ __forceinline__ void lane_geo(int& n2, int& slot) {
     constexpr int G = Shape<M>::G;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if constexpr (G <= 32) {
-        n2 = lane % G;
-        slot = warp * (32 / G) + lane / G;
-    } else {
-        n2 = lane + 32 * (warp % (G / 32));
-        slot = warp / (G / 32);
-    }
+    n2 = lane % G;
+    slot = warp * (32 / G) + lane / G;
 }
 
 // Barrier of one line's lane group: the warp's own lanes for G <= 32, the
 // warps of the line (named barrier 1 + slot; every one of their G threads
-// arrives) for G = 64, 128.
+// arrives) for larger groups (the wide and the
+// fixed-point lines).
 template <int G> __device__ __forceinline__ void line_sync(int slot) {
     if constexpr (G <= 32) {
         __syncwarp();
@@ -235,31 +226,22 @@ template <int M, bool SWZ> __device__ __forceinline__ int tpos(int R, int c) {
 
 // Steps 1-4.  v: this lane's E values in four-step order.  buf: this line's
 // buffer.  On return buf[k] = Z[k], k = 0..M-1 (visible to the warp).
-template <typename T, int M, bool INV, bool SWZ = false>
-__device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>* __restrict__ tw2, int n2, int slot) {
+template <typename T, int M, bool SWZ>
+__device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>* __restrict__ tw2, int n2) {
     constexpr int E = Shape<M>::E, G = Shape<M>::G, J = E / G;
-    DIF<T, E, INV, 0>::run(v);
-    if constexpr (!INV) {
-        // twiddles W_M^{n2 k1}: k1 = bitrev(r) is below E/2 for even r; for odd
-        // r it is the even partner's + E/2, so W^{n2 k1} = W^{n2 k1'} W^{(E/2) n2}
-        // (half the table loads; measured faster in the forward kernels, which
-        // are shared-memory/load bound, slower in the inverse ones)
-        const cplx<T> wh = tw2[(E / 2) * G + n2];
+    DIF<T, E, false, 0>::run(v);
+    // twiddles W_M^{n2 k1}: k1 = bitrev(r) is below E/2 for even r; for odd
+    // r it is the even partner's + E/2, so W^{n2 k1} = W^{n2 k1'} W^{(E/2) n2}
+    // (half the table loads: the kernels are shared-memory and load bound)
+    const cplx<T> wh = tw2[(E / 2) * G + n2];
 #pragma unroll
-        for (int r = 0; r < E; r += 2) {
-            const int k1 = bitrev<E>(r);
-            const cplx<T> w = tw2[k1 * G + n2];
-            buf[tpos<M, SWZ>(k1, n2)] = cmul(v[r], w);
-            buf[tpos<M, SWZ>(k1 + E / 2, n2)] = cmul(v[r + 1], cmul(w, wh));
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int k1 = bitrev<E>(r);
-            buf[tpos<M, SWZ>(k1, n2)] = cmulc(v[r], tw2[k1 * G + n2]);
-        }
+    for (int r = 0; r < E; r += 2) {
+        const int k1 = bitrev<E>(r);
+        const cplx<T> w = tw2[k1 * G + n2];
+        buf[tpos<M, SWZ>(k1, n2)] = cmul(v[r], w);
+        buf[tpos<M, SWZ>(k1 + E / 2, n2)] = cmul(v[r + 1], cmul(w, wh));
     }
-    line_sync<G>(slot);
+    __syncwarp();
     if constexpr (SWZ && wide_reads<M>() && std::is_same<T, float>::value) {
 #pragma unroll
         for (int j = 0; j < J; ++j)
@@ -275,17 +257,17 @@ __device__ __forceinline__ void fourstep(cplx<T>* v, cplx<T>* buf, const cplx<T>
 #pragma unroll
             for (int m = 0; m < G; ++m) v[j * G + m] = buf[tpos<M, SWZ>(n2 * J + j, m)];
     }
-    line_sync<G>(slot);
+    __syncwarp();
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        if (j == 0) DIF<T, G, INV, 0>::run(v);
-        else DIF<T, G, INV, G>::run(v);
+        if (j == 0) DIF<T, G, false, 0>::run(v);
+        else DIF<T, G, false, G>::run(v);
     }
 #pragma unroll
     for (int j = 0; j < J; ++j)
 #pragma unroll
         for (int r = 0; r < G; ++r) buf[(n2 * J + j) + E * bitrev<G>(r)] = v[j * G + r];
-    line_sync<G>(slot);
+    __syncwarp();
 }
 
 // Forward pack from a real line x in global memory (16-byte aligned):
@@ -298,15 +280,9 @@ __device__ __forceinline__ void pack_fwd_global(const float* __restrict__ x, cpl
     for (int n1 = 0; n1 < E / 2; ++n1) {
         const float4 q = __ldcg(reinterpret_cast<const float4*>(x) + (G * n1 + n2));   // L2 only: keeps L1 for the tables
         v[n1] = mk(q.x, q.z);
-        if constexpr (G <= 32) {
-            const float ox = __shfl_xor_sync(0xffffffffu, q.w, G - 1);
-            const float oy = __shfl_xor_sync(0xffffffffu, q.y, G - 1);
-            v[E - 1 - n1] = mk(ox, oy);
-        } else {
-            // the partner lane G - 1 - n2 sits in the other warp: load its quad too
-            const float4 p = __ldg(reinterpret_cast<const float4*>(x) + (G * n1 + (G - 1 - n2)));
-            v[E - 1 - n1] = mk(p.w, p.y);
-        }
+        const float ox = __shfl_xor_sync(0xffffffffu, q.w, G - 1);
+        const float oy = __shfl_xor_sync(0xffffffffu, q.y, G - 1);
+        v[E - 1 - n1] = mk(ox, oy);
     }
 }
 

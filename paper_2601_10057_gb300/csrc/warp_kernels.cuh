@@ -1,5 +1,5 @@
 // warp_kernels.cuh -- FP32 forward passes built on the warp-level line FFT
-// (row pass N = 2M in 128 .. 4096, column pass the same).  Same data flow as the block-FFT kernels of
+// (N = 2M in 128 .. 4096).  Same data flow as the block-FFT kernels of
 // step_kernels.cuh:
 //   kw_rowdct_T    forward DCT-II along x, transposed write (RT rows per CTA)
 //   kw_coldct_gram forward DCT-II along y of the 8 fields of KC spectral rows,
@@ -15,33 +15,6 @@
 namespace ccm {
 
 constexpr int kWarps = 8;
-
-// Exact (double-float) sum over the G lanes of one line: inside the warp for
-// G <= 32; for G = 32 W each of the W warps sums its part, the parts go
-// through `sm` (W float2 per line slot) and every warp adds them in the same
-// order.
-template <int G>
-__device__ __forceinline__ double line_sum_exact(float hi, float lo, int slot, float2* sm) {
-    if constexpr (G <= 32) {
-        return group_sum_exact<G>(hi, lo);
-    } else {
-        constexpr int W = G / 32;
-        const float2 h = group_sum_df<32>(hi, lo);
-        const int part = (threadIdx.x >> 5) % W;
-        if ((threadIdx.x & 31) == 0) sm[W * slot + part] = h;
-        wf::line_sync<G>(slot);
-        float2 a = sm[W * slot];
-#pragma unroll
-        for (int w = 1; w < W; ++w) {
-            const float2 b = sm[W * slot + w];
-            df_add2(a.x, a.y, b.x, b.y);
-        }
-        wf::line_sync<G>(slot);        // the slots may be written again by a later call
-        return (double)a.x + (double)a.y;
-    }
-}
-
-
 
 // Pair-ordered spectra of the warp path: for each spectral row kx and each
 // of the 7 stored fields (f0', S, H, Q, K, g0', L_P), the float4 of modes
@@ -101,7 +74,7 @@ kw_rowdct_T(const float* __restrict__ in, float* __restrict__ out,
     {
         cplx<float> v[E];
         wf::pack_fwd_global<M>(in + CCM_IXW(f * NN + (size_t)(y0 + slot) * N, N, NF * NN), v, n2);
-        wf::fourstep<float, M, false, true>(v, buf, tw2, n2, slot);
+        wf::fourstep<float, M, true>(v, buf, tw2, n2);
     }
     __syncthreads();
     // DCT post-process fused into the transposed write.  Item (r4, k) takes
@@ -183,7 +156,7 @@ kw_coldct_gram(const float* __restrict__ in, float* __restrict__ spec, double* _
     {
         cplx<float> v[E];
         wf::pack_fwd_global<M>(in + CCM_IXW(f * NN + (size_t)(kx0 + kc) * N, N, NF * NN), v, n2);
-        wf::fourstep<float, M, false, true>(v, bufs + (size_t)slot * Gm::BUF, tw2, n2, slot);
+        wf::fourstep<float, M, true>(v, bufs + (size_t)slot * Gm::BUF, tw2, n2);
     }
     __syncthreads();
     float acc[NRED2];

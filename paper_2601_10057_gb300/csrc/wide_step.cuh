@@ -14,6 +14,31 @@
 namespace ccm {
 namespace lf {
 
+// Exact (double-float) sum over the G lanes of one line: inside the warp for
+// G <= 32; for G = 32 W each of the W warps sums its part, the parts go
+// through `sm` (W float2 per line slot) and every warp adds them in the same
+// order.
+template <int G>
+__device__ __forceinline__ double line_sum_exact(float hi, float lo, int slot, float2* sm) {
+    if constexpr (G <= 32) {
+        return group_sum_exact<G>(hi, lo);
+    } else {
+        constexpr int W = G / 32;
+        const float2 h = group_sum_df<32>(hi, lo);
+        const int part = (threadIdx.x >> 5) % W;
+        if ((threadIdx.x & 31) == 0) sm[W * slot + part] = h;
+        wf::line_sync<G>(slot);
+        float2 a = sm[W * slot];
+#pragma unroll
+        for (int w = 1; w < W; ++w) {
+            const float2 b = sm[W * slot + w];
+            df_add2(a.x, a.y, b.x, b.y);
+        }
+        wf::line_sync<G>(slot);        // the slots may be written again by a later call
+        return (double)a.x + (double)a.y;
+    }
+}
+
 // ------------------------------------------------------------------ forward rows
 // 4096-point lines: clusters of two CTAs of four rows each (write_modes_pair).
 // Shorter lines take the warp-level kernels of warp_kernels.cuh, which move a
