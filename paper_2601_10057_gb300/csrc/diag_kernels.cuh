@@ -113,8 +113,8 @@ k_dnorm(const T* __restrict__ phn, const T* __restrict__ pho, const T* __restric
             auto w = [&](int ii, int jj) { return at(psnew, N, ii, jj) - (2.0 * at(psn, N, ii, jj) - at(pso, N, ii, jj)); };
             const double pC = ph(i, j), wC = w(i, j);
             auto mob = [&](double x) { double s = x * x - 1.0; return 1.0 - M0 * s * s; };
-            if (i + 1 < N) { double d = w(i + 1, j) - wC; v[0] = fma(d * d, rcp_(mob(0.5 * (pC + ph(i + 1, j)))), v[0]); }
-            if (j + 1 < N) { double d = w(i, j + 1) - wC; v[0] = fma(d * d, rcp_(mob(0.5 * (pC + ph(i, j + 1)))), v[0]); }
+            if (i + 1 < N) { double d = w(i + 1, j) - wC; v[0] += d * d / mob(0.5 * (pC + ph(i + 1, j))); }
+            if (j + 1 < N) { double d = w(i, j + 1) - wC; v[0] += d * d / mob(0.5 * (pC + ph(i, j + 1))); }
         }
     }
     block_sum_store<1, double>(v, part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x), sred);

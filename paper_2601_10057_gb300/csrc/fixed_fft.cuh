@@ -525,18 +525,5 @@ template <int M> __device__ __forceinline__ vec4<double> unpack_item(const cx* z
     return {line_double(a.x, ex), line_double(b.y, ex), line_double(a.y, ex), line_double(b.x, ex)};
 }
 
-// 1 / d for d > 0 well inside the FP64 range: hardware seed (20 bits or more)
-// and one cubically convergent Newton step (e = 1 - d r, r (1 + e + e^2)),
-// error below 2 units in the last place; plain division otherwise.
-__device__ __forceinline__ double recip(double d) {
-    const unsigned h = (unsigned)__double2hiint(d);
-    if (h - 0x02000000u >= 0x7b000000u) return 1.0 / d;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    e = fma(e, e, e);
-    return fma(r, e, r);
-}
-
 }  // namespace xf
 }  // namespace ccm

@@ -226,8 +226,8 @@ __global__ void kx_weights(const double* __restrict__ ev, SpecCoef sc, double* _
     constexpr size_t N = 2 * M;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < N * N; q += (size_t)gridDim.x * blockDim.x) {
         const double s = ev[q / N] + ev[slot_mode<M>((int)(q % N) >> 1, (int)(q & 1))];
-        isig[q] = recip(fma(fma(sc.C3, s, sc.C2), s, sc.C1));
-        itau[q] = recip(fma(sc.lam, s, sc.Ct));
+        isig[q] = 1.0 / fma(fma(sc.C3, s, sc.C2), s, sc.C1);
+        itau[q] = 1.0 / fma(sc.lam, s, sc.Ct);
     }
 }
 
@@ -375,8 +375,8 @@ kx_col_solve(const double* __restrict__ in, double* __restrict__ out, const int4
         for (int u = 0; u < 2; ++u) {
             const int i = u ? item_slot2<M>(k) : k;
             const double sx = evx + __ldg(ev + slot_mode<M>(i, 0)), sy = evx + __ldg(ev + slot_mode<M>(i, 1));
-            const double x = line_double(z[u].x, ex, tf.p) * recip(c0 + sx * (c1 + c2 * sx));
-            const double y = line_double(z[u].y, ex, tf.p) * recip(c0 + sy * (c1 + c2 * sy));
+            const double x = line_double(z[u].x, ex, tf.p) / (c0 + sx * (c1 + c2 * sx));
+            const double y = line_double(z[u].y, ex, tf.p) / (c0 + sy * (c1 + c2 * sy));
             reinterpret_cast<double2*>(buf)[i] = make_double2(x, y);
             mx = max(mx, max(mag_hi(x), mag_hi(y)));
         }

@@ -876,27 +876,6 @@ __device__ __forceinline__ double from_order_key(long long k) {
     return __longlong_as_double(k >= 0 ? k : k ^ 0x7fffffffffffffffLL);
 }
 
-// 1/x and 1/sqrt(x) for positive normal x, error within two units in the last
-// place: hardware seed (20 bits or more) and one step of third order (e = 1 -
-// d r, r (1 + e + e^2); e = 1 - x y^2, y (1 + e/2 + 3 e^2/8)).  Three and five
-// dependent FP64 instructions instead of the library routines' longer chains.
-__device__ __forceinline__ double rcp_(double d) {
-    const unsigned h = (unsigned)__double2hiint(d) & 0x7fffffffu;
-    if (h - 0x02000000u >= 0x7b000000u) return 1.0 / d;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    e = fma(e, e, e);
-    return fma(r, e, r);
-}
-__device__ __forceinline__ double rsqrt_(double x) {
-    if ((unsigned)__double2hiint(x) - 0x02000000u >= 0x7b000000u) return rsqrt(x);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x * y, y, 1.0);
-    return fma(y * e, fma(e, 0.375, 0.5), y);
-}
-
 // rows [b * per, min(n, (b + 1) * per)) of an n-row array belong to slice b
 __device__ __forceinline__ void solve_slice(int n, int b, int nslices, int& r0, int& cnt) {
     const int per = (n + nslices - 1) / nslices;
@@ -1028,7 +1007,7 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
     }
     const double h2 = co.h2;
     // normalisations 1/(2 sqrt I_V), 1/sqrt I_W, 1/sqrt I_Z (lanes 0, 1, 2)
-    const double rr = rsqrt_(h2 * (lane == 0 ? IV : lane == 1 ? IW : IZ));
+    const double rr = rsqrt(h2 * (lane == 0 ? IV : lane == 1 ? IW : IZ));
     const double nS = 0.5 * __shfl_sync(FULL, rr, 0), nQ = __shfl_sync(FULL, rr, 1), nK = __shfl_sync(FULL, rr, 2);
     // reference SAVs X_bar (Step 1 with the increments taken about phi_bar), lane q < 4
     constexpr double third = 1.0 / 3.0;
@@ -1080,7 +1059,7 @@ k_solve(const P* __restrict__ p1, int nb1, const P* __restrict__ p2, int nb2,
             return;
         }
         a = __shfl_sync(FULL, a, i == k ? 6 * piv + j : i == piv ? 6 * k + j : l);
-        const double rinv = rcp_(__shfl_sync(FULL, a, 6 * k + k));
+        const double rinv = 1.0 / __shfl_sync(FULL, a, 6 * k + k);
         const double akj = __shfl_sync(FULL, a, 6 * k + j) * rinv;
         const double aik = __shfl_sync(FULL, a, 6 * i + k);
         a = (i == k) ? akj : a - aik * akj;
