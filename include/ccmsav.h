@@ -337,7 +337,9 @@ int ccmsav_mass_noalloc(const void* psi, int N, int precision, double L,
  * uses Mob = 0.01, dt = 1e-6 and ten steps (T = 1e-5) with Neumann ghosts.
  *
  * Device pointers f, u, phi hold N*N values of the solver's precision
- * (FP64 or FP32), row-major, 16-byte aligned; f and u may be the same array.
+ * (FP64 or FP32), row-major; f and u may be the same array.  Neumann and
+ * Dirichlet fields are 16-byte aligned, else CCMSAV_EINVAL; periodic ones may
+ * start at any value (FP32 from N = 64 on: 8-byte aligned for the faster kernels).
  * The calls are asynchronous on the solver's stream (ccmsav_solver_sync waits
  * for it).  The solver owns its tables and one N x N scratch field (complex
  * for periodic) and frees them in ccmsav_solver_destroy. */

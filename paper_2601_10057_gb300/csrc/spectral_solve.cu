@@ -3,6 +3,7 @@
 // closing remarks on other boundaries) and the initial-condition smoother of
 // Appendix F, behind the ccmsav_solver_* entry points of include/ccmsav.h.
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -101,6 +102,10 @@ template <typename T> int setup(ccmsav_solver* s) {
     return cudaStreamSynchronize(s->st) == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
 }
 
+bool aligned(const void* p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
+// The Neumann and Dirichlet kernels access 16 bytes at a time.
+bool accepts(const ccmsav_solver* s, const void* p) { return s->bc == CCMSAV_BC_PERIODIC || aligned(p, 16); }
+
 template <typename T> int solve(ccmsav_solver* s, const double c[3], const T* f, T* u) {
     const int N = s->N;
     if constexpr (sizeof(T) == sizeof(double))
@@ -111,7 +116,8 @@ template <typename T> int solve(ccmsav_solver* s, const double c[3], const T* f,
             return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
         }
     if constexpr (sizeof(T) == sizeof(float))
-        if (s->lc && ccm::lf::solve_ok(s->lt, c)) {
+        // the half-spectrum rows move float pairs; the general periodic kernels single values, from any address of a float
+        if (s->lc && aligned(f, sizeof(float2)) && aligned(u, sizeof(float2)) && ccm::lf::solve_ok(s->lt, c)) {
             float2* a = static_cast<float2*>(s->scratch);      // N^2 complex values: the half spectrum twice
             float2* b = a + (size_t)N * (N / 2);
             s->lo->prow_fwd(f, a, s->lt, s->st);
@@ -202,7 +208,7 @@ extern "C" int ccmsav_solver_create(ccmsav_solver_t** out, int N, double L, int 
 }
 
 extern "C" int ccmsav_solver_solve(ccmsav_solver_t* s, const double coef[3], const void* f, void* u) {
-    if (!s || !coef || !f || !u) return CCMSAV_EINVAL;
+    if (!s || !coef || !f || !u || !accepts(s, f) || !accepts(s, u)) return CCMSAV_EINVAL;
     for (int i = 0; i < 3; ++i) if (!std::isfinite(coef[i])) return CCMSAV_EINVAL;
     if (coef[1] < 0.0 || coef[2] < 0.0) return CCMSAV_EINVAL;
     if (!(coef[0] + s->smin * (coef[1] + coef[2] * s->smin) > 0.0)) return CCMSAV_EINVAL;
@@ -212,7 +218,7 @@ extern "C" int ccmsav_solver_solve(ccmsav_solver_t* s, const double coef[3], con
 }
 
 extern "C" int ccmsav_solver_smooth(ccmsav_solver_t* s, double eps, double mobility, double dt, int nsteps, void* phi) {
-    if (!s || !phi || nsteps < 0) return CCMSAV_EINVAL;
+    if (!s || !phi || nsteps < 0 || !accepts(s, phi)) return CCMSAV_EINVAL;
     if (!(std::isfinite(eps) && eps > 0.0 && std::isfinite(mobility) && mobility >= 0.0 && std::isfinite(dt) && dt > 0.0))
         return CCMSAV_EINVAL;
     return s->precision == CCMSAV_FP64 ? smooth<double>(s, eps, mobility, dt, nsteps, static_cast<double*>(phi))
