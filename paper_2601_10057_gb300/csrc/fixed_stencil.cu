@@ -58,9 +58,10 @@ bool make_stencil(const StencilCoef<double>& c, StencilFix& k) {
     const int g = exp_of(std::max(std::max(c.gin, c.gout), std::max(std::fabs(c.bin), std::fabs(c.bout)))) + 2;
     const double gi = std::ldexp(c.gin, -g), go = std::ldexp(c.gout, -g), bi = std::ldexp(c.bin, -g), bo = std::ldexp(c.bout, -g);
     const double ai = gi * c.psin, ao = go * c.psout, ci = 0.5 * ai * c.psin + bi, co = 0.5 * ao * c.psout + bo;
-    // |psi| <= 3: P below 4, |f_in| + |f_out| below 3 (the sums of 2^10 cells fit)
+    // |psi| <= 3: P below 4; |f_in| + |f_out| and the cell's (1 + p) f_in + (1 - p) f_out, at most twice the larger one, below 8
     if ((gi + go) * 3.0 + std::fabs(ai) + std::fabs(ao) > 3.9) return false;
-    if (0.5 * (gi + go) * 9.0 + 3.0 * (std::fabs(ai) + std::fabs(ao)) + std::fabs(ci) + std::fabs(co) > 7.9) return false;
+    const double fi = 4.5 * gi + 3.0 * std::fabs(ai) + std::fabs(ci), fo = 4.5 * go + 3.0 * std::fabs(ao) + std::fabs(co);
+    if (2.0 * std::max(fi, fo) > 7.9) return false;
     k.al = factor(0.5 * (gi + go)); k.al0 = q60(0.5 * (ai + ao));
     k.be = factor(0.5 * (gi - go)); k.be0 = q60(0.5 * (ai - ao));
     k.d2 = factor(0.5 * (gi - go)); k.d1 = q60(-(ai - ao)); k.d0 = q60(ci - co);

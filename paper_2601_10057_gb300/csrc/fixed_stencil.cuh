@@ -152,7 +152,7 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
     ll* sP = sph + H1 * W1;                             // psi*, then P 2^-g
     ll* sdq = sP + H1 * W1;                             // psi^n - psi^{n-1}
     ll* slb = sdq + H1 * W1;                            // h^2 Lap 3 phi_bar / 8
-    __shared__ ll ssum[NW][4];
+    __shared__ longlong2 ssum[NW][4];                   // (value 2^27 and up, below)
     __shared__ ll smin[NW];
     __shared__ float stiny[NW][3];
     const int bx = blockIdx.x, by = blockIdx.y, i0 = bx * TX, j0 = by * TYB;
@@ -305,14 +305,15 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
         }
         S_ = N_;
     }
-    // sums with 53 fractional bits over the warp (at most 2^10 cells of size below 2), then FP64
-    ll v[4] = {accV, accA, accB, accZ};
+    // Warp sums of the threads' 56-bit sums (nine cells below 8 at most), exact and without overflow: in pieces of 27,
+    // 27 and 10 bits, the upper two put together in units of 2^27.
+    const ll v[4] = {accV, accA, accB, accZ};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        ll x = (v[q] + 4) >> 3;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) ssum[tid >> 5][q] = x;
+        const unsigned p0 = __reduce_add_sync(0xffffffffu, (unsigned)v[q] & 0x7ffffffu);
+        const unsigned p1 = __reduce_add_sync(0xffffffffu, (unsigned)(v[q] >> 27) & 0x7ffffffu);
+        const int p2 = __reduce_add_sync(0xffffffffu, (int)(v[q] >> 54));
+        if (lane == 0) ssum[tid >> 5][q] = make_longlong2(((ll)p2 << 27) + p1, p0);
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -330,7 +331,7 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
         double r = 0.0;
         auto sum = [&](int q) {
             double s = 0.0;
-            for (int w = 0; w < NW; ++w) s += to_double(fx{ssum[w][q]}, -53);
+            for (int w = 0; w < NW; ++w) s += to_double(fx{ssum[w][q].x}, -29) + to_double(fx{ssum[w][q].y}, -56);
             for (int w = 0; q < 3 && w < NW; ++w) s += (double)stiny[w][q] * 0x1p-120;
             return s;
         };
