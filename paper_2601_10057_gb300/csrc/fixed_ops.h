@@ -20,21 +20,21 @@ __host__ __device__ constexpr Fac fac(long long w) {
 
 // Coefficients of the fixed-point stencil (fixed_stencil.cuh).  x_c: factors;
 // _exp: exponents of the outputs (value = fixed 2^exp); long long: with 60
-// fractional bits.  al .. s0: P 2^-g = (al psi - al0) + p (be psi - be0),
-// (f_in -+ f_out) 2^-g = (d2 psi + d1) psi + d0 and s2, s1, s0.
+// fractional bits.  p_in, p_out: gamma/2 2^-pa; f_in, f_out: 2 gamma 2^-fa;
+// |beta_in|, |beta_out| <= 2^fb.
 struct StencilFix {
     int bdf1;
-    int f_exp, s_exp, h_exp, q_exp, p_exp, gexp;
-    Fac f_lap, f_lap2, f_th, f_bar, s_c, betaf, h_p, h_l, q_x, q_t, M0, al, be, d2, s2, qpi;
-    long long beta, al0, be0, d1, d0, s1, s0;
-    double g_c, l_c, wV, wA, wB, wZ;
+    int f_exp, s_exp, h_exp, q_exp, pa, fa, fb;
+    Fac f_lap, f_lap2, f_th, f_bar, s_c, betaf, h_p, h_l, q_x, q_t, M0, p_in, p_out, f_in, f_out, qpi;
+    long long beta;
+    double g_c, wV, wA, wB;
 };
 // false: parameters outside the kernel's range (the caller takes k_stencil)
 bool make_stencil(const StencilCoef<double>& c, StencilFix& k);
 int stencil_setup(int N);                // shared-memory opt-in of the kernel for N x N fields
 int stencil_rows(int N);                 // partial rows it writes
 void stencil(const double* phn, const double* pho, const double* psn, const double* pso, double* out, double* part, int N,
-             const StencilFix& k, const StencilCoef<double>& c, cudaStream_t st);
+             const StencilFix& k, const StencilCoef<double>& c, const DevScalars* sc, cudaStream_t st);
 int stencil_oob(unsigned* flag);         // as Ops::oob
 
 // Twiddle and pair tables of one line length (device, one allocation: the

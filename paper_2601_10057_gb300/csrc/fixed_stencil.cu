@@ -54,25 +54,19 @@ bool make_stencil(const StencilCoef<double>& c, StencilFix& k) {
     const double qx = 2.0 * c.inv_eps2, qt = 3.0 * c.inv_h2;
     const int qe = exp_of(std::max(qx, qt)) + 1;
     k.q_x = factor(std::ldexp(qx, -qe)); k.q_t = factor(std::ldexp(qt, -qe)); k.q_exp = qe - Q;
-    // P, K, I_Z: gamma 2^-g <= 1/4
-    const int g = exp_of(std::max(std::max(c.gin, c.gout), std::max(std::fabs(c.bin), std::fabs(c.bout)))) + 2;
-    const double gi = std::ldexp(c.gin, -g), go = std::ldexp(c.gout, -g), bi = std::ldexp(c.bin, -g), bo = std::ldexp(c.bout, -g);
-    const double ai = gi * c.psin, ao = go * c.psout, ci = 0.5 * ai * c.psin + bi, co = 0.5 * ao * c.psout + bo;
-    // |psi| <= 3: P below 4; |f_in| + |f_out| and the cell's (1 + p) f_in + (1 - p) f_out, at most twice the larger one, below 8
-    if ((gi + go) * 3.0 + std::fabs(ai) + std::fabs(ao) > 3.9) return false;
-    const double fi = 4.5 * gi + 3.0 * std::fabs(ai) + std::fabs(ci), fo = 4.5 * go + 3.0 * std::fabs(ao) + std::fabs(co);
-    if (2.0 * std::max(fi, fo) > 7.9) return false;
-    k.al = factor(0.5 * (gi + go)); k.al0 = q60(0.5 * (ai + ao));
-    k.be = factor(0.5 * (gi - go)); k.be0 = q60(0.5 * (ai - ao));
-    k.d2 = factor(0.5 * (gi - go)); k.d1 = q60(-(ai - ao)); k.d0 = q60(ci - co);
-    k.s2 = factor(0.5 * (gi + go)); k.s1 = q60(-(ai + ao)); k.s0 = q60(ci + co);
+    // P, K, I_Z: gamma/2 2^-pa <= 1/4, 2 gamma 2^-fa <= 1/2 (|u| <= 4 units: P' <= 2, f' <= 3)
+    const int ga = exp_of(std::max(c.gin, c.gout));
+    k.pa = ga + 1;
+    k.p_in = factor(std::ldexp(c.gin, -k.pa - 1)); k.p_out = factor(std::ldexp(c.gout, -k.pa - 1));
+    k.fa = ga + 2;
+    k.f_in = factor(std::ldexp(c.gin, 1 - k.fa)); k.f_out = factor(std::ldexp(c.gout, 1 - k.fa));
+    const double bm = std::max(std::fabs(c.bin), std::fabs(c.bout));
+    k.fb = bm == 0.0 ? -2000 : exp_of(bm);
     k.qpi = factor(0.78539816339744830962);
-    k.gexp = k.p_exp = g - Q;
     k.M0 = factor(c.M0);
     // g0' = lam kq Lap(psi^n - psi^{n-1}), kq = -2/3 (BDF1: 0); L_P
     k.g_c = c.bdf1 ? 0.0 : c.lam * (-2.0 / 3.0) * c.inv_h2;
-    k.l_c = std::ldexp(c.inv_h2, g);
-    k.wV = c.quarter_inv_eps; k.wA = 3.0 * c.inv_h2; k.wB = c.inv_eps2; k.wZ = std::ldexp(1.0, g);
+    k.wV = c.quarter_inv_eps; k.wA = 3.0 * c.inv_h2; k.wB = c.inv_eps2;
     return true;
 }
 
@@ -90,11 +84,11 @@ int stencil_rows(int N) {
     return with_tile(N, [&](auto tx, auto ty) { return (N / decltype(tx)::value) * (N / decltype(ty)::value); });
 }
 void stencil(const double* phn, const double* pho, const double* psn, const double* pso, double* out, double* part, int N,
-             const StencilFix& k, const StencilCoef<double>& c, cudaStream_t st) {
+             const StencilFix& k, const StencilCoef<double>& c, const DevScalars* sc, cudaStream_t st) {
     with_tile(N, [&](auto tx, auto ty) {
         constexpr int X = decltype(tx)::value, Y = decltype(ty)::value;
         k_stencil_fixed<X, kTileY, Y><<<dim3(N / X, N / Y), dim3(X, kTileY), fixed_stencil_smem<X, Y>(), st>>>(
-            phn, pho, psn, pso, out, part, N, k, c);
+            phn, pho, psn, pso, out, part, N, k, c, sc);
         return 0;
     });
 }

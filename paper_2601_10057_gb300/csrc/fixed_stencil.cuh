@@ -30,9 +30,14 @@
 // every SM one); now bound by instruction issue (65 % of the slots busy, DRAM
 // 15 %).
 //
-// Range: |phi*| <= 1.5, |phi_bar| < 4/3, |psi*| <= 3, face differences of phi*
+// Concentrations are in a unit of their own (psi_unit, from psi_in, psi_out and
+// the conserved mean), and the osmotic terms P, f_in, f_out of a tile scaled by
+// the largest |psi* - psi_in|, |psi* - psi_out| in it: with 60 absolute bits and
+// psi of size 1e-3 I_Z was off by 2e-11, at 1e-6 by 5e-6.
+//
+// Range: |phi*| <= 1.5, |phi_bar| < 4/3, |psi*| <= 3 units, face differences of phi*
 // up to 1/4, of 3 phi_bar up to 1 and of the normalised flux up to 1.5,
-// |psi^n - psi^{n-1}| <= 1/2.  A CTA with a cell
+// |psi^n - psi^{n-1}| <= 1/2 unit.  A CTA with a cell
 // outside (steeper profiles than 4 cells per interface width, diverging or
 // non-finite states) evaluates its tile in FP64 instead (stencil_tile).
 #pragma once
@@ -72,14 +77,15 @@ template <int S> __device__ __forceinline__ ll sqrv(Fac a) {
 constexpr int Q = 60;                             // fractional bits of the fields
 constexpr ll kOne = 1LL << Q;
 
-// x with Q fractional bits, rounded; |x| >= 4, infinities and NaN set bad
-__device__ __forceinline__ ll to_q(double x, bool& bad) {
+// x 2^-p with Q fractional bits, rounded; |x 2^-p| >= 4, infinities and NaN set
+// bad.  |p| <= 900.
+__device__ __forceinline__ ll to_q(double x, bool& bad, int p = 0) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     const int e = (int)((hi >> 20) & 0x7ffu);
-    bad |= e > 1024;
+    bad |= e > 1024 + p;
     const unsigned m = (hi & 0xfffffu) | 0x100000u;     // subnormals and zero: far below the last bit
     unsigned H = __funnelshift_l(lo, m, 10), Lw = lo << 10;
-    const int r = max(0, min(1024 - e, 63));            // mantissa at bit 62 -> 2 units, rounded by the last shift
+    const int r = max(0, min(1024 + p - e, 63));        // mantissa at bit 62 -> 2 units, rounded by the last shift
     if (r >= 32) { Lw = H; H = 0; }
     Lw = __funnelshift_r(Lw, H, r);
     H >>= r & 31;
@@ -140,16 +146,46 @@ __device__ __forceinline__ Face face(ll pm, ll pp, ll Pm, ll Pp, Fac M0, ll& m) 
     return f;
 }
 
+// Binary exponent p of the unit of psi: the largest of |psi_in|, |psi_out| and of
+// the conserved mean lies in 2^(p - 2) .. 2^(p - 1), whatever unit a
+// concentration is given in (three units are six times it or more).  The largest
+// |psi| is at least the mean, so a mean above 2^(p - 7) keeps the error of psi
+// (2^-61 units) below that of FP64.  kNoUnit: smaller means (and units far from
+// 1), which take the FP64 stencil.
+constexpr int kNoUnit = 0x40000000;
+__device__ __forceinline__ int psi_unit(double mean, double psin, double psout) {
+    const int em = (int)(mag_hi(mean) >> 20), e = max(max((int)(mag_hi(psin) >> 20), (int)(mag_hi(psout) >> 20)), em);
+    return em + 5 < e || e < 1021 - 300 || e > 1021 + 300 ? kNoUnit : e - 1021;
+}
+
+// Bitwise or of x over the CTA (two words); s: NW words of 64 bits, read after
+// the next barrier by or_all.
+__device__ __forceinline__ void or_warp(unsigned long long x, unsigned long long* s) {
+    const unsigned l = __reduce_or_sync(0xffffffffu, (unsigned)x), h = __reduce_or_sync(0xffffffffu, (unsigned)(x >> 32));
+    if ((threadIdx.x & 31) == 0) *s = ((unsigned long long)h << 32) | l;
+}
+template <int NW> __device__ __forceinline__ unsigned long long or_all(const unsigned long long* s) {
+    unsigned long long x = s[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) x |= s[w];
+    return x;
+}
+// Magnitude of x but for the last unit (one's complement), for or_warp
+__device__ __forceinline__ unsigned long long mag_bits(ll x) { return (unsigned long long)(x ^ (x >> 63)); }
+// Left shift that brings values of those bits below 2^top
+__device__ __forceinline__ int room(unsigned long long bits, int top) { return max(0, top - 64 + __clzll((ll)bits)); }
+
+// One tile; false if a cell lies outside the range (what has been written is
+// then to be written again).
 template <int TX, int TY, int TYB>
-__global__ void __launch_bounds__(TX * TY, TX * TY <= 128 ? 4 : 2)
-k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, const double* __restrict__ psn,
-                const double* __restrict__ pso, double* __restrict__ out, double* __restrict__ part, int N,
-                const __grid_constant__ StencilFix k, const __grid_constant__ StencilCoef<double> c) {
-    extern __shared__ __align__(16) unsigned char smraw[];
+__device__ __forceinline__ bool
+fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* __restrict__ pho, const double* __restrict__ psn,
+           const double* __restrict__ pso, double* __restrict__ out, double* __restrict__ part, int N, const StencilFix& k,
+           const StencilCoef<double>& c, const DevScalars* __restrict__ sc) {
     constexpr int W2 = TX + 4, W1 = TX + 2, H1 = TYB + 2, NT = TX * TY, RPT = TYB / TY, NW = NT / 32;
     ll* sbar = reinterpret_cast<ll*>(smraw);            // 3 phi_bar, [TYB+4][W2]
     ll* sph = sbar + (TYB + 4) * W2;                    // phi*, [H1][W1] each below
-    ll* sP = sph + H1 * W1;                             // psi*, then P 2^-g
+    ll* sP = sph + H1 * W1;                             // psi*, then P'
     ll* sdq = sP + H1 * W1;                             // psi^n - psi^{n-1}
     ll* slb = sdq + H1 * W1;                            // h^2 Lap 3 phi_bar / 8
     __shared__ longlong2 ssum[NW][4];                   // (value 2^27 and up, below)
@@ -159,7 +195,12 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
     const int tid = threadIdx.y * TX + threadIdx.x;
     const size_t NN = (size_t)N * N;
     const bool two = !k.bdf1;
+    const int pe = psi_unit(sc->mass_mode, c.psin, c.psout);
+    if (pe == kNoUnit) return false;                    // the whole grid
     bool bad = false;
+    const ll pin = to_q(c.psin, bad, pe), pout = to_q(c.psout, bad, pe);
+    __shared__ unsigned long long sou[NW];
+    unsigned long long ou = 0;                          // psi* - psi_in and psi* - psi_out
     {   // halo load, as in stencil_tile
         constexpr int RH = TYB + 4, NR = RH / TY, NI = NR + 1, NB = NI < 4 ? NI : 4;
         static_assert(RH % TY == 0 && 4 * RH <= NT && TYB % TY == 0, "halo load mapping");
@@ -199,8 +240,9 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
                     sbar[lj * W2 + li] = b3;
                     if (lj >= 1 && lj <= TYB + 2 && li >= 1 && li <= TX + 2) {
                         const int o = (lj - 1) * W1 + (li - 1);
-                        const ll s = to_q(rc[b], bad), du = two ? s - to_q(rd[b], bad) : 0;
+                        const ll s = to_q(rc[b], bad, pe), du = two ? s - to_q(rd[b], bad, pe) : 0;
                         bad |= outside(s + du, hi_of(3.0)) || outside(du, hi_of(0.5));
+                        ou |= mag_bits(s + du - pin) | mag_bits(s + du - pout);
                         sph[o] = ps;
                         sP[o] = s + du;
                         sdq[o] = du;
@@ -209,8 +251,15 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
             }
         }
     }
+    or_warp(ou, &sou[tid >> 5]);
     __syncthreads();
-    // one-halo region: h^2 Lap 3 phi_bar, P; on the tile's own cells K and the I_Z term
+    // The osmotic terms of u = psi* - psi_in, psi* - psi_out (both exact, below 4): u times 2^su, below 1 where it can be,
+    // P = P' 2^p_exp, f = gamma/2 u^2 + beta = f' 2^f_exp with |P'| <= 2, |f'| <= 3.
+    const int su = room(or_all<NW>(sou), Q), fe0 = k.fa + 2 * (pe - su), f_exp = max(fe0, k.fb), fd = min(f_exp - fe0, 63);
+    const int p_exp = k.pa + pe - su;
+    const ll bin = to_q(c.bin, bad, f_exp), bout = to_q(c.bout, bad, f_exp);
+    const ll half_fd = fd ? 1LL << (fd - 1) : 0;
+    // one-halo region: h^2 Lap 3 phi_bar, P'; on the tile's own cells K and the I_Z term
     ll accZ = 0;
 #pragma unroll 1
     for (int q = tid; q < W1 * H1; q += NT) {
@@ -219,20 +268,20 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
         const ll C = b[0], dE = b[1] - C, dW = b[-1] - C, dN = b[W2] - C, dS = b[-W2] - C;
         bad |= outside(dE, hi_of(1.0)) || outside(dW, hi_of(1.0)) || outside(dN, hi_of(1.0)) || outside(dS, hi_of(1.0));
         slb[q] = (((dE + dW) + (dN + dS)) + 4) >> 3;
-        const ll ps = sP[q];
+        const ll ui = (sP[q] - pin) << su, uo = (sP[q] - pout) << su;
         ll sp, cp;
         sincos_half_pi(sph[q], sp, cp);
         const Fac spf = split(sp);
-        // P 2^-g = (al psi - al0) + p (be psi - be0)
-        sP[q] = (mulc(ps, k.al) - k.al0) + mulc(mulc(ps, k.be) - k.be0, spf);
+        // P = (1 + p) gamma_in u_in / 2 + (1 - p) gamma_out u_out / 2
+        const ll Pi = mulc(ui, k.p_in), Po = mulc(uo, k.p_out);
+        sP[q] = (Pi + Po) + mulc(Pi - Po, spf);
         const int gi = i0 + li1 - 1, gj = j0 + lj1 - 1;
         if (lj1 >= 1 && lj1 <= TYB && li1 >= 1 && li1 <= TX && CCM_OK(4 * NN + (size_t)gj * N + gi, 8 * NN)) {
-            // (f_in -+ f_out) 2^-g as polynomials in psi
-            const Fac pf = split(ps);
-            const ll D = mulv<Q>(split(mulc(ps, k.d2) + k.d1), pf) + k.d0;
-            const ll S = mulv<Q>(split(mulc(ps, k.s2) + k.s1), pf) + k.s0;
-            out[4 * NN + (size_t)gj * N + gi] = to_double(fx{mulc(mulc(D, split(cp)), k.qpi)}, k.gexp);
-            accZ += (S + mulc(D, spf) + 8) >> 4;
+            const ll fi = ((mulc(sqrv<Q + 2>(split(ui)), k.f_in) + half_fd) >> fd) + bin;
+            const ll fo = ((mulc(sqrv<Q + 2>(split(uo)), k.f_out) + half_fd) >> fd) + bout;
+            const ll D = fi - fo;
+            out[4 * NN + (size_t)gj * N + gi] = to_double(fx{mulc(mulc(D, split(cp)), k.qpi)}, f_exp - Q);
+            accZ += (fi + fo + mulc(D, spf) + 8) >> 4;
         }
     }
     __syncthreads();
@@ -286,9 +335,9 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
             out[NN + g] = to_double(fx{mulc(p3m - mulv<Q>(pf, k.betaf), k.s_c)}, k.s_exp);
             out[2 * NN + g] = to_double(fx{mulc(p3m, k.h_p) - mulc(lapp, k.h_l)}, k.h_exp);
             out[3 * NN + g] = to_double(fx{mulc(X, k.q_x) - mulc(T, k.q_t)}, k.q_exp);
-            out[5 * NN + g] = to_double(fx{PC}, k.p_exp);
-            out[6 * NN + g] = to_double(fx{lapd}, -Q) * k.g_c;
-            out[7 * NN + g] = to_double(fx{(E_.fl - W_.fl) + (N_.fl - S_.fl)}, -Q) * k.l_c;
+            out[5 * NN + g] = to_double(fx{PC}, p_exp - Q);
+            out[6 * NN + g] = to_double(fx{lapd}, pe - Q) * k.g_c;
+            out[7 * NN + g] = to_double(fx{(E_.fl - W_.fl) + (N_.fl - S_.fl)}, p_exp - Q) * c.inv_h2;
         }
         // Away from the interfaces the three terms are below the last bit; there they are added in FP32, so that
         // a state without any interface (phi within 1e-9 of +-1 everywhere) still has its radicands.
@@ -323,21 +372,18 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mmin = min(mmin, __shfl_xor_sync(0xffffffffu, mmin, o));
     if (lane == 0) smin[tid >> 5] = mmin;
-    if (__syncthreads_or(bad)) {                        // uniform over the CTA
-        stencil_tile<double, TX, TY, TYB>(smraw, phn, pho, psn, pso, out, part, N, c, bx, by, gridDim.x);
-        return;
-    }
+    if (__syncthreads_or(bad)) return false;
     if (tid < NRED1) {
         double r = 0.0;
-        auto sum = [&](int q) {
+        auto sum = [&](int q, int e = 0) {
             double s = 0.0;
-            for (int w = 0; w < NW; ++w) s += to_double(fx{ssum[w][q].x}, -29) + to_double(fx{ssum[w][q].y}, -56);
+            for (int w = 0; w < NW; ++w) s += to_double(fx{ssum[w][q].x}, e - 29) + to_double(fx{ssum[w][q].y}, e - 56);
             for (int w = 0; q < 3 && w < NW; ++w) s += (double)stiny[w][q] * 0x1p-120;
             return s;
         };
         if (tid == 0) r = sum(0) * k.wV;
         else if (tid == 1) r = sum(1) * k.wA + sum(2) * k.wB;
-        else if (tid == 2) r = sum(3) * k.wZ;
+        else if (tid == 2) r = sum(3, f_exp);
         else if (tid == 8) {
             ll m = smin[0];
             for (int w = 1; w < NW; ++w) m = min(m, smin[w]);
@@ -345,6 +391,19 @@ k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, 
         }
         part[(size_t)(by * gridDim.x + bx) * NRED1 + tid] = r;
     }
+    return true;
+}
+
+template <int TX, int TY, int TYB>
+__global__ void __launch_bounds__(TX * TY, TX * TY <= 128 ? 4 : 2)
+k_stencil_fixed(const double* __restrict__ phn, const double* __restrict__ pho, const double* __restrict__ psn,
+                const double* __restrict__ pso, double* __restrict__ out, double* __restrict__ part, int N,
+                const __grid_constant__ StencilFix k, const __grid_constant__ StencilCoef<double> c,
+                const DevScalars* __restrict__ sc) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    // uniform over the CTA
+    if (!fixed_tile<TX, TY, TYB>(smraw, phn, pho, psn, pso, out, part, N, k, c, sc))
+        stencil_tile<double, TX, TY, TYB>(smraw, phn, pho, psn, pso, out, part, N, c, blockIdx.x, blockIdx.y, gridDim.x);
 }
 
 }  // namespace xf

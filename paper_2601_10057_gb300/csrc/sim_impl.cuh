@@ -1153,7 +1153,7 @@ public:
         if constexpr (std::is_same<T, double>::value) {
             xf::StencilFix k;
             if (xo && (fixed = xf::make_stencil(c, k))) {
-                xf::stencil(phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, k, c, st);
+                xf::stencil(phi[cur], phi[prev], psi[cur], psi[prev], bufA, part1, N, k, c, sc, st);
                 so.nb1 = nb1x;
             }
         }

@@ -65,3 +65,44 @@ def test_sums_of_large_terms(N, case, monkeypatch):
     else:
         p, phi = p.replace(beta=1.0), _half_zero(N, p.L)
     _assert_same(*_both(monkeypatch, p, phi, psi))
+
+
+@pytest.mark.parametrize("N", [64, 256])
+@pytest.mark.parametrize("scale", [1e3, 30.0, 1e-2, 1e-4, 1e-6, 1e-9, 1e-100])
+def test_unit_of_the_concentration(N, scale, monkeypatch):
+    """The same vesicle with the concentration in another unit."""
+    w = I.workload("one_vesicle", N=N, dt=1e-7 / max(1.0, scale * scale))
+    p = w.params.replace(psi_in=scale * w.params.psi_in, psi_out=scale * w.params.psi_out)
+    _assert_same(*_both(monkeypatch, p, w.phi0, scale * w.psi0))
+
+
+@pytest.mark.parametrize("N", [64, 256])
+@pytest.mark.parametrize("amp", [1e-2, 1e-4, 1e-6])
+def test_concentration_close_to_the_preferred_one(N, amp, monkeypatch):
+    """psi within amp of psi_in = psi_out: f is gamma/2 (psi - psi_in)^2.  FP64
+    rounds psi* by 2^-54, relative to the smallest |psi - psi_in| (0.05 amp) 2^-49 / amp;
+    I_Z is twice as far off, its root as far as that."""
+    w = I.workload("one_vesicle", N=N, dt=1e-7)
+    p = w.params.replace(psi_in=0.65, psi_out=0.65)
+    got, want = _both(monkeypatch, p, w.phi0, 0.65 + amp * (w.psi0 - 0.65))
+    _assert_same(got, want, 1e-12 + 2.0**-49 / amp)
+
+
+@pytest.mark.parametrize("ratio", [1e-1, 1e-2, 1e-4, 0.0])
+def test_concentration_far_below_the_preferred_one(ratio, monkeypatch):
+    """psi against psi_in and psi_out of order one, down to the FP64 stencil's
+    part (means below 1/32 of them) and to psi = 0."""
+    w = I.workload("one_vesicle", N=128, dt=1e-9)
+    got, want = _both(monkeypatch, w.params, w.phi0, ratio * w.psi0)
+    _assert_same(got, want)
+
+
+@pytest.mark.parametrize("bg", [(1e-3, -2e-3), (2e4, 7e4), (5e9, 5e9)])
+@pytest.mark.parametrize("gamma", [0.0, 1e2, 1e5])
+def test_osmotic_constants(gamma, bg, monkeypatch):
+    """beta_in, beta_out far below and far above gamma psi^2."""
+    w = I.workload("one_vesicle", N=128, dt=1e-9)
+    p = w.params.replace(gamma_in=gamma, gamma_out=2.0 * gamma, beta_in=bg[0], beta_out=bg[1])
+    if gamma == 0.0:
+        p = p.replace(beta_out=abs(bg[1]))
+    _assert_same(*_both(monkeypatch, p, w.phi0, w.psi0))
