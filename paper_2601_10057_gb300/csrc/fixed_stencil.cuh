@@ -172,6 +172,7 @@ template <int NW> __device__ __forceinline__ unsigned long long or_all(const uns
 }
 // Magnitude of x but for the last unit (one's complement), for or_warp
 __device__ __forceinline__ unsigned long long mag_bits(ll x) { return (unsigned long long)(x ^ (x >> 63)); }
+__device__ __forceinline__ ll shl(ll x, int s) { return (ll)((unsigned long long)x << s); }
 // Left shift that brings values of those bits below 2^top
 __device__ __forceinline__ int room(unsigned long long bits, int top) { return max(0, top - 64 + __clzll((ll)bits)); }
 
@@ -190,7 +191,6 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
     ll* slb = sdq + H1 * W1;                            // h^2 Lap 3 phi_bar / 8
     __shared__ longlong2 ssum[NW][4];                   // (value 2^27 and up, below)
     __shared__ ll smin[NW];
-    __shared__ float stiny[NW][3];
     const int bx = blockIdx.x, by = blockIdx.y, i0 = bx * TX, j0 = by * TYB;
     const int tid = threadIdx.y * TX + threadIdx.x;
     const size_t NN = (size_t)N * N;
@@ -199,7 +199,8 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
     if (pe == kNoUnit) return false;                    // the whole grid
     bool bad = false;
     const ll pin = to_q(c.psin, bad, pe), pout = to_q(c.psout, bad, pe);
-    __shared__ unsigned long long sou[NW];
+    __shared__ unsigned long long soa[NW], sou[NW];
+    unsigned long long oa = 0;                          // |phi*| - 1
     unsigned long long ou = 0;                          // psi* - psi_in and psi* - psi_out
     {   // halo load, as in stencil_tile
         constexpr int RH = TYB + 4, NR = RH / TY, NI = NR + 1, NB = NI < 4 ? NI : 4;
@@ -243,6 +244,8 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
                         const ll s = to_q(rc[b], bad, pe), du = two ? s - to_q(rd[b], bad, pe) : 0;
                         bad |= outside(s + du, hi_of(3.0)) || outside(du, hi_of(0.5));
                         ou |= mag_bits(s + du - pin) | mag_bits(s + du - pout);
+                        const ll sg = ps >> 63;
+                        oa |= mag_bits((ps ^ sg) - sg - kOne);
                         sph[o] = ps;
                         sP[o] = s + du;
                         sdq[o] = du;
@@ -251,8 +254,15 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
             }
         }
     }
+    or_warp(oa, &soa[tid >> 5]);
     or_warp(ou, &sou[tid >> 5]);
     __syncthreads();
+    // The SAV sums take phi^3 - phi and the face differences times 2^sa, phi^2 - 1 - beta times 2^sv, so that a tile
+    // away from the interfaces (and a state without any) has its sums to the same relative accuracy as one across an
+    // interface.  With | |phi*| - 1 | <= oa the three are at most 2.5 oa (|phi*| <= 3/2), 2 oa and 2.5 oa + |beta|; where
+    // sa > 0 a tile holds one phase (differences below 1/4; across phases they are above 7/4, out of range).
+    const unsigned long long oat = or_all<NW>(soa);
+    const int sa = room(oat, 57), sv = room(3 * oat + 3 + (unsigned long long)llabs(k.beta), 59);
     // The osmotic terms of u = psi* - psi_in, psi* - psi_out (both exact, below 4): u times 2^su, below 1 where it can be,
     // P = P' 2^p_exp, f = gamma/2 u^2 + beta = f' 2^f_exp with |P'| <= 2, |f'| <= 3.
     const int su = room(or_all<NW>(sou), Q), fe0 = k.fa + 2 * (pe - su), f_exp = max(fe0, k.fb), fd = min(f_exp - fe0, 63);
@@ -268,7 +278,7 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
         const ll C = b[0], dE = b[1] - C, dW = b[-1] - C, dN = b[W2] - C, dS = b[-W2] - C;
         bad |= outside(dE, hi_of(1.0)) || outside(dW, hi_of(1.0)) || outside(dN, hi_of(1.0)) || outside(dS, hi_of(1.0));
         slb[q] = (((dE + dW) + (dN + dS)) + 4) >> 3;
-        const ll ui = (sP[q] - pin) << su, uo = (sP[q] - pout) << su;
+        const ll ui = shl(sP[q] - pin, su), uo = shl(sP[q] - pout, su);
         ll sp, cp;
         sincos_half_pi(sph[q], sp, cp);
         const Fac spf = split(sp);
@@ -288,7 +298,6 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
     const int gi = i0 + threadIdx.x, li = threadIdx.x + 1, lane = tid & 31;
     const int r0 = threadIdx.y * RPT;
     ll accV = 0, accA = 0, accB = 0, mmin = 1LL << 62;
-    float tiny[3] = {0.f, 0.f, 0.f};                    // the same three sums times 2^120
     ll mN;
     Face S_;
     {
@@ -339,19 +348,14 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
             out[6 * NN + g] = to_double(fx{lapd}, pe - Q) * k.g_c;
             out[7 * NN + g] = to_double(fx{(E_.fl - W_.fl) + (N_.fl - S_.fl)}, p_exp - Q) * c.inv_h2;
         }
-        // Away from the interfaces the three terms are below the last bit; there they are added in FP32, so that
-        // a state without any interface (phi within 1e-9 of +-1 everywhere) still has its radicands.
-        if (__all_sync(0xffffffffu, !outside(vv, hi_of(0x1p-14)) && (sd2 >> 32) == 0)) {
-            const float fv = __ll2float_rn(vv), f3 = __ll2float_rn(p3m), fp = __ll2float_rn(pC) * 0x1p-60f;
-            const float fe = __ll2float_rn(E_.d), fw = __ll2float_rn(W_.d), fn = __ll2float_rn(N_.d), fs = __ll2float_rn(S_.d);
-            tiny[0] = fmaf(fv, fv, tiny[0]);
-            tiny[1] = fmaf(fp * fp, (fe * fe + fw * fw) + (fn * fn + fs * fs), tiny[1]);
-            tiny[2] = fmaf(f3, f3, tiny[2]);
-        } else {
-            accV += (sqrv<Q>(split(vv)) + 8) >> 4;
-            accA += (mulv<Q>(split(sd2), split(p2)) + 8) >> 4;
-            accB += (sqrv<Q>(split(p3m)) + 8) >> 4;
-        }
+        // the terms of the SAV sums, scaled
+        ll a2 = sd2;
+        if (sa)
+            a2 = (sqrv<Q>(split(shl(E_.d, sa))) + sqrv<Q>(split(shl(W_.d, sa)))) +
+                 (sqrv<Q>(split(shl(N_.d, sa))) + sqrv<Q>(split(shl(S_.d, sa))));
+        accV += (sqrv<Q>(split(shl(vv, sv))) + 8) >> 4;
+        accA += (mulv<Q>(split(a2), split(p2)) + 8) >> 4;
+        accB += (sqrv<Q>(split(shl(p3m, sa))) + 8) >> 4;
         S_ = N_;
     }
     // Warp sums of the threads' 56-bit sums (nine cells below 8 at most), exact and without overflow: in pieces of 27,
@@ -365,24 +369,18 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
         if (lane == 0) ssum[tid >> 5][q] = make_longlong2(((ll)p2 << 27) + p1, p0);
     }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const float x = warp_sum(tiny[q]);
-        if (lane == 0) stiny[tid >> 5][q] = x;
-    }
-#pragma unroll
     for (int o = 16; o > 0; o >>= 1) mmin = min(mmin, __shfl_xor_sync(0xffffffffu, mmin, o));
     if (lane == 0) smin[tid >> 5] = mmin;
     if (__syncthreads_or(bad)) return false;
     if (tid < NRED1) {
         double r = 0.0;
-        auto sum = [&](int q, int e = 0) {
+        auto sum = [&](int q, int e) {
             double s = 0.0;
             for (int w = 0; w < NW; ++w) s += to_double(fx{ssum[w][q].x}, e - 29) + to_double(fx{ssum[w][q].y}, e - 56);
-            for (int w = 0; q < 3 && w < NW; ++w) s += (double)stiny[w][q] * 0x1p-120;
             return s;
         };
-        if (tid == 0) r = sum(0) * k.wV;
-        else if (tid == 1) r = sum(1) * k.wA + sum(2) * k.wB;
+        if (tid == 0) r = sum(0, -2 * sv) * k.wV;
+        else if (tid == 1) r = sum(1, -2 * sa) * k.wA + sum(2, -2 * sa) * k.wB;
         else if (tid == 2) r = sum(3, f_exp);
         else if (tid == 8) {
             ll m = smin[0];

@@ -106,3 +106,19 @@ def test_osmotic_constants(gamma, bg, monkeypatch):
     if gamma == 0.0:
         p = p.replace(beta_out=abs(bg[1]))
     _assert_same(*_both(monkeypatch, p, w.phi0, w.psi0))
+
+
+@pytest.mark.parametrize("beta", [0.0, 1e-3, 0.3])
+@pytest.mark.parametrize("amp", [1e-12, 1e-10, 1e-9, 1e-7, 1e-5, 1e-4, 1e-3])
+@pytest.mark.parametrize("N", [64, 512])
+def test_savs_of_a_state_without_an_interface(N, amp, beta, monkeypatch):
+    """phi between 1 - 2.5 amp and 1 - 0.5 amp: the radicands are sums of terms of
+    size amp^2 (I_V: about beta^2), so the SAVs show their accuracy.  FP64 rounds
+    phi* and phi*^2 by 2^-54, relative to |phi*^2 - 1| >= amp 2^-53 / amp; four
+    times that for the terms of a step."""
+    p = I.growth_params(eps=8.0 / N, dt=1e-6, L=1.0, beta=beta)
+    x = (np.arange(N) + 0.5) / N
+    phi = 1.0 - amp * (1.5 + np.cos(np.pi * x)[None, :] * np.cos(2 * np.pi * x)[:, None])
+    psi = 0.5 + 0.1 * np.cos(np.pi * x)[:, None] * np.ones(N)[None, :]
+    got, want = _both(monkeypatch, p, phi, psi, 3)
+    _assert_same(got, want, 1e-12 + 2.0**-51 / amp)
