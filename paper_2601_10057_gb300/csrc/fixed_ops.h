@@ -25,9 +25,9 @@ __host__ __device__ constexpr Fac fac(long long w) {
 struct StencilFix {
     int bdf1;
     int f_exp, s_exp, h_exp, q_exp, pa, fa, fb;
-    Fac f_lap, f_lap2, f_th, f_bar, s_c, betaf, h_p, h_l, q_x, q_t, M0, p_in, p_out, f_in, f_out, qpi;
+    Fac f_lap, f_lap2, f_th, s_c, betaf, h_p, h_l, q_x, q_t, M0, p_in, p_out, f_in, f_out, qpi;
     long long beta;
-    double g_c, wV, wA, wB;
+    double g_c, bar, wV, wA, wB;
 };
 // false: parameters outside the kernel's range (the caller takes k_stencil)
 bool make_stencil(const StencilCoef<double>& c, StencilFix& k);

@@ -37,11 +37,11 @@ bool make_stencil(const StencilCoef<double>& c, StencilFix& k) {
     k = StencilFix{};
     k.bdf1 = c.bdf1;
     // f0'
-    const double f1 = c.C2 * (8.0 / 3.0) * c.inv_h2, f2 = c.C3 * (8.0 / 3.0) * c.inv_h2 * c.inv_h2, f3 = c.Mth * c.inv_h2,
-                 f4 = c.betap / 3.0;
-    const int fe = exp_of(std::max(std::max(std::fabs(f1), std::fabs(f2)), std::max(std::fabs(f3), std::fabs(f4)))) + 2;
+    const double f1 = c.C2 * (8.0 / 3.0) * c.inv_h2, f2 = c.C3 * (8.0 / 3.0) * c.inv_h2 * c.inv_h2, f3 = c.Mth * c.inv_h2;
+    const int fe = exp_of(std::max(std::max(std::fabs(f1), std::fabs(f2)), std::fabs(f3))) + 2;
     k.f_lap = factor(std::ldexp(f1, -fe)); k.f_lap2 = factor(std::ldexp(f2, -fe));
-    k.f_th = factor(std::ldexp(f3, -fe)); k.f_bar = factor(std::ldexp(f4, -fe));
+    k.f_th = factor(std::ldexp(f3, -fe));
+    k.bar = c.betap / 3.0;
     k.f_exp = fe - Q;
     // S, H, Q
     const int se = exp_of(c.inv_eps);

@@ -15,7 +15,9 @@
 //   exact sums of differences that add up to zero over the grid, take their
 //   coefficient in FP64: a product rounded at the last bit of the fixed-point
 //   value is not conservative (psi 7e-14 off after two steps at N = 4096,
-//   against 6e-16).
+//   against 6e-16).  So does the term of f0' in phi_bar (beta > 0), which is the
+//   same in every cell of a phase: at the scale of the Lap^2 term its rounding
+//   moved phi's mean by 1.4e-13 a step (N = 2048, gamma_bend = 1, dt = 1e-4).
 //   The nonlocal bending term uses the identity
 //     h^2 [phi |grad phi|^2 - div(phi^2 grad phi)]
 //       = -1/2 phi (sum_f d_f^2 + 2 phi h^2 Lap phi) - 1/2 sum_f +-d_f^3
@@ -337,10 +339,12 @@ fixed_tile(unsigned char* smraw, const double* __restrict__ phn, const double* _
         const ll lC = slb[o];
         const ll lap2 = ((slb[o + 1] - lC) + (slb[o - 1] - lC)) + ((slb[o + W1] - lC) + (slb[o - W1] - lC));
         const ll bC = sbar[(jj + 2) * W2 + li + 1];
-        const ll f0 = ((mulc(lC, k.f_lap) - mulc(lap2, k.f_lap2)) - (mulc(lapp, k.f_th) + mulc(bC, k.f_bar)));
+        const ll f0 = (mulc(lC, k.f_lap) - mulc(lap2, k.f_lap2)) - mulc(lapp, k.f_th);
         const ll vv = p2m - k.beta;
         if (CCM_OK(7 * NN + g, 8 * NN)) {
-            out[g] = to_double(fx{f0}, k.f_exp);
+            double f = to_double(fx{f0}, k.f_exp);
+            if (k.bar != 0.0) f = fma(-k.bar, to_double(fx{bC}, -Q), f);
+            out[g] = f;
             out[NN + g] = to_double(fx{mulc(p3m - mulv<Q>(pf, k.betaf), k.s_c)}, k.s_exp);
             out[2 * NN + g] = to_double(fx{mulc(p3m, k.h_p) - mulc(lapp, k.h_l)}, k.h_exp);
             out[3 * NN + g] = to_double(fx{mulc(X, k.q_x) - mulc(T, k.q_t)}, k.q_exp);

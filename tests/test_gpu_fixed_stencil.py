@@ -122,3 +122,14 @@ def test_savs_of_a_state_without_an_interface(N, amp, beta, monkeypatch):
     psi = 0.5 + 0.1 * np.cos(np.pi * x)[:, None] * np.ones(N)[None, :]
     got, want = _both(monkeypatch, p, phi, psi, 3)
     _assert_same(got, want, 1e-12 + 2.0**-51 / amp)
+
+
+@pytest.mark.parametrize("beta", [0.0, 0.1, 0.3, 1.0])
+def test_mean_of_phi_with_a_stiff_bending_term(beta, monkeypatch):
+    """f0' holds beta phi_bar beside a bending term of coefficients ten million
+    times larger; in the bulk it is the same in all cells.  Two steps of three
+    roundings at |phi| = 1 (phi_bar, the increment, the sum) on either path:
+    2e-15."""
+    w = I.workload("one_vesicle", N=2048)
+    got, want = _both(monkeypatch, w.params.replace(beta=beta, gamma_bend=1.0, dt=1e-4), w.phi0, w.psi0)
+    assert abs((got[0] - want[0]).mean()) <= 2e-15
