@@ -14,10 +14,15 @@
 //            the transform.  It is taken per lane (the values that one lane
 //            transforms in registers) and per line: the line is shifted right
 //            by s0 before the first in-register pass so that no lane can
-//            exceed 2^60, and by sh more at the twiddles between the passes,
+//            exceed 2^60, and by more at the twiddles between the passes,
 //            so that the line cannot.  Localised lines and sparse spectra
 //            (most of this scheme's: the interface, the low modes) need
-//            neither; a dense line shifts by log2 of its length in all;
+//            neither; a dense line shifts by log2 of its length in all, on
+//            long lines in both later passes by what each can add: a
+//            shift's rounding grows by the square root of the length still to
+//            be transformed, and all of it at the first twiddle left dense
+//            lines of N = 4096 and 8192 further off than FP64 ones (8192: 1.2e-15
+//            against 4.1e-16 .. 4.9e-16);
 //   twiddles 64-bit constants with 62 fractional bits (error 2^-63; FP64
 //            twiddles carry 2^-54), products rounded at the last bit.
 // The error is thus a few units of 2^-60 of the line's L1 norm, below that of
@@ -132,17 +137,23 @@ __device__ __forceinline__ cx twidx(cx x, int i) {
     return cmulf<!INV>(x, CFac{fac(cos64(j)), fac(cos64(j + 48))});     // exp(+i ...), conjugated for the forward one
 }
 
+// One level of a radix-2 decimation in frequency on v[OFF .. OFF + R)
+template <int R, bool INV, int OFF>
+__device__ __forceinline__ void level(cx* v) {
+#pragma unroll
+    for (int i = 0; i < R / 2; ++i) {
+        const cx a = v[OFF + i], b = v[OFF + i + R / 2];
+        v[OFF + i] = a + b;
+        v[OFF + i + R / 2] = twidx<R, INV>(a - b, i);
+    }
+}
+
 // Radix-2 decimation in frequency on v[OFF .. OFF + R): natural input, output
 // v[OFF + r] = X[bitrev_R(r)].
 template <int R, bool INV, int OFF>
 struct DIFX {
     static __device__ __forceinline__ void run(cx* v) {
-#pragma unroll
-        for (int i = 0; i < R / 2; ++i) {
-            const cx a = v[OFF + i], b = v[OFF + i + R / 2];
-            v[OFF + i] = a + b;
-            v[OFF + i + R / 2] = twidx<R, INV>(a - b, i);
-        }
+        level<R, INV, OFF>(v);
         DIFX<R / 2, INV, OFF>::run(v);
         DIFX<R / 2, INV, OFF + R / 2>::run(v);
     }
@@ -175,6 +186,9 @@ template <int M> struct Geo {
     static constexpr int BUF = ((A * P + 7) / 8) * 8 + 1;
     static constexpr size_t SMEM = (size_t)LINES * BUF * sizeof(cx);
     static constexpr int MINB = 512 / THREADS > 4 ? 4 : 512 / THREADS;       // at most 128 registers
+    static constexpr bool STAGED = M >= 1024;              // shifts in both passes (shorter lines: all at the first twiddle)
+    static constexpr int LOG_C = C == 4 ? 2 : C == 8 ? 3 : 4;
+    static_assert(1 << LOG_C == C, "");
     static_assert(THREADS % 32 == 0, "whole warps");
 };
 
@@ -277,12 +291,34 @@ __device__ __forceinline__ fx shift_fx(fx a, int sh) {
 }
 __device__ __forceinline__ cx shift_cx(cx a, int sh) { return mk(shift_fx(a.x, sh), shift_fx(a.y, sh)); }
 
-// v: this lane's E values, components below 2^60.6.  Shifts the line right by
+// DIFX<Z> with a shift after its second level, the last one with products.  A
+// product by W_8 takes values of modulus below 2^60.5, so the inputs are below
+// 2^58 (Z = 16: four are added before it) or 2^59 (Z = 8: two), or their whole sum
+// is below 2^60: that part of the shift (kPre bits) comes before.
+template <int Z> constexpr int kPre = Z == 16 ? 2 : 1;
+template <int Z, bool INV>
+__device__ __forceinline__ void dif_shift(cx* v, int sh) {
+    static_assert(Z == 8 || Z == 16, "");
+    level<Z, INV, 0>(v);
+    level<Z / 2, INV, 0>(v);
+    level<Z / 2, INV, Z / 2>(v);
+    if (sh) {
+#pragma unroll
+        for (int i = 0; i < Z; ++i) v[i] = shift_cx(v[i], sh);
+    }
+    DIFX<Z / 4, INV, 0>::run(v);
+    DIFX<Z / 4, INV, Z / 4>::run(v);
+    DIFX<Z / 4, INV, Z / 2>::run(v);
+    DIFX<Z / 4, INV, 3 * (Z / 4)>::run(v);
+}
+
+// v: this lane's E values, components below 2^62.  Shifts the line right by
 // s0 (returned through ex, which it is added to) so that no lane's first pass
-// can exceed 2^60, and sets sh, the further shift at the twiddles that keeps
-// the line below 2^60 (ex also counts it).
+// can exceed 2^60, and sets the further shifts (ex also counts them): sh.x at
+// the first twiddle for the second pass, a sum over C lanes, and sh.y for the
+// last one, most of it between that one's levels.
 template <int M>
-__device__ __forceinline__ void fit_line(cx* v, int slot, LineSm<M>& sm, int& ex, int& sh) {
+__device__ __forceinline__ void fit_line(cx* v, int slot, LineSm<M>& sm, int& ex, int2& sh) {
     constexpr int E = Geo<M>::E;
     unsigned acc = 0;                                  // lane sum of |re| + |im| in units of 2^38, rounded up
 #pragma unroll
@@ -294,12 +330,14 @@ __device__ __forceinline__ void fit_line(cx* v, int slot, LineSm<M>& sm, int& ex
     const float tot = line_sum<M>((float)acc, slot, sm) * 1.001f;
     const int s0 = max(0, top - 22);
     const int et = ((__float_as_int(tot) >> 23) & 0xff) - 126;          // line sum below 2^et
-    sh = max(0, et - 22 - s0);
+    const int e2 = Geo<M>::STAGED ? min(et, top + Geo<M>::LOG_C) : et;
+    sh.x = max(0, e2 - 22 - s0);
+    sh.y = max(0, et - 22 - s0 - sh.x);
     if (s0 > 0) {
 #pragma unroll
         for (int i = 0; i < E; ++i) v[i] = shift_cx(v[i], s0);
     }
-    ex += s0 + sh;
+    ex += s0 + sh.x + sh.y;
 }
 
 // ------------------------------------------------------------------ line transform
@@ -318,7 +356,7 @@ __device__ __forceinline__ CFac ld_fac(const int4* __restrict__ t) {
 // Lanes run along d in step 2 and along k1 in the last step: both reads and
 // the natural-order write are free of bank conflicts.
 template <int M, bool INV>
-__device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict__ tw, int n2, int slot, int sh) {
+__device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict__ tw, int n2, int slot, int2 sh) {
     using Gm = Geo<M>;
     constexpr int A = Gm::A, C = Gm::C, D = Gm::D, G = Gm::G, P = Gm::P;
     DIFX<A, INV, 0>::run(v);
@@ -327,9 +365,10 @@ __device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict_
         const int k1 = wf::bitrev<A>(r);
         cx u = v[r];
         if (k1) u = cmulf<INV>(u, ld_fac(tw + k1 * G + n2));
-        buf[k1 * P + n2] = shift_cx(u, sh);
+        buf[k1 * P + n2] = shift_cx(u, sh.x);
     }
     sync_line<M>(slot);
+    const int pre = Gm::STAGED ? min(sh.y, kPre<D>) : 0;        // of sh.y, before the last pass
     if constexpr (D > 1) {
         const int4* __restrict__ t3 = tw + M;
 #pragma unroll
@@ -343,7 +382,9 @@ __device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict_
 #pragma unroll
             for (int r = 0; r < C; ++r) {
                 const int kc = wf::bitrev<C>(r);
-                row[D * kc] = kc ? cmulf<INV>(u[r], ld_fac(t3 + kc * D + d)) : u[r];
+                if (kc) u[r] = cmulf<INV>(u[r], ld_fac(t3 + kc * D + d));
+                if (Gm::STAGED && pre) u[r] = shift_cx(u[r], pre);
+                row[D * kc] = u[r];
             }
         }
         sync_line<M>(slot);
@@ -359,7 +400,8 @@ __device__ __forceinline__ void fft_line(cx* v, cx* buf, const int4* __restrict_
 #pragma unroll
     for (int j = 0; j < A / Z; ++j) {
         const int q = n2 + G * j, k1 = q % A, kc = q / A;
-        DIFX<Z, INV, 0>::run(v + j * Z);
+        if constexpr (Gm::STAGED) dif_shift<Z, INV>(v + j * Z, sh.y - pre);
+        else DIFX<Z, INV, 0>::run(v + j * Z);
 #pragma unroll
         for (int r = 0; r < Z; ++r) {
             const int kd = wf::bitrev<Z>(r);
@@ -444,7 +486,8 @@ __device__ __forceinline__ int forward_line(const double* __restrict__ x, cx* bu
                                              int slot, LineSm<M>& sm, bool odd_row) {
     constexpr int E = Geo<M>::E, G = Geo<M>::G;
     cx v[E];
-    int ex, sh;
+    int ex;
+    int2 sh;
     bool bad;
     {
         double d[2 * E];
@@ -498,15 +541,17 @@ __device__ __forceinline__ int inverse_line(unsigned mx, cx* buf, const int4* __
     if constexpr (!OWN) sync_line<M>(slot);
     const bool bad = mx >= 0x7ff00000u;
     const int em = max((int)(mx >> 20), 1);
-    // room for the pairs: a sample of z is at most 4 sqrt(2) times the largest mode
+    // Room for the pairs: with modes below 2^59 the second product takes a sum of two values below 2^59.5, and a sample
+    // of z is below 2^61.5.  The bits left are what the small modes of a line with a large mean are rounded by.
 #pragma unroll 1
     for (int i = 0; i < E / 2; ++i) {
         const int k = n2 + G * i;
         const double2 p = reinterpret_cast<const double2*>(buf)[k], q = reinterpret_cast<const double2*>(buf)[item_slot2<M>(k)];
-        pre_item<M>(mk(to_fixed(p.x, em + 2), to_fixed(p.y, em + 2)), mk(to_fixed(q.x, em + 2), to_fixed(q.y, em + 2)), ti, k,
+        pre_item<M>(mk(to_fixed(p.x, em + 1), to_fixed(p.y, em + 1)), mk(to_fixed(q.x, em + 1), to_fixed(q.y, em + 1)), ti, k,
                     buf);
     }
-    int ex = em + 2 - 1082 + ti.p, sh;
+    int ex = em + 1 - 1082 + ti.p;
+    int2 sh;
     sync_line<M>(slot);
     cx v[E];
 #pragma unroll
