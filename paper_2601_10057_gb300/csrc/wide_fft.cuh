@@ -54,12 +54,53 @@ __device__ __forceinline__ cf ld_c(const float2* __restrict__ t) {
     return mk(w.x, w.y);
 }
 
+// x W_R^i, W_R = exp(-2 pi i / R) (INV: conjugate), with the constants as a high
+// and a low part.  Their rounding is the same in every line; a 16-point DFT has
+// more of them than the radix-8 passes of the block-level transforms, and with
+// rounded ones a line of 2048 or 4096 values was 3 - 6 % further off than theirs.
+template <int R, bool INV>
+__device__ __forceinline__ cf twid(cf x, int i) {
+    static_assert(R <= 16, "");
+    const int j = (i * (32 / R)) & 31;                 // below 16
+    if (j == 0) return x;
+    if (j == 8) return INV ? mk(-x.y, x.x) : mk(x.y, -x.x);
+    double c, s;
+    wf::w32(j, c, s);
+    const float ch = (float)c, cl = (float)(c - (double)ch);
+    if (j == 4 || j == 12) {
+        auto mul = [&](float t) { return fmaf(t, ch, t * cl); };
+        const float p = mul(x.x + x.y), m = mul(x.x - x.y);      // c = +-sqrt(1/2); j = 4: (p, -m), j = 12: (m, p)
+        if (j == 4) return INV ? mk(m, p) : mk(p, -m);
+        return INV ? mk(p, -m) : mk(m, p);
+    }
+    const float sh = (float)s, sl = (float)(s - (double)sh);
+    auto dot = [](float a, float h, float l, float b, float g, float k) { return fmaf(a, h, fmaf(b, g, fmaf(a, l, b * k))); };
+    return INV ? mk(dot(x.x, ch, cl, x.y, -sh, -sl), dot(x.y, ch, cl, x.x, sh, sl))
+               : mk(dot(x.x, ch, cl, x.y, sh, sl), dot(x.y, ch, cl, x.x, -sh, -sl));
+}
+// In-register radix-2 decimation in frequency on v[OFF .. OFF + R): natural
+// input, output v[OFF + r] = X[bitrev_R(r)].
+template <int R, bool INV, int OFF>
+struct DIF {
+    static __device__ __forceinline__ void run(cf* v) {
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) {
+            const cf a = v[OFF + i], b = v[OFF + i + R / 2];
+            v[OFF + i] = a + b;
+            v[OFF + i + R / 2] = twid<R, INV>(a - b, i);
+        }
+        DIF<R / 2, INV, OFF>::run(v);
+        DIF<R / 2, INV, OFF + R / 2>::run(v);
+    }
+};
+template <bool INV, int OFF> struct DIF<1, INV, OFF> { static __device__ __forceinline__ void run(cf*) {} };
+
 // The unnormalised DFT of a line (fixed_fft.cuh, fft_line, has the passes).
 template <int M, bool INV>
 __device__ __forceinline__ void fft_line(cf* v, cf* buf, const float2* __restrict__ tw, int n2, int slot) {
     using Gm = Geo<M>;
     constexpr int A = Gm::A, C = Gm::C, D = Gm::D, G = Gm::G, P = Gm::P;
-    wf::DIF<float, A, INV, 0>::run(v);
+    DIF<A, INV, 0>::run(v);
 #pragma unroll
     for (int r = 0; r < A; ++r) {
         const int k1 = wf::bitrev<A>(r);
@@ -77,7 +118,7 @@ __device__ __forceinline__ void fft_line(cf* v, cf* buf, const float2* __restric
             cf u[C];
 #pragma unroll
             for (int c = 0; c < C; ++c) u[c] = row[D * c];
-            wf::DIF<float, C, INV, 0>::run(u);
+            DIF<C, INV, 0>::run(u);
 #pragma unroll
             for (int r = 0; r < C; ++r) {
                 const int kc = wf::bitrev<C>(r);
@@ -98,7 +139,7 @@ __device__ __forceinline__ void fft_line(cf* v, cf* buf, const float2* __restric
 #pragma unroll
     for (int j = 0; j < A / Z; ++j) {
         const int q = n2 + G * j, k1 = q % A, kc = q / A;
-        wf::DIF<float, Z, INV, 0>::run(v + j * Z);
+        DIF<Z, INV, 0>::run(v + j * Z);
 #pragma unroll
         for (int r = 0; r < Z; ++r) {
             const int kd = wf::bitrev<Z>(r);
