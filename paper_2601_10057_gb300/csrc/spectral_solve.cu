@@ -116,13 +116,13 @@ template <typename T> int solve(ccmsav_solver* s, const double c[3], const T* f,
             return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
         }
     if constexpr (sizeof(T) == sizeof(float))
-        // the half-spectrum rows move float pairs; the general periodic kernels single values, from any address of a float
+        // the forward rows move float pairs; the general periodic kernels single values, from any address of a float
         if (s->lc && aligned(f, sizeof(float2)) && aligned(u, sizeof(float2)) && ccm::lf::solve_ok(s->lt, c)) {
             float2* a = static_cast<float2*>(s->scratch);      // N^2 complex values: the half spectrum twice
             float2* b = a + (size_t)N * (N / 2);
             s->lo->prow_fwd(f, a, s->lt, s->st);
             s->lc->pcol(a, b, s->ltc, s->lt, c, s->st);
-            s->lo->prow_inv(b, u, s->lt, s->st);
+            s->lc->prow_inv(b, u, s->ltc, s->st);
             s->launches += 3;
             return cudaPeekAtLastError() == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
         } else if (s->lo && !s->lc && ccm::lf::solve_ok(s->lt, c)) {

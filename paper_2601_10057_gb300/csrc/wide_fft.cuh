@@ -95,8 +95,19 @@ struct DIF {
 };
 template <bool INV, int OFF> struct DIF<1, INV, OFF> { static __device__ __forceinline__ void run(cf*) {} };
 
+// x times the table's entry q (INV: its conjugate); LO: with the entry's low part, lo values further on
+template <bool INV, bool LO>
+__device__ __forceinline__ cf twiddle(cf x, const float2* __restrict__ t, int q, int lo) {
+    const cf w = ld_c(t + q);
+    if constexpr (!LO) return INV ? cmulc(x, w) : cmul(x, w);
+    const cf l = ld_c(t + q + lo);
+    const float wy = INV ? -w.y : w.y, ly = INV ? -l.y : l.y;
+    return mk(fmaf(x.x, w.x, fmaf(-x.y, wy, fmaf(x.x, l.x, -x.y * ly))), fmaf(x.y, w.x, fmaf(x.x, wy, fmaf(x.y, l.x, x.x * ly))));
+}
+
 // The unnormalised DFT of a line (fixed_fft.cuh, fft_line, has the passes).
-template <int M, bool INV>
+// LO: the tables' low parts as well (the periodic solver).
+template <int M, bool INV, bool LO = false>
 __device__ __forceinline__ void fft_line(cf* v, cf* buf, const float2* __restrict__ tw, int n2, int slot) {
     using Gm = Geo<M>;
     constexpr int A = Gm::A, C = Gm::C, D = Gm::D, G = Gm::G, P = Gm::P;
@@ -105,7 +116,7 @@ __device__ __forceinline__ void fft_line(cf* v, cf* buf, const float2* __restric
     for (int r = 0; r < A; ++r) {
         const int k1 = wf::bitrev<A>(r);
         cf u = v[r];
-        if (k1) { const cf w = ld_c(tw + k1 * G + n2); u = INV ? cmulc(u, w) : cmul(u, w); }
+        if (k1) u = twiddle<INV, LO>(u, tw, k1 * G + n2, 2 * M);
         buf[k1 * P + n2] = u;
     }
     sync_line<M>(slot);
@@ -122,7 +133,7 @@ __device__ __forceinline__ void fft_line(cf* v, cf* buf, const float2* __restric
 #pragma unroll
             for (int r = 0; r < C; ++r) {
                 const int kc = wf::bitrev<C>(r);
-                if (kc) { const cf w = ld_c(t3 + kc * D + d); u[r] = INV ? cmulc(u[r], w) : cmul(u[r], w); }
+                if (kc) u[r] = twiddle<INV, LO>(u[r], t3, kc * D + d, 2 * M);
                 row[D * kc] = u[r];
             }
         }
@@ -215,13 +226,14 @@ template <int M> __device__ __forceinline__ void pre_item(cf s1, cf s2, const Pa
 
 // Inverse transform of the line whose pre-processed values lie in buf
 // (visible to the line's lanes) to natural-order samples in buf.
-template <int M> __device__ __forceinline__ void inverse_line(cf* buf, const float2* __restrict__ tw, int n2, int slot) {
+template <int M, bool LO = false>
+__device__ __forceinline__ void inverse_line(cf* buf, const float2* __restrict__ tw, int n2, int slot) {
     constexpr int E = Geo<M>::E, G = Geo<M>::G;
     cf v[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) v[i] = buf[G * i + n2];
     sync_line<M>(slot);
-    fft_line<M, true>(v, buf, tw, n2, slot);
+    fft_line<M, true, LO>(v, buf, tw, n2, slot);
 }
 
 // ------------------------------------------------------------------ transposed writes

@@ -141,7 +141,8 @@ kl_row_inv(const float* in, float* out, const float2* __restrict__ tw, PairTab t
 //   E = (Z[k] + conj Z[M-k])/2, O = (Z[k] - conj Z[M-k])/(2i),
 // and only the columns kx = 0 .. M-1 are transformed along y (complex lines of
 // length N), the real rows X[0] and X[M] together as the column X[0] + i X[M].
-// Half the lines and half the traffic of full-length complex transforms.
+// Half the lines and half the traffic of full-length complex transforms, but for
+// the last pass (kp_row_inv).
 
 // Row spectra of LINES rows, written transposed: outc[kx N + y].
 template <int M>
@@ -159,7 +160,7 @@ kp_row_fwd(const float* __restrict__ in, float2* __restrict__ outc, const float2
         cf v[E];
 #pragma unroll
         for (int i = 0; i < E; ++i) v[i] = ld_c(x + G * i + n2);
-        fft_line<M, false>(v, bufs + (size_t)slot * Gm::BUF, tw, n2, slot);
+        fft_line<M, false, true>(v, bufs + (size_t)slot * Gm::BUF, tw, n2, slot);
     }
     __syncthreads();
 #pragma unroll 1
@@ -175,10 +176,9 @@ kp_row_fwd(const float* __restrict__ in, float2* __restrict__ outc, const float2
                 a[r] = mk(A.x + A.y, A.x - A.y);              // X[0] and X[M]
                 b[r] = mk(B.x, -B.y);                         // X[M/2] = conj Z[M/2]
             } else {
-                const cf e = mk(0.5f * (A.x + B.x), 0.5f * (A.y - B.y));
-                const cf o = cmul(w, mk(0.5f * (A.y + B.y), 0.5f * (B.x - A.x)));
-                a[r] = e + o;
-                b[r] = mk(e.x - o.x, o.y - e.y);
+                const cf e = mk(0.5f * (A.x + B.x), 0.5f * (A.y - B.y)), o = mk(0.5f * (A.y + B.y), 0.5f * (B.x - A.x));
+                a[r] = mk(fmaf(w.x, o.x, fmaf(-w.y, o.y, e.x)), fmaf(w.x, o.y, fmaf(w.y, o.x, e.y)));       // e + w o
+                b[r] = mk(fmaf(-w.x, o.x, fmaf(w.y, o.y, e.x)), fmaf(w.x, o.y, fmaf(w.y, o.x, -e.y)));      // conj(e - w o)
             }
         }
         *reinterpret_cast<float4*>(outc + (size_t)k * N + y0 + 2 * r2) = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
@@ -196,7 +196,7 @@ __device__ __forceinline__ float recip_mode(float2 ex, float2 ey, const DivCoef&
 
 // LINES columns kx of N complex values (Geo of line length N): FFT along y,
 // division, inverse FFT, transposed write outc[y (N/2) + kx].  sc: the
-// normalisation 1 / (2 N (N/2)) of the inverse passes and of the row split.
+// normalisation 1 / N^2 of the two inverse passes.
 template <int N>
 __global__ void __launch_bounds__(Geo<N>::THREADS, Geo<N>::MINB)
 kp_col(const float2* __restrict__ inc, float2* __restrict__ outc, const float2* __restrict__ tw,
@@ -213,7 +213,7 @@ kp_col(const float2* __restrict__ inc, float2* __restrict__ outc, const float2* 
         cf v[E];
 #pragma unroll
         for (int i = 0; i < E; ++i) v[i] = ld_c(inc + (size_t)kx * N + G * i + n2);
-        fft_line<N, false>(v, buf, tw, n2, slot);
+        fft_line<N, false, true>(v, buf, tw, n2, slot);
     }
     const float2 ex = __ldg(ev + kx);
     if (kx != 0) {
@@ -237,7 +237,7 @@ kp_col(const float2* __restrict__ inc, float2* __restrict__ outc, const float2* 
         }
     }
     sync_line<N>(slot);
-    inverse_line<N>(buf, tw, n2, slot);
+    inverse_line<N, true>(buf, tw, n2, slot);
     __syncthreads();
 #pragma unroll 2
     for (int q = threadIdx.x; q < R2 * N; q += Gm::THREADS) {
@@ -247,41 +247,36 @@ kp_col(const float2* __restrict__ inc, float2* __restrict__ outc, const float2* 
     }
 }
 
-// Inverse of kp_row_fwd on LINES rows inc[y M + kx]: real rows out[y N + x].
-template <int M>
-__global__ void __launch_bounds__(Geo<M>::THREADS, Geo<M>::MINB)
-kp_row_inv(const float2* __restrict__ inc, float* __restrict__ out, const float2* __restrict__ tw, PairTab t) {
-    using Gm = Geo<M>;
-    constexpr int N = Gm::N, E = Gm::E, G = Gm::G;
+// Inverse of kp_row_fwd: LINES rows inc[y (N/2) + kx] to real rows out[y N + x],
+// as full complex lines (Geo of line length N) whose imaginary part is dropped.
+// Half-length lines (as in the forward pass) are half the work but carry all of
+// the transform's rounding in the result instead of half of its variance: with
+// them the solve was 1.12 times as far off as with full-length transforms
+// throughout (N = 32 .. 4096, up to 1.33 where the divisor damps the noise of
+// the earlier passes).
+template <int N>
+__global__ void __launch_bounds__(Geo<N>::THREADS, Geo<N>::MINB)
+kp_row_inv(const float2* __restrict__ inc, float* __restrict__ out, const float2* __restrict__ tw) {
+    using Gm = Geo<N>;
+    constexpr int M = N / 2, E = Gm::E, G = Gm::G;
     extern __shared__ __align__(16) unsigned char smraw[];
     int n2, slot;
-    lane_of<M>(n2, slot);
+    lane_of<N>(n2, slot);
     cf* buf = reinterpret_cast<cf*>(smraw) + (size_t)slot * Gm::BUF;
     const int y = blockIdx.x * Gm::LINES + slot;
     const float2* row = inc + (size_t)y * M;
 #pragma unroll
     for (int j = 0; j < E / 2; ++j) {
-        const int k = n2 + G * j, i2 = item_slot2<M>(k);
-        const cf A = ld_c(row + k), B = ld_c(row + i2);
-        if (k == 0) {
-            buf[0] = mk(A.x + A.y, A.x - A.y);                // 2 (E + i O), E = (X[0] + X[M])/2, O = (X[0] - X[M])/2
-            buf[i2] = mk(2.f * B.x, -2.f * B.y);
-        } else {
-            // 2 (E + i O): E = (X[k] + conj X[M-k])/2, O = conj(W) (X[k] - conj X[M-k])/2
-            const cf w = mk(__ldg(t.wa + k).x, __ldg(t.wa + k).y);
-            const cf e = mk(A.x + B.x, A.y - B.y), o = cmulc(mk(A.x - B.x, A.y + B.y), w);
-            buf[k] = mk(e.x - o.y, e.y + o.x);
-            buf[i2] = mk(e.x + o.y, o.x - e.y);
-        }
+        const int k = n2 + G * j;
+        const cf A = ld_c(row + k);
+        buf[k] = k == 0 ? mk(A.x, 0.f) : A;                   // row 0 holds X[0] + i X[M]
+        buf[k == 0 ? M : N - k] = k == 0 ? mk(A.y, 0.f) : conj_(A);
     }
-    sync_line<M>(slot);
-    inverse_line<M>(buf, tw, n2, slot);
-    float2* dst = reinterpret_cast<float2*>(out + (size_t)y * N);
+    sync_line<N>(slot);
+    inverse_line<N, true>(buf, tw, n2, slot);
+    float* dst = out + (size_t)y * N;
 #pragma unroll
-    for (int i = 0; i < E; ++i) {
-        const cf z = buf[G * i + n2];
-        dst[G * i + n2] = make_float2(z.x, z.y);
-    }
+    for (int i = 0; i < E; ++i) dst[G * i + n2] = buf[G * i + n2].x;
 }
 
 }  // namespace lf

@@ -54,7 +54,7 @@ void pcol(const float2* inc, float2* outc, const Tables& t, const Tables& tev, c
                                                                1.0f / ((float)M * (float)M));
 }
 void prow_inv(const float2* inc, float* u, const Tables& t, cudaStream_t st) {
-    kp_row_inv<M><<<GRID, Gm::THREADS, Gm::SMEM, st>>>(inc, u, t.tw, PairTab{t.pf, t.pib});
+    kp_row_inv<M><<<M / Gm::LINES, Gm::THREADS, Gm::SMEM, st>>>(inc, u, t.tw);      // rows of length M
 }
 int oob(unsigned* flag) {
     *flag = 0;

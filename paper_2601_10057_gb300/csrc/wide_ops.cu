@@ -27,15 +27,16 @@ const Ops* wide_ops(int M) {
 int make_tables(const Ops* o, Tables& t, const double* he, double smin, cudaStream_t st) {
     const int M = o->M, N = 2 * M, G = M / o->A, B = o->C * o->D, np = M / 2 + 1;
     t.M = M;
-    std::vector<float2> tw(2 * (size_t)M, make_float2(0.f, 0.f)), ev(N);
-    auto root = [](double j, double n) {                     // exp(-2 pi i j / n)
-        const double a = 2.0 * M_PI * j / n;
-        return make_float2((float)std::cos(a), (float)(-std::sin(a)));
+    std::vector<float2> tw(4 * (size_t)M, make_float2(0.f, 0.f)), ev(N);
+    auto root = [&](size_t at, double j, double n) {         // exp(-2 pi i j / n): high parts, the low parts 2 M further on
+        const double c = std::cos(2.0 * M_PI * j / n), s = -std::sin(2.0 * M_PI * j / n);
+        tw[at] = make_float2((float)c, (float)s);
+        tw[at + 2 * (size_t)M] = make_float2((float)(c - (double)tw[at].x), (float)(s - (double)tw[at].y));
     };
     for (int k1 = 0; k1 < o->A; ++k1)
-        for (int n2 = 0; n2 < G; ++n2) tw[(size_t)k1 * G + n2] = root((double)((long)n2 * k1 % M), M);
+        for (int n2 = 0; n2 < G; ++n2) root((size_t)k1 * G + n2, (double)((long)n2 * k1 % M), M);
     for (int kc = 0; kc < o->C; ++kc)
-        for (int d = 0; d < o->D; ++d) tw[(size_t)M + kc * o->D + d] = root((double)((long)d * kc % B), B);
+        for (int d = 0; d < o->D; ++d) root((size_t)M + kc * o->D + d, (double)((long)d * kc % B), B);
     std::vector<float4> pf(np), pi(np);
     std::vector<float2> pfb(np), pib(np);
     const double c0 = std::sqrt(1.0 / N), c1 = std::sqrt(2.0 / N), s0 = 1.0 / (M * c0), s1 = 1.0 / (M * c1), q = M_PI / 4.0;

@@ -6,7 +6,7 @@
 namespace ccm {
 namespace lf {
 
-// Tables of one solver (device): the twiddles of the two exchanges [2 M], the
+// Tables of one solver (device): the twiddles of the two exchanges [2 M] and their low parts [2 M], the
 // pair factors (PairTab) and the 1D eigenvalues times 2^-shift as
 // (high, low) float pairs.
 struct Tables {
@@ -27,8 +27,8 @@ struct Ops {
     // from c, or from the device (dcoef); dskip: fields to leave alone (both may be null).
     void (*solve)(const float* f, float* u, float* scr, const Tables& t, const double c[3], const double* dcoef,
                   const int* dskip, int nf, bool dst, cudaStream_t st);
-    // periodic solver: the row passes of N = 2M (tables of M) and the column
-    // pass of N = M (tables of M and of the eigenvalues, tev)
+    // periodic solver: the forward row pass of N = 2M (tables of M), the column pass of N = M
+    // (tables of M and of the eigenvalues, tev) and the inverse row pass of N = M
     void (*prow_fwd)(const float* f, float2* outc, const Tables& t, cudaStream_t st);
     void (*pcol)(const float2* inc, float2* outc, const Tables& t, const Tables& tev, const double c[3], cudaStream_t st);
     void (*prow_inv)(const float2* inc, float* u, const Tables& t, cudaStream_t st);

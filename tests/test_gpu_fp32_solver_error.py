@@ -12,7 +12,7 @@ from paper_2601_10057_gb300 import inputs as I
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("bc", ["neumann", "dirichlet"])
+@pytest.mark.parametrize("bc", ["neumann", "dirichlet", "periodic"])
 def test_error_is_no_larger_than_the_general_kernels(bc):
     """Coefficients times 2^90 lie outside the wide lines' range and take the
     general kernels; the solution is 2^-90 times as large, exactly.  Geometric
