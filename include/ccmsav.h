@@ -262,7 +262,8 @@ int ccmsav_set_group_points(ccmsav_t* h, long long points);
 long long ccmsav_group_points(ccmsav_t* h);
 
 /* Index checks of a library built with -DCCMSAV_BOUNDS (a separate
- * libccmsav_bounds.so, for testing): the step kernels check every element
+ * libccmsav_bounds.so, for testing): the step kernels, and the solver's line
+ * kernels (FP64 Neumann and Dirichlet and FP32, N >= 64), check every element
  * index of their field, spectrum and level accesses against the array's
  * size; an index outside sets bit 1 (a load, redirected to element 0) or
  * bit 2 (a store, dropped) of a device flag.  Returns the flags raised by
@@ -365,6 +366,9 @@ int ccmsav_solver_smooth(ccmsav_solver_t* s, double eps, double mobility, double
 
 /* Wait for the solver's queued work. */
 int ccmsav_solver_sync(ccmsav_solver_t* s);
+
+/* ccmsav_bounds_flag of the solver's kernels. */
+int ccmsav_solver_bounds_flag(ccmsav_solver_t* s);
 
 /* Kernel launches queued by the solver since creation. */
 long long ccmsav_solver_launch_count(ccmsav_solver_t* s);

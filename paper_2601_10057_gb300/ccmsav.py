@@ -101,6 +101,7 @@ def load(path: Optional[str] = None) -> C.CDLL:
         "ccmsav_solver_solve": (i, [vp, _DP, vp, vp]),
         "ccmsav_solver_smooth": (i, [vp, d, d, d, i, vp]),
         "ccmsav_solver_sync": (i, [vp]),
+        "ccmsav_solver_bounds_flag": (i, [vp]),
         "ccmsav_solver_launch_count": (C.c_longlong, [vp]),
         "ccmsav_solver_destroy": (None, [vp]),
     }
@@ -294,6 +295,10 @@ def ccmsav_solver_smooth(s, eps: float, mobility: float, dt: float, nsteps: int,
 
 def ccmsav_solver_sync(s) -> int:
     return load().ccmsav_solver_sync(s)
+
+
+def ccmsav_solver_bounds_flag(s) -> int:
+    return load().ccmsav_solver_bounds_flag(s)
 
 
 def ccmsav_solver_launch_count(s) -> int:

@@ -214,7 +214,7 @@ kx_gram_rows(const double* __restrict__ spec, double* __restrict__ part, int N, 
         for (int j = threadIdx.x; j < N; j += kGramThreads) {
             double v[NF];
 #pragma unroll
-            for (int f = 0; f < NF; ++f) v[f] = __ldg(spec + ((size_t)kx * NF + f) * N + j);
+            for (int f = 0; f < NF; ++f) v[f] = __ldg(spec + CCM_IX(((size_t)kx * NF + f) * N + j, (size_t)NF * N * N));
             gram_mode(acc, v, __ldg(isig + (size_t)kx * N + j), __ldg(itau + (size_t)kx * N + j));
         }
     gram_store<kGramThreads>(acc, part + (size_t)blockIdx.x * NRED2, sm);
@@ -363,7 +363,8 @@ kx_col_solve(const double* __restrict__ in, double* __restrict__ out, const int4
     lane_of<M>(n2, slot);
     cx* buf = bufs + (size_t)slot * Gm::BUF;
     const int x0 = blockIdx.x * Gm::LINES, kx = x0 + slot;
-    const int ex = forward_line<M, false>(in + blockIdx.y * fstride + (size_t)kx * N, buf, tw2, n2, slot, sm, false);
+    const size_t n = gridDim.y * fstride;
+    const int ex = forward_line<M, false>(in + CCM_IXW(blockIdx.y * fstride + (size_t)kx * N, N, n), buf, tw2, n2, slot, sm, false);
     const double evx = ev[kx];
     unsigned mx = 0;
 #pragma unroll 1
@@ -383,7 +384,7 @@ kx_col_solve(const double* __restrict__ in, double* __restrict__ out, const int4
     }
     inverse_line<M, true>(mx, buf, tw2, ti, n2, slot, sm);
     __syncthreads();
-    write_transposed<M>(bufs, sm, out, blockIdx.y * fstride, x0, ~(size_t)0);
+    write_transposed<M>(bufs, sm, out, blockIdx.y * fstride, x0, n);
 }
 
 // Inverse DCT along x of LINES rows (in place allowed).  DST: times (-1)^(i+j).
@@ -400,8 +401,8 @@ kx_row_inv(const double* in, double* out, const int4* __restrict__ tw2, PairTab 
     lane_of<M>(n2, slot);
     cx* buf = reinterpret_cast<cx*>(smraw) + (size_t)slot * Gm::BUF;
     const int y = blockIdx.x * Gm::LINES + slot;
-    const size_t o = blockIdx.y * fstride + (size_t)y * N;
-    const unsigned mx = load_modes<M>(buf, in + o, n2);
+    const size_t o = blockIdx.y * fstride + (size_t)y * N, n = gridDim.y * fstride;
+    const unsigned mx = load_modes<M>(buf, in + CCM_IXW(o, N, n), n2);
     const int ex = inverse_line<M, false>(mx, buf, tw2, ti, n2, slot, sm);
 #pragma unroll 2
     for (int m = n2; m < M / 2; m += G) {
@@ -410,7 +411,7 @@ kx_row_inv(const double* in, double* out, const int4* __restrict__ tw2, PairTab 
             const double s = (y & 1) ? -1.0 : 1.0;
             v.a *= s; v.b *= -s; v.c *= s; v.d *= -s;
         }
-        st4(out + o + 4 * m, v);
+        if (CCM_OKW(o + 4 * m, 4, n)) st4(out + o + 4 * m, v);
     }
 }
 

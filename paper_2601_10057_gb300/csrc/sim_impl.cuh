@@ -765,10 +765,10 @@ public:
         CCM_CUDA(cudaStreamSynchronize(st));
         CCM_CUDA(cudaMemcpyFromSymbol(&v, g_oob_flag, sizeof(v)));
         CCM_CUDA(cudaMemcpyToSymbol(g_oob_flag, &z, sizeof(z)));
-        unsigned x = 0;
-        unsigned y = 0;
+        unsigned x = 0, y = 0, w = 0;
         if (xo && (xo->oob(&x) || xf::stencil_oob(&y))) return CCMSAV_ECUDA;
-        return (int)(v | x | y);
+        if (clo && clo->oob(&w)) return CCMSAV_ECUDA;
+        return (int)(v | x | y | w);
 #else
         return CCMSAV_EINVAL;
 #endif

@@ -230,6 +230,19 @@ extern "C" int ccmsav_solver_sync(ccmsav_solver_t* s) {
     return cudaStreamSynchronize(s->st) == cudaSuccess ? CCMSAV_OK : CCMSAV_ECUDA;
 }
 
+extern "C" int ccmsav_solver_bounds_flag(ccmsav_solver_t* s) {
+    if (!s) return CCMSAV_EINVAL;
+#ifdef CCMSAV_BOUNDS
+    unsigned x = 0, y = 0, z = 0;
+    if (cudaStreamSynchronize(s->st) != cudaSuccess || (s->xo && s->xo->oob(&x)) || (s->lo && s->lo->oob(&y)) ||
+        (s->lc && s->lc->oob(&z)))
+        return CCMSAV_ECUDA;
+    return (int)(x | y | z);
+#else
+    return CCMSAV_EINVAL;
+#endif
+}
+
 extern "C" long long ccmsav_solver_launch_count(ccmsav_solver_t* s) { return s ? s->launches : 0; }
 
 extern "C" void ccmsav_solver_destroy(ccmsav_solver_t* s) { release(s); }

@@ -83,7 +83,7 @@ kl_col_solve(const float* __restrict__ in, float* __restrict__ out, const float2
     lane_of<M>(n2, slot);
     cf* buf = bufs + (size_t)slot * Gm::BUF;
     const int x0 = blockIdx.x * Gm::LINES, kx = x0 + slot;
-    forward_line<M, false>(in + blockIdx.y * fstride + (size_t)kx * N, buf, tw, n2, slot, false);
+    forward_line<M, false>(in + CCM_IXW(blockIdx.y * fstride + (size_t)kx * N, N, gridDim.y * fstride), buf, tw, n2, slot, false);
     const float2 ex = __ldg(ev + kx);
 #pragma unroll 2
     for (int j = 0; j < E / 2; ++j) {
@@ -99,7 +99,7 @@ kl_col_solve(const float* __restrict__ in, float* __restrict__ out, const float2
     sync_line<M>(slot);
     inverse_line<M>(buf, tw, n2, slot);
     __syncthreads();
-    write_samples<M, Gm::LINES>(bufs, out + blockIdx.y * fstride + x0, x0, (size_t)N * N);
+    write_samples<M, Gm::LINES>(bufs, out + blockIdx.y * fstride + x0, blockIdx.y * fstride + x0, gridDim.y * fstride);
 }
 
 // Inverse DCT along x of LINES rows (in place allowed).  DST: times (-1)^(i+j).
@@ -115,7 +115,8 @@ kl_row_inv(const float* in, float* out, const float2* __restrict__ tw, PairTab t
     lane_of<M>(n2, slot);
     cf* buf = reinterpret_cast<cf*>(smraw) + (size_t)slot * Gm::BUF;
     const int y = blockIdx.x * Gm::LINES + slot;
-    const float* row = in + blockIdx.y * fstride + (size_t)y * N;
+    const size_t o = blockIdx.y * fstride + (size_t)y * N, n = gridDim.y * fstride;
+    const float* row = in + CCM_IXW(o, N, n);
 #pragma unroll
     for (int j = 0; j < E / 2; ++j) {
         const int k = n2 + G * j, i2 = item_slot2<M>(k);
@@ -123,13 +124,13 @@ kl_row_inv(const float* in, float* out, const float2* __restrict__ tw, PairTab t
     }
     sync_line<M>(slot);
     inverse_line<M>(buf, tw, n2, slot);
-    float* dst = out + blockIdx.y * fstride + (size_t)y * N;
 #pragma unroll
     for (int j = 0; j < E / 2; ++j) {
         const int m = n2 + G * j;
+        if (!CCM_OKW(o + 4 * m, 4, n)) continue;
         const cf a = buf[m], b = buf[M - 1 - m];
         const float s = DST && (y & 1) ? -1.f : 1.f;    // x = 4m is even: signs (+, -, +, -) times (-1)^y
-        *reinterpret_cast<float4*>(dst + 4 * m) =
+        *reinterpret_cast<float4*>(out + o + 4 * m) =
             DST ? make_float4(s * a.x, -s * b.y, s * a.y, -s * b.x) : make_float4(a.x, b.y, a.y, b.x);
     }
 }
@@ -156,7 +157,7 @@ kp_row_fwd(const float* __restrict__ in, float2* __restrict__ outc, const float2
     lane_of<M>(n2, slot);
     const int y0 = blockIdx.x * Gm::LINES;
     {
-        const float2* x = reinterpret_cast<const float2*>(in + (size_t)(y0 + slot) * N);
+        const float2* x = reinterpret_cast<const float2*>(in + CCM_IXW((size_t)(y0 + slot) * N, N, (size_t)N * N));
         cf v[E];
 #pragma unroll
         for (int i = 0; i < E; ++i) v[i] = ld_c(x + G * i + n2);
@@ -181,8 +182,9 @@ kp_row_fwd(const float* __restrict__ in, float2* __restrict__ outc, const float2
                 b[r] = mk(fmaf(-w.x, o.x, fmaf(w.y, o.y, e.x)), fmaf(w.x, o.y, fmaf(w.y, o.x, -e.y)));      // conj(e - w o)
             }
         }
-        *reinterpret_cast<float4*>(outc + (size_t)k * N + y0 + 2 * r2) = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
-        *reinterpret_cast<float4*>(outc + (size_t)item_slot2<M>(k) * N + y0 + 2 * r2) = make_float4(b[0].x, b[0].y, b[1].x, b[1].y);
+        const size_t oa = (size_t)k * N + y0 + 2 * r2, ob = (size_t)item_slot2<M>(k) * N + y0 + 2 * r2;
+        if (CCM_OKW(oa, 2, (size_t)M * N)) *reinterpret_cast<float4*>(outc + oa) = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+        if (CCM_OKW(ob, 2, (size_t)M * N)) *reinterpret_cast<float4*>(outc + ob) = make_float4(b[0].x, b[0].y, b[1].x, b[1].y);
     }
 }
 
@@ -212,7 +214,7 @@ kp_col(const float2* __restrict__ inc, float2* __restrict__ outc, const float2* 
     {
         cf v[E];
 #pragma unroll
-        for (int i = 0; i < E; ++i) v[i] = ld_c(inc + (size_t)kx * N + G * i + n2);
+        for (int i = 0; i < E; ++i) v[i] = ld_c(inc + CCM_IX((size_t)kx * N + G * i + n2, (size_t)M * N));
         fft_line<N, false, true>(v, buf, tw, n2, slot);
     }
     const float2 ex = __ldg(ev + kx);
@@ -243,7 +245,8 @@ kp_col(const float2* __restrict__ inc, float2* __restrict__ outc, const float2* 
     for (int q = threadIdx.x; q < R2 * N; q += Gm::THREADS) {
         const int r2 = q % R2, y = q / R2;
         const cf a = bufs[(size_t)(2 * r2) * Gm::BUF + y], b = bufs[(size_t)(2 * r2 + 1) * Gm::BUF + y];
-        *reinterpret_cast<float4*>(outc + (size_t)y * M + x0 + 2 * r2) = make_float4(a.x, a.y, b.x, b.y);
+        const size_t o = (size_t)y * M + x0 + 2 * r2;
+        if (CCM_OKW(o, 2, (size_t)M * N)) *reinterpret_cast<float4*>(outc + o) = make_float4(a.x, a.y, b.x, b.y);
     }
 }
 
@@ -264,7 +267,7 @@ kp_row_inv(const float2* __restrict__ inc, float* __restrict__ out, const float2
     lane_of<N>(n2, slot);
     cf* buf = reinterpret_cast<cf*>(smraw) + (size_t)slot * Gm::BUF;
     const int y = blockIdx.x * Gm::LINES + slot;
-    const float2* row = inc + (size_t)y * M;
+    const float2* row = inc + CCM_IXW((size_t)y * M, M, (size_t)M * N);
 #pragma unroll
     for (int j = 0; j < E / 2; ++j) {
         const int k = n2 + G * j;
@@ -274,9 +277,11 @@ kp_row_inv(const float2* __restrict__ inc, float* __restrict__ out, const float2
     }
     sync_line<N>(slot);
     inverse_line<N, true>(buf, tw, n2, slot);
-    float* dst = out + (size_t)y * N;
 #pragma unroll
-    for (int i = 0; i < E; ++i) dst[G * i + n2] = buf[G * i + n2].x;
+    for (int i = 0; i < E; ++i) {
+        const size_t o = (size_t)y * N + G * i + n2;
+        if (CCM_OK(o, (size_t)N * N)) out[o] = buf[G * i + n2].x;
+    }
 }
 
 }  // namespace lf

@@ -32,7 +32,7 @@ struct Ops {
     void (*prow_fwd)(const float* f, float2* outc, const Tables& t, cudaStream_t st);
     void (*pcol)(const float2* inc, float2* outc, const Tables& t, const Tables& tev, const double c[3], cudaStream_t st);
     void (*prow_inv)(const float2* inc, float* u, const Tables& t, cudaStream_t st);
-    int (*oob)(unsigned* flag);
+    int (*oob)(unsigned* flag);         // index-check flag of the translation unit: read and cleared (CCMSAV_BOUNDS)
 };
 
 const Ops* wide_ops(int M);              // M = 32 .. 4096, else null
