@@ -235,8 +235,8 @@ int ccmsav_profile_read(ccmsav_t* h, int sim, double ms[8], long long* nsteps);
  * least 2 % faster) and restores the state (the
  * fields and scalars are unchanged afterwards).  Candidates (FP32): the
  * warp-level four-step FFT kernels with a shared-memory carveout of 72, 58
- * or 100 percent for the three 8-line transform kernels, and the CTA-level
- * Stockham FFT kernels; FP64 has one schedule.  The choice is recorded
+ * or 100 percent for the two of them (72 alone at N = 8192, whose kernels do not
+ * depend on it), and the CTA-level Stockham FFT kernels; FP64 has one schedule.  The choice is recorded
  * for each (N, precision) of the handle in a process-wide table, from which
  * handles created later start.  For several simulations a second stage then
  * times the launch-group size (ccmsav_set_group_points: the current value,

@@ -343,12 +343,13 @@ int ccmsav_autotune(ccmsav_t* h, int steps, double* report) {
     // what the handle runs (a schedule that is faster for one simulation
     // alone can be slower when the simulations share the GPU).
     const int k = (steps < 3 ? 3 : steps + 2) / 3 * 3;
-    bool any_warp = false;
+    bool any_warp = false, any_carveout = false;
     for (ccm::SimBase* s : h->sims) {
         if ((r = s->tune_save())) return r;
         any_warp = any_warp || s->tune_has_warp();
+        any_carveout = any_carveout || s->tune_has_carveout();
     }
-    const std::vector<ccm::TuneChoice> cand = ccm::tune_candidates(any_warp);
+    const std::vector<ccm::TuneChoice> cand = ccm::tune_candidates(any_warp, any_carveout);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) r = CCMSAV_ECUDA;
     auto drop_batch = [&]() {

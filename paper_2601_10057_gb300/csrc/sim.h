@@ -9,15 +9,19 @@ namespace ccm {
 
 // Schedule chosen by the autotuner for one (grid size, precision): the FFT
 // path of the line transforms (warp-level four-step FFT or CTA-level Stockham
-// FFT) and the shared-memory carveout of the three 8-line warp-FFT kernels.
+// FFT) and the shared-memory carveout of the two warp-FFT kernels.
 // Process-wide, so handles created later with the same N start from it.
 struct TuneChoice { int warp = 1; int carveout = 72; double ms = 0.0, ms_default = 0.0; };
-// Candidate schedules, the default first: warp-FFT kernels at carveouts of
-// 72, 58 and 100 percent (where the warp path exists), then the block FFT.
-inline std::vector<TuneChoice> tune_candidates(bool have_warp) {
+// Candidate schedules, the default first: warp-FFT kernels (where the warp path
+// exists) at a carveout of 72 and, where they run at all (N <= 4096; longer lines
+// take kernels without that choice), of 58 and 100 percent, then the block FFT.
+inline std::vector<TuneChoice> tune_candidates(bool have_warp, bool have_carveout) {
     std::vector<TuneChoice> c;
     if (have_warp)
-        for (int cv : {72, 58, 100}) { TuneChoice t; t.warp = 1; t.carveout = cv; c.push_back(t); }
+        for (int cv : {72, 58, 100}) {
+            if (cv != 72 && !have_carveout) continue;
+            TuneChoice t; t.warp = 1; t.carveout = cv; c.push_back(t);
+        }
     TuneChoice b; b.warp = 0; b.carveout = 72; c.push_back(b);
     return c;
 }
@@ -58,6 +62,7 @@ public:
     virtual int tune_load() = 0;                   // back to the kept state
     virtual void tune_free() = 0;
     virtual bool tune_has_warp() const = 0;
+    virtual bool tune_has_carveout() const = 0;
     virtual int tune_apply(int warp, int carveout) = 0;
     virtual int tune_record(int warp, int carveout, double ms, double ms_default) = 0;
     virtual int autotune_apply_cached() = 0;       // take this N's recorded schedule

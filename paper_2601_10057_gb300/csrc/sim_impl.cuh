@@ -678,6 +678,7 @@ public:
     }
 
     bool tune_has_warp() const override { return have_warp; }
+    bool tune_has_carveout() const override { return have_warp && M <= 2048; }
 
     int tune_apply(int warp, int carveout) override {
         TuneChoice c;
@@ -705,7 +706,7 @@ public:
         k = (k + 2) / 3 * 3;
         int r = tune_save();
         if (r) return r;
-        const std::vector<TuneChoice> cand = tune_candidates(have_warp);
+        const std::vector<TuneChoice> cand = tune_candidates(have_warp, tune_has_carveout());
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) r = CCMSAV_ECUDA;
         double best = 1e300, dflt = 0.0;
