@@ -27,10 +27,10 @@
 // and hands its north face on as the next row's south face, and takes its west
 // face from the lane on its left (lane 0 evaluates it).
 //
-// Measured (one step, event times): N = 2048 1475 -> 358 us, N = 512 113 -> 36 us,
-// N = 64 112 -> 14 us (the last two mostly from tiles small enough to give
-// every SM one); now bound by instruction issue (65 % of the slots busy, DRAM
-// 15 %).
+// Measured (one step, event times, no tile outside the range): N = 2048 1475 ->
+// 397 us, N = 512 113 -> 39 us, N = 64 112 -> 15 us (the last two mostly from
+// tiles small enough to give every SM one); now bound by instruction issue (61 %
+// of the slots busy, DRAM 13 %).
 //
 // Concentrations are in a unit of their own (psi_unit, from psi_in, psi_out and
 // the conserved mean), and the osmotic terms P, f_in, f_out of a tile scaled by
@@ -39,9 +39,11 @@
 //
 // Range: |phi*| <= 1.5, |phi_bar| < 4/3, |psi*| <= 3 units, face differences of phi*
 // up to 1/4, of 3 phi_bar up to 1 and of the normalised flux up to 1.5,
-// |psi^n - psi^{n-1}| <= 1/2 unit.  A CTA with a cell
-// outside (steeper profiles than 4 cells per interface width, diverging or
-// non-finite states) evaluates its tile in FP64 instead (stencil_tile).
+// |psi^n - psi^{n-1}| <= 1/2 unit.  A CTA with a cell outside (steep profiles,
+// diverging or non-finite states) evaluates its tile in FP64 (stencil_tile) after
+// that.  A profile of four cells' width has differences of 0.18; evolving states
+// of that width were found at 0.21 (N = 256), 0.24 - 0.34 (N = 128) and up to 0.75
+// (N = 64, dt = 1e-4: most tiles of most steps, 57 us a step instead of 40).
 #pragma once
 #include "step_kernels.cuh"
 #include "fixed_fft.cuh"

@@ -68,7 +68,7 @@ public:
     PostTw<T>* twP = nullptr;
     double* ev = nullptr;
     DevScalars* sc = nullptr;
-    // FP32 warp-FFT path (N = 128 .. 2048): twiddle matrix W_M^{n2 k1} and FP32 eigenvalues
+    // FP32 warp-FFT and wide-line path (N = 128 .. 8192): twiddle matrix W_M^{n2 k1} (to N = 4096) and FP32 eigenvalues
     bool warp_path = false;
     cplx<float>* tw2 = nullptr;
     float* evf = nullptr;
@@ -77,7 +77,7 @@ public:
     float2 twF0{};
     wf::PairTwTab pair_tab() const { return wf::PairTwTab{twF, twF0}; }
     // FP64 path (N >= 64): the fixed-point line transforms and 1/sigma, 1/tau of
-    // the handle's time step in the order of their spectra
+    // the handle's time step in the order of their spectra (two more fields of N x N)
     const xf::Ops* xo = nullptr;
     xf::Tables xt;
     double* isig = nullptr;

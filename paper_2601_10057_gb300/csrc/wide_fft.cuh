@@ -1,12 +1,13 @@
-// wide_fft.cuh -- FP32 lines of M complex values on M / 16 lanes (sixteen
-// values each), for kernels that want many warps per SM: the standalone
-// solver at every size and the long lines of the step.
+// wide_fft.cuh -- FP32 lines of M complex values on M / A lanes (A = 16 values
+// each, 8 and 4 on short lines, see Shape), for kernels that want many warps per
+// SM: the standalone solver and the classical preconditioner at every length,
+// the step's recovery and inverse-row kernels from N = 128 on, and its forward
+// kernels at N = 8192.
 //
 // The line layout is that of fixed_fft.cuh (M = A C D, two exchanges through
-// the line's buffer, lines on one to eight warps).  warp_fft.cuh keeps a line
+// the line's buffer, lines on a part of a warp to eight warps).  warp_fft.cuh keeps a line
 // on one warp with up to 64 values per lane: fewer exchanges, and the faster
-// one up to M = 1024 in the step, but at M = 2048 and 4096 it needs 219 - 255
-// registers per thread and eight warps per SM then wait on memory.
+// one in the step's forward kernels up to N = 4096 (wide_step.cuh has both times).
 #pragma once
 #include <cooperative_groups.h>
 #include "dct_device.cuh"

@@ -5,7 +5,7 @@
 // The inverse kernels wait on memory, and on warp-level lines (32 or 64 values
 // per lane, 72 - 128 registers) they held 16 - 24 warps per SM; with sixteen
 // values per lane 32 warps fit: N = 2048 recovery 61 -> 45 us, inverse rows
-// 40 -> 31; N = 8192 1112 -> 743, 839 -> 394.  The recovery kernel takes one field per CTA (the phi CTAs,
+// 40 -> 30; N = 8192 1112 -> 743, 839 -> 395.  The recovery kernel takes one field per CTA (the phi CTAs,
 // five spectra, come first, the lighter psi CTAs fill the tail).
 #pragma once
 #include "warp_kernels.cuh"
