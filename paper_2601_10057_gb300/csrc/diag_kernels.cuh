@@ -123,15 +123,17 @@ k_dnorm(const T* __restrict__ phn, const T* __restrict__ pho, const T* __restric
 // The sums set_state needs for FP32 fields: columns 0 - 4 of k_diag (initial
 // SAVs and arc length) in the FP32 arithmetic of the step's own stencil
 // (sin/cos by the same polynomials) with double-float accumulation per thread,
-// in column 13 the FP64 sum of psi and in column 5 the number of cells with a
-// non-finite value (the other columns are 0).  k_diag evaluates every cell in
+// and, if asked (set_state checks and sums host fields while it uploads them), in
+// column 13 the FP64 sum of psi and in column 5 the number of cells with a
+// non-finite value (the other columns are 0; 74 us at N = 2048
+// with all fourteen columns added in FP64, 62 with five).  k_diag evaluates every cell in
 // FP64, whose issue rate on GB300 makes it a millisecond at N = 2048 and 17 ms
 // at N = 8192; this pass costs about as much as reading the two fields.
 struct InitCoefF { float inv_h, eps, inv_eps, beta, gin, gout, psin, psout, bin, bout; };
 
 static __global__ void __launch_bounds__(256)
 k_init_sums_f32(const float* __restrict__ a, const float* __restrict__ psi, double* __restrict__ part, int N,
-                InitCoefF c) {
+                InitCoefF c, int psi_sum) {
     __shared__ double sred[8 * NDIAG];
     const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     float hi[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, lo[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -150,8 +152,10 @@ k_init_sums_f32(const float* __restrict__ a, const float* __restrict__ psi, doub
             const float gbar = 0.5f * (gE * gE + gW * gW) + 0.5f * (gN * gN + gS * gS);
             const float a2 = aC * aC, vv = a2 - 1.0f - c.beta, a3 = aC * (a2 - 1.0f);
             const float ps = psi[(size_t)j * N + i];
-            psum += (double)ps;
-            bad += !(isfinite(aC) && isfinite(ps));
+            if (psi_sum) {
+                psum += (double)ps;
+                bad += !(isfinite(aC) && isfinite(ps));
+            }
             float sp, cp;
             sincospi_<float>(0.5f * aC, &sp, &cp);
             const float fin = 0.5f * c.gin * (ps - c.psin) * (ps - c.psin) + c.bin;
@@ -165,11 +169,19 @@ k_init_sums_f32(const float* __restrict__ a, const float* __restrict__ psi, doub
             for (int q = 0; q < 5; ++q) df_add(hi[q], lo[q], v[q]);
         }
     }
-    double v[NDIAG];
+    double* row = part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * NDIAG;
+    double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, (double)bad, psum};
 #pragma unroll
-    for (int q = 0; q < NDIAG; ++q)
-        v[q] = q < 5 ? (double)hi[q] + (double)lo[q] : q == 5 ? (double)bad : q == 13 ? psum : 0.0;
-    block_sum_store<NDIAG, double>(v, part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * NDIAG, sred);
+    for (int q = 0; q < 5; ++q) v[q] = (double)hi[q] + (double)lo[q];
+    if (psi_sum) {
+        block_sum_store<7, double>(v, row, sred);
+        if (threadIdx.x == 6) { row[13] = row[6]; row[6] = 0.0; }      // thread 6 wrote it
+        if (threadIdx.x >= 7 && threadIdx.x < 13) row[threadIdx.x] = 0.0;
+    } else {
+        double w[5] = {v[0], v[1], v[2], v[3], v[4]};
+        block_sum_store<5, double>(w, row, sred);
+        if (threadIdx.x >= 5 && threadIdx.x < NDIAG) row[threadIdx.x] = 0.0;
+    }
 }
 
 // lamsum += scale * sum(part[0..nb)) in a fixed order (one block).

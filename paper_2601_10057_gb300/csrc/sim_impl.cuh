@@ -1035,15 +1035,15 @@ public:
         return CCMSAV_OK;
     }
 
-    // The sums of set_state over the current level (k_diag's columns; FP32:
+    // The sums of set_state over the current level (k_diag's columns; FP32: column 13 only with psi_sum, and then
     // column 5 counts the cells with a non-finite value).
-    int init_sums(double s[NDIAG]) {
+    int init_sums(double s[NDIAG], int psi_sum) {
         if constexpr (std::is_same<T, float>::value) {
             // the five sums in the step's FP32 arithmetic
             const double hh = h();
             InitCoefF ic{(float)(1.0 / hh), (float)p.eps, (float)(1.0 / p.eps), (float)p.beta, (float)p.gamma_in,
                          (float)p.gamma_out, (float)p.psi_in, (float)p.psi_out, (float)p.beta_in, (float)p.beta_out};
-            k_init_sums_f32<<<g_dg, 256, 0, st>>>(phi[cur], psi[cur], partd, N, ic);
+            k_init_sums_f32<<<g_dg, 256, 0, st>>>(phi[cur], psi[cur], partd, N, ic, psi_sum);
         } else {
             k_diag<T, true><<<g_dg, 256, 0, st>>>(phi[cur], phi[cur], psi[cur], partd, N, diag_coef());
         }
@@ -1080,7 +1080,7 @@ public:
         double psum = 0.0;
         int r = upload_levels(phi0, psi0, phi1, psi1, &psum);
         double s[NDIAG];
-        if (r == CCMSAV_OK) r = init_sums(s);
+        if (r == CCMSAV_OK) r = init_sums(s, 0);
         if (r == CCMSAV_OK) r = init_scalars(s, psum);
         if (r) { have_state = false; return r; }   // the levels were overwritten: no state
         have_state = true; poisoned = false;
@@ -1096,7 +1096,7 @@ public:
         CCM_CUDA(cudaMemcpyAsync(phi[prev], dphi, fb, cudaMemcpyDeviceToDevice, st));
         CCM_CUDA(cudaMemcpyAsync(psi[prev], dpsi, fb, cudaMemcpyDeviceToDevice, st));
         double s[NDIAG];
-        int r = init_sums(s);
+        int r = init_sums(s, 1);
         if (r) return r;
         if (std::is_same<T, float>::value) {
             if (s[5] != 0.0 || !std::isfinite(s[13])) return CCMSAV_ENONFINITE;
